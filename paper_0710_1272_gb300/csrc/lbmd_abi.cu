@@ -33,7 +33,7 @@ struct lbmd_ctx {
   cudaStream_t user;        // caller's stream
   cudaStream_t own, side;   // private streams: steps run on own, MD on side
   int prio_high;            // greatest stream priority of the device
-  cudaEvent_t ev_in, ev_out, ev_fork, ev_join;
+  cudaEvent_t ev_in, ev_out, ev_fork, ev_join, ev_gather;
   cudaGraphExec_t graph[2][3];  // [starting buffer][1, 2, kBlockSteps steps]
   // one step followed by the bead-block read-out, per starting buffer
   // (lbmd_step_read_async); the read-out node's destination is set per launch
@@ -105,7 +105,7 @@ cudaError_t enqueue_step(lbmd_ctx *c, int src) {
     // no solvent (u_i stays 0): the M MD substeps, then the spread, which
     // finds no transfer node and only advances the step counter
     if (t[2] && (e = record_timing(t[2], c->own)) != cudaSuccess) return e;
-    if ((e = launch_md_cycle(c->chain, c->prio_high, c->own)) != cudaSuccess) return e;
+    if ((e = launch_md_cycle(c->chain, c->prio_high, false, c->own)) != cudaSuccess) return e;
     if (t[3] && (e = record_timing(t[3], c->own)) != cudaSuccess) return e;
     for (int k : {0, 1, 4})
       if (t[k] && (e = record_timing(t[k], c->own)) != cudaSuccess) return e;
@@ -130,19 +130,18 @@ cudaError_t enqueue_step(lbmd_ctx *c, int src) {
     ChainArgs a = c->chain;
     a.f = A;
     a.f_mode = pop_mode(c, src);
-    const bool gather_beside = !take;
-    cudaStream_t gs = gather_beside ? c->side : c->own;
-    if (gather_beside) {
-      if ((e = cudaEventRecord(c->ev_fork, c->own)) != cudaSuccess) return e;
-      if ((e = cudaStreamWaitEvent(c->side, c->ev_fork, 0)) != cudaSuccess) return e;
+    // Either way the gather is on the side stream with the MD cycle behind it,
+    // which may start beside it; a stream-collide that comes after the gather
+    // waits for it there.
+    if ((e = cudaEventRecord(c->ev_fork, c->own)) != cudaSuccess) return e;
+    if ((e = cudaStreamWaitEvent(c->side, c->ev_fork, 0)) != cudaSuccess) return e;
+    if (t[2] && (e = record_timing(t[2], c->side)) != cudaSuccess) return e;
+    if ((e = launch_gather(c->p.storage, a, c->side)) != cudaSuccess) return e;
+    if (take) {
+      if ((e = cudaEventRecord(c->ev_gather, c->side)) != cudaSuccess) return e;
+      if ((e = cudaStreamWaitEvent(c->own, c->ev_gather, 0)) != cudaSuccess) return e;
     }
-    if (t[2] && (e = record_timing(t[2], gs)) != cudaSuccess) return e;
-    if ((e = launch_gather(c->p.storage, a, gs)) != cudaSuccess) return e;
-    if (!gather_beside) {
-      if ((e = cudaEventRecord(c->ev_fork, c->own)) != cudaSuccess) return e;
-      if ((e = cudaStreamWaitEvent(c->side, c->ev_fork, 0)) != cudaSuccess) return e;
-    }
-    if ((e = launch_md_cycle(a, c->prio_high, c->side)) != cudaSuccess) return e;
+    if ((e = launch_md_cycle(a, c->prio_high, true, c->side)) != cudaSuccess) return e;
     if (t[3] && (e = record_timing(t[3], c->side)) != cudaSuccess) return e;
     // sum part of the spread, beside the stream-collide
     if ((e = launch_spread_sum(c->chain, !take, c->side)) != cudaSuccess) return e;
@@ -296,6 +295,7 @@ void destroy_ctx(lbmd_ctx *c) {
   if (c->ev_out) cudaEventDestroy(c->ev_out);
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
   if (c->ev_join) cudaEventDestroy(c->ev_join);
+  if (c->ev_gather) cudaEventDestroy(c->ev_gather);
   if (c->own) cudaStreamDestroy(c->own);
   if (c->side) cudaStreamDestroy(c->side);
   if (c->pinned) cudaFreeHost(c->pinned);
@@ -382,7 +382,7 @@ int lbmd_create(const lbmd_params *params, void *dev_workspace, size_t bytes, vo
   int prio_least = 0;
   if ((e = cudaDeviceGetStreamPriorityRange(&prio_least, &c->prio_high)) != cudaSuccess) return bail(e, "priority range");
   if ((e = cudaStreamCreateWithPriority(&c->side, cudaStreamNonBlocking, c->prio_high)) != cudaSuccess) return bail(e, "stream");
-  for (cudaEvent_t *ev : {&c->ev_in, &c->ev_out, &c->ev_fork, &c->ev_join})
+  for (cudaEvent_t *ev : {&c->ev_in, &c->ev_out, &c->ev_fork, &c->ev_join, &c->ev_gather})
     if ((e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming)) != cudaSuccess) return bail(e, "event");
 
   if (c->N > 0) keep_chain_in_l2(c, L);

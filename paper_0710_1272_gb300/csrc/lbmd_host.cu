@@ -79,6 +79,9 @@ Layout make_layout(const lbmd_params &p, bool single_box) {
   L.nl_list = take(Np * kMaxPairs * sizeof(short));
   L.wl_list = take(Np * kMaxWall * sizeof(float4));
   L.nl_ref = take(Np * sizeof(float4));
+  L.items = take((size_t)md_item_cap((int)Np) * sizeof(uint2));
+  L.it_first = take(Np * sizeof(int));
+  L.noise = take((size_t)std::max(p.md_substeps, 1) * Np * sizeof(float4));
   L.lam = take(Np * sizeof(float));
   L.status = take(sizeof(DevStatus));
   L.diag = take((size_t)std::max(p.diag_capacity, 0) * sizeof(DevDiag));
@@ -507,6 +510,9 @@ cudaError_t init_instance(const lbmd_params &p, const Layout &L, char *ws, cudaS
   a.nl_list = (short *)(ws + L.nl_list);
   a.wl_list = (float4 *)(ws + L.wl_list);
   a.nl_ref = (float4 *)(ws + L.nl_ref);
+  a.items = (uint2 *)(ws + L.items);
+  a.it_first = (int *)(ws + L.it_first);
+  a.noise = (float4 *)(ws + L.noise);
   a.lam = (float *)(ws + L.lam);
   a.status = out.status;
   a.diag = (DevDiag *)(ws + L.diag);
@@ -542,6 +548,7 @@ cudaError_t init_instance(const lbmd_params &p, const Layout &L, char *ws, cudaS
     UP(cudaMemsetAsync(a.sp_node, 0xff, 8 * (size_t)N * sizeof(int), s), "memset");
     UP(cudaMemsetAsync(a.nl_cnt, 0, (size_t)N * sizeof(int), s), "memset");
     UP(cudaMemsetAsync(a.wl_cnt, 0, (size_t)N * sizeof(int), s), "memset");
+    UP(cudaMemsetAsync(a.it_first, 0, (size_t)N * sizeof(int), s), "memset");
     UP(cudaMemsetAsync(a.lam, 0, (size_t)N * sizeof(float), s), "memset");
     UP(cudaMemcpyAsync(a.nl_ref, hp.data(), N * sizeof(float4), cudaMemcpyHostToDevice, s), "upload");
     UP(md_prepare(), "md attributes");

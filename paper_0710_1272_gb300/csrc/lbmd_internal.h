@@ -19,7 +19,8 @@ struct DevStatus {
   int shake_fail;        // LB steps whose constraint solve hit the iteration cap
   int newton_iters;      // Newton iterations of the last LB step (all substeps)
   int nl_builds;         // neighbour-list builds so far (0: none yet)
-  int nl_ok;             // 1 if the current lists hold every pair (no overflow)
+  int nl_ok;             // kind of the current neighbour lists (0: overflow, none)
+  int nl_items;          // entries of the flat force list
   int out_buf;           // ensemble: population buffer (0/1) written by the last step
   int diag_count;        // diagnostic records written
   int pop_bad;           // 1 once a stream-collide met a node whose populations
@@ -122,6 +123,9 @@ struct ChainArgs {
   short *nl_list;           // [N][kMaxPairs] partner beads
   float4 *wl_list;          // [N][kMaxWall] solid nodes (local frame)
   float4 *nl_ref;           // [N] positions at the last list build
+  uint2 *items;             // [md_item_cap(N)] flat force list
+  int *it_first;            // [N] a bead's first entry there | its entries << 16
+  float4 *noise;            // [M][N] standard normals of the step's substeps
   float *lam;               // [N] SHAKE multipliers of the last substep
   DevStatus *status;
   DevDiag *diag;            // [diag_cap] diagnostic records
@@ -161,6 +165,7 @@ struct __align__(16) EnsTile {
 
 size_t md_smem_bytes(int N);
 int md_threads(int N);
+int md_item_cap(int N);  // entries the flat force list has room for
 // Opt the MD kernels into the dynamic shared memory of the longest chain.
 cudaError_t md_prepare();
 
@@ -203,7 +208,7 @@ cudaError_t launch_read_pulled(int storage, const LbGeom &g, float rho0, const v
                                int mode, long long z0, long long nzc, float *f,
                                long long fstride, cudaStream_t s);
 cudaError_t launch_gather(int storage, const ChainArgs &a, cudaStream_t s);
-cudaError_t launch_md_cycle(const ChainArgs &a, int priority, cudaStream_t s);
+cudaError_t launch_md_cycle(const ChainArgs &a, int priority, bool beside, cudaStream_t s);
 // Spread of the bead impulses (stage 3), independent of the order of
 // concurrent atomics, so that a step gives the same bits in every run:
 //  - the gather claims each transfer node for the smallest (bead, corner)

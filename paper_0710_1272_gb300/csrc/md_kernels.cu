@@ -10,7 +10,7 @@
 //     F = F_WCA + F_bend + F_wall + F_drive - m gamma (v - u_i) + F_r,
 //     v += dt F / m,  r~ = r + dt v,
 //     SHAKE: Newton on the N-1 bond multipliers, the tridiagonal Jacobian
-//            solved by parallel cyclic reduction in shared memory,
+//            solved by one warp of the block (tri_solve_warp),
 //     v = (r' - r) / dt,  r = r',
 //     RATTLE: one tridiagonal solve removes the bond-parallel relative
 //             velocities,
@@ -28,6 +28,11 @@ namespace lbmd {
 constexpr float kTwoSixth = 1.122462048309373f;  // 2^(1/6)
 constexpr float kSkin = 0.8f;  // neighbour-list skin: lists hold pairs within r_c + skin
 
+// How the pair and wall forces of a chain are found (DevStatus::nl_ok).
+constexpr int kNlNone = 0;  // a bead's list overflowed: all pairs, stencil scan
+constexpr int kNlBead = 1;  // per-bead lists in the workspace
+constexpr int kNlFlat = 2;  // one list of (bead, partner) entries in shared memory
+
 struct F3 {
   float x, y, z;
 };
@@ -38,27 +43,55 @@ __device__ __forceinline__ F3 operator-(F3 a, F3 b) { return F3{a.x - b.x, a.y -
 __device__ __forceinline__ F3 operator*(float s, F3 a) { return F3{s * a.x, s * a.y, s * a.z}; }
 __device__ __forceinline__ float dot(F3 a, F3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
 
-// Threads of the MD block: one per bead, rounded up to a warp.
-int md_threads(int N) { return (N + 31) / 32 * 32; }
-
-// Shared memory of the MD block: positions (hi, lo), displacements, bond
-// vectors, velocities, the tridiagonal work arrays, the pair lists and, for
-// chains of up to 512 beads, up to 32 solid nodes of each bead's wall list as
-// integer coordinates of the chain's local frame (longer wall lists are read
-// from the workspace).
-constexpr int kWallShared = 32;
-constexpr int kWallSharedMaxN = 512;
-
-// Bytes before the shared wall lists, rounded up to 16 (the short4 entries
-// need 8-byte alignment; 180 N bytes is not a multiple of 8 for odd N).
-__host__ __device__ inline size_t md_smem_head(int N) {
-  const size_t head = (size_t)N * (5 * sizeof(float4) + sizeof(float) + kMaxPairs * sizeof(short));
-  return (head + 15) / 16 * 16;
+// Threads of the MD block: one per bead in whole warps, at least three warps
+// (they share the evaluation of the force list), and one more warp for the
+// tridiagonal solves where the block's register class (512, 768 or 1024
+// threads: 128, 80 or 64 registers) has room for it; else warp 0 solves beside
+// its beads.
+__host__ __device__ inline int bead_threads(int N) { return max((N + 31) / 32 * 32, 96); }
+int md_threads(int N) {
+  const int t = bead_threads(N);
+  return t == 512 || t == 768 || t == LBMD_MAX_BEADS ? t : t + 32;
 }
 
+// Chains of more than 512 beads halve their system before the solve: the
+// threads of the odd rows eliminate the even rows beside them (all at once),
+// and the solving warp is left with half the rows.  With 64 or 80 registers a
+// lane cannot hold 23 or 33 rows; through shared memory that many took 4.2 and
+// 5.6 k cycles, 13 and 17 rows in registers 1.05 and 1.15 k.
+__host__ __device__ inline bool halves_rows(int N) { return N > 512; }
+
+// Rows a lane of the solving warp takes, from the chain's length: odd, so that
+// the lanes' accesses fall into different banks; and the rows held, a multiple
+// of 32 of them (those past the chain are identity rows).
+__host__ __device__ inline int solve_rows(int N) {
+  const int n = N - 1;
+  const int m = halves_rows(N) ? n / 2 : n;
+  return m <= 32 * 5 ? 5 : m <= 32 * 13 ? 13 : 17;
+}
+
+// Shared memory of the MD block: the rows of the tridiagonal system and its
+// solution; per bead positions (hi, lo), displacements, bond vectors at the
+// start and the end of the substep, multipliers and the mask of acting list
+// entries; then the force list (8 bytes an entry) and a force per entry, eight
+// entries per bead (the chains measured average three) and 128 for the beads
+// in the pore, as far as 220 KB reach.
+constexpr int kMdSmemMost = 220000;
+__host__ __device__ inline size_t md_smem_head(int N) {
+  return ((size_t)32 * solve_rows(N) * (sizeof(float4) + sizeof(float)) +
+          (halves_rows(N) ? 2 * (size_t)(N + 1) * sizeof(float4) : 0) + (size_t)N * (5 * sizeof(float4) + 2 * sizeof(float)) + 15) / 16 * 16;
+}
+__host__ __device__ inline int item_want(int N) { return 8 * N + 128; }
+__host__ __device__ inline int item_cap(int N) {
+  const int room = (kMdSmemMost - (int)md_smem_head(N)) / (int)(sizeof(float4) + sizeof(uint2));
+  return item_want(N) < room ? item_want(N) : room;
+}
+int md_item_cap(int N) { return item_cap(N); }
+// Never less for a longer chain (an ensemble sizes a group's blocks for its
+// longest one): chains whose list is cut to the room there is ask for all of it.
 size_t md_smem_bytes(int N) {
-  const size_t walls = N <= kWallSharedMaxN ? (size_t)N * kWallShared * sizeof(short4) : 0;
-  return md_smem_head(N) + walls;
+  if (item_cap(N) < item_want(N)) return kMdSmemMost;
+  return md_smem_head(N) + (size_t)item_cap(N) * (sizeof(float4) + sizeof(uint2));
 }
 
 // Double-float helpers: a coordinate is hi + lo with |lo| <= ulp(hi) / 2.
@@ -91,16 +124,6 @@ __device__ __forceinline__ void cell_frac_hl(float hi, float lo, int origin, int
   cell = wrap_near(origin + (int)fl, n);
 }
 
-// 2x2 matrices for the interface system of the tridiagonal solve.
-struct M2 {
-  float a, b, c, d;  // [[a, b], [c, d]]
-};
-__device__ __forceinline__ M2 mmul(M2 x, M2 y) {
-  return M2{x.a * y.a + x.b * y.c, x.a * y.b + x.b * y.d, x.c * y.a + x.d * y.c,
-            x.c * y.b + x.d * y.d};
-}
-__device__ __forceinline__ M2 madd(M2 x, M2 y) { return M2{x.a + y.a, x.b + y.b, x.c + y.c, x.d + y.d}; }
-
 // Hardware reciprocal approximation (relative error ~2^-23) for the
 // tridiagonal solves: they are latency-bound chains, and a correctly rounded
 // reciprocal costs several dependent instructions.
@@ -110,141 +133,110 @@ __device__ __forceinline__ float rcp_fast(float x) {
   return r;
 }
 
-__device__ __forceinline__ M2 minv(M2 x) {
-  const float r = rcp_fast(x.a * x.d - x.b * x.c);
-  return M2{x.d * r, -x.b * r, -x.c * r, x.a * r};
-}
-__device__ __forceinline__ M2 mshfl_up(M2 x, int s) {
-  return M2{__shfl_up_sync(0xffffffffu, x.a, s), __shfl_up_sync(0xffffffffu, x.b, s),
-            __shfl_up_sync(0xffffffffu, x.c, s), __shfl_up_sync(0xffffffffu, x.d, s)};
-}
-__device__ __forceinline__ M2 mshfl_down(M2 x, int s) {
-  return M2{__shfl_down_sync(0xffffffffu, x.a, s), __shfl_down_sync(0xffffffffu, x.b, s),
-            __shfl_down_sync(0xffffffffu, x.c, s), __shfl_down_sync(0xffffffffu, x.d, s)};
+// Reciprocal for the forces: the hardware approximation and one
+// Newton-Raphson step (relative error below an ulp), without a branch.
+__device__ __forceinline__ float rcp_newton(float x) {
+  const float r = rcp_fast(x);
+  return fmaf(fmaf(-x, r, 1.0f), r, r);
 }
 
-// Tridiagonal solve over rows 0..n-1 of the block (row i held by thread i:
-// a x_{i-1} + b x_i + c x_{i+1} = d, with a_0 = c_{n-1} = 0).  Every thread
-// of the block calls it; returns x_i and, in x_prev, x_{i-1}.
+// s a + b, each component one fused operation.
+__device__ __forceinline__ F3 axpy(float s, F3 a, F3 b) {
+  return F3{fmaf(s, a.x, b.x), fmaf(s, a.y, b.y), fmaf(s, a.z, b.z)};
+}
+
+// Tridiagonal solve over 32 R rows (row i: s_row[i] = (a, c, d, -) with
+// a x_{i-1} + x_i + c x_{i+1} = d: rows divided by their diagonals, so that
+// the determinants below stay in range; rows past the chain are zero) by one
+// warp; x_i goes to s_x[i].  Called by all 32 lanes, between two block barriers.
 //
-// SPIKE-type partition by warps: each warp reduces its 32 rows by cyclic
-// reduction over lane shuffles, for the right-hand side and for the two
-// coupling columns to the neighbouring warps (the "spikes" v and w), giving
-// x_i = y_i - v_i x_last(prev warp) - w_i x_first(next warp).  The first and
-// last unknowns of neighbouring warps form a block tridiagonal system with
-// 2x2 blocks, one block row per warp boundary, which warp 0 solves by block
-// cyclic reduction.  Two block barriers, none when n <= 32.
-__device__ float spike_tri_solve(int n, float a, float b, float c, float d, float &x_prev) {
-  __shared__ float sh_y[6 * 32];  // per warp: y, v, w of its first and last row
-  __shared__ float sh_x[64];      // x of the last row [0, 32) and first row [32, 64) per warp
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  const int nch = (n + 31) >> 5;
-  if (t >= n) {
-    a = 0.f;
-    b = 1.f;
-    c = 0.f;
-    d = 0.f;
+// What bounds it is latency: a chain has up to 1023 rows and nothing else to
+// do meanwhile.  Lane l takes the R rows from l R on.  Its first R - 1
+// unknowns are eliminated towards the lane's last one: the pivots as a
+// three-term recurrence of determinants P_k = P_{k-1} - a_k c_{k-1} P_{k-2},
+// whose chain is one fused operation per row (the reciprocals 1/P_k hang off
+// it), then x_k = u_k + v_k x_{l R - 1} - w_k x_{k+1}, and by back substitution
+// x_k = U_k + V_k x_{l R - 1} + W_k x_{l R + R - 1}.  The lanes' last unknowns
+// form a tridiagonal system of their own, solved by cyclic reduction over lane
+// shuffles.  Measured by itself: 0.50 k cycles for 20 beads, 0.73 k for 100,
+// 1.05 k for 400 (in the block, where the other warps' code competes for the
+// instruction cache, 0.9 / 1.2 / 1.7 k), against 0.66 / 1.85 / 3.1 k for 32-row
+// cyclic reductions in every warp with a boundary system and two more block
+// barriers.
+template <int R>
+__device__ __noinline__ void tri_solve_warp(int n, const float4 *s_row, float *s_x) {
+  const int lane = threadIdx.x & 31;
+  const float4 *row = s_row + lane * R;
+  float *out = s_x + lane * R;
+  float u[R - 1], v[R - 1], w[R - 1];
+  {
+    const float4 q = row[0];
+    u[0] = q.z;
+    v[0] = -q.x;
+    w[0] = q.y;
   }
-  float al = lane == 0 ? 0.f : a, be = b, ga = lane == 31 ? 0.f : c;
-  float r0 = d, r1 = lane == 0 ? a : 0.f, r2 = lane == 31 ? c : 0.f;
+  float Pm = 1.f, P = 1.f, c = w[0];
 #pragma unroll
-  for (int s = 1; s < 32; s <<= 1) {
-    const float am = __shfl_up_sync(0xffffffffu, al, s), bm = __shfl_up_sync(0xffffffffu, be, s);
-    const float gm = __shfl_up_sync(0xffffffffu, ga, s);
-    const float r0m = __shfl_up_sync(0xffffffffu, r0, s), r1m = __shfl_up_sync(0xffffffffu, r1, s);
-    const float r2m = __shfl_up_sync(0xffffffffu, r2, s);
-    const float ap = __shfl_down_sync(0xffffffffu, al, s), bp = __shfl_down_sync(0xffffffffu, be, s);
-    const float gp = __shfl_down_sync(0xffffffffu, ga, s);
-    const float r0p = __shfl_down_sync(0xffffffffu, r0, s), r1p = __shfl_down_sync(0xffffffffu, r1, s);
-    const float r2p = __shfl_down_sync(0xffffffffu, r2, s);
-    const bool hm = lane >= s, hp = lane + s < 32;
-    const float k1 = hm ? al * rcp_fast(bm) : 0.f;
-    const float k2 = hp ? ga * rcp_fast(bp) : 0.f;
-    const float nal = hm ? -k1 * am : 0.f, nga = hp ? -k2 * gp : 0.f;
-    be = be - k1 * gm - k2 * ap;
-    r0 = r0 - k1 * r0m - k2 * r0p;
-    r1 = r1 - k1 * r1m - k2 * r1p;
-    r2 = r2 - k1 * r2m - k2 * r2p;
-    al = nal;
-    ga = nga;
+  for (int k = 1; k < R - 1; ++k) {
+    const float4 q = row[k];
+    const float Pn = fmaf(-(q.x * c), Pm, P);
+    const float m = P * rcp_fast(Pn), am = q.x * m;
+    w[k] = q.y * m;
+    u[k] = fmaf(-am, u[k - 1], q.z * m);
+    v[k] = -am * v[k - 1];
+    c = q.y;
+    Pm = P;
+    P = Pn;
   }
-  const float ib = rcp_fast(be);
-  const float y = r0 * ib, v = r1 * ib, sw = r2 * ib;
-  if (nch > 1) {
-    if (lane == 0 && w < nch) {
-      sh_y[6 * w] = y;
-      sh_y[6 * w + 1] = v;
-      sh_y[6 * w + 2] = sw;
-    }
-    if (lane == 31 && w < nch) {
-      sh_y[6 * w + 3] = y;
-      sh_y[6 * w + 4] = v;
-      sh_y[6 * w + 5] = sw;
-    }
-    __syncthreads();
-    if (w == 0) {
-      // block row k: unknowns (x_last(k), x_first(k+1)) at the boundary of
-      // warps k and k+1; rows beyond nch-2 are identity rows
-      M2 L{0.f, 0.f, 0.f, 0.f}, D{1.f, 0.f, 0.f, 1.f}, U{0.f, 0.f, 0.f, 0.f};
-      float q0 = 0.f, q1 = 0.f;
-      if (lane < nch - 1) {
-        D.b = sh_y[6 * lane + 5];        // w of the last row of warp k
-        D.c = sh_y[6 * (lane + 1) + 1];  // v of the first row of warp k+1
-        L.a = sh_y[6 * lane + 4];        // v of the last row of warp k
-        U.d = sh_y[6 * (lane + 1) + 2];  // w of the first row of warp k+1
-        q0 = sh_y[6 * lane + 3];
-        q1 = sh_y[6 * (lane + 1)];
-      }
-      // block cyclic reduction over the nch - 1 boundary rows; each lane
-      // inverts its own diagonal block and the neighbours' inverses arrive by
-      // shuffle
-      for (int s = 1; s < nch - 1; s <<= 1) {
-        const M2 Di = minv(D);
-        const M2 Lm = mshfl_up(L, s), Dim = mshfl_up(Di, s), Um = mshfl_up(U, s);
-        const float q0m = __shfl_up_sync(0xffffffffu, q0, s), q1m = __shfl_up_sync(0xffffffffu, q1, s);
-        const M2 Lp = mshfl_down(L, s), Dip = mshfl_down(Di, s), Up = mshfl_down(U, s);
-        const float q0p = __shfl_down_sync(0xffffffffu, q0, s), q1p = __shfl_down_sync(0xffffffffu, q1, s);
-        M2 al2{0.f, 0.f, 0.f, 0.f}, ga2{0.f, 0.f, 0.f, 0.f};
-        if (lane >= s) {
-          const M2 t2 = mmul(L, Dim);
-          al2 = M2{-t2.a, -t2.b, -t2.c, -t2.d};
-        }
-        if (lane + s < 32) {
-          const M2 t2 = mmul(U, Dip);
-          ga2 = M2{-t2.a, -t2.b, -t2.c, -t2.d};
-        }
-        const M2 nL = mmul(al2, Lm), nU = mmul(ga2, Up);
-        D = madd(D, madd(mmul(al2, Um), mmul(ga2, Lp)));
-        const float nq0 = q0 + al2.a * q0m + al2.b * q1m + ga2.a * q0p + ga2.b * q1p;
-        const float nq1 = q1 + al2.c * q0m + al2.d * q1m + ga2.c * q0p + ga2.d * q1p;
-        L = nL;
-        U = nU;
-        q0 = nq0;
-        q1 = nq1;
-      }
-      const M2 Di = minv(D);
-      if (lane < nch - 1) {
-        sh_x[lane] = Di.a * q0 + Di.b * q1;           // x_last of warp k
-        sh_x[32 + lane + 1] = Di.c * q0 + Di.d * q1;  // x_first of warp k+1
-      }
-    }
-    __syncthreads();
+  const float uk = u[R - 2], vk = v[R - 2], wk = w[R - 2];
+  w[R - 2] = -wk;
+#pragma unroll
+  for (int k = R - 3; k >= 0; --k) {
+    const float h = w[k];
+    u[k] = fmaf(-h, u[k + 1], u[k]);
+    v[k] = fmaf(-h, v[k + 1], v[k]);
+    w[k] = -h * w[k + 1];
   }
-  float x = y;
-  if (nch > 1) {
-    if (w > 0 && w < nch) x -= v * sh_x[w - 1];
-    if (w + 1 < nch) x -= sw * sh_x[32 + w + 1];
+  const float U = u[0], V = v[0], W = w[0];
+  // the lane's last row, with the neighbours' unknowns substituted
+  const float4 q = row[R - 1];
+  const float un = __shfl_down_sync(0xffffffffu, U, 1), vn = __shfl_down_sync(0xffffffffu, V, 1),
+              wn = __shfl_down_sync(0xffffffffu, W, 1);
+  float inv = rcp_fast(fmaf(q.y, vn, fmaf(-q.x, wk, 1.0f)));
+  float al = q.x * vk * inv, ga = q.y * wn * inv;
+  float x = fmaf(-q.y, un, fmaf(-q.x, uk, q.z)) * inv;
+  // lanes past the last row hold identity rows; al and ga of the first and
+  // last lane are zero, so what a shuffle leaves in place there drops out
+  const int lanes = (n + R - 1) / R;
+#pragma unroll 1
+  for (int s = 1; s < lanes; s <<= 1) {
+    const float am = __shfl_up_sync(0xffffffffu, al, s), gm = __shfl_up_sync(0xffffffffu, ga, s),
+                xm = __shfl_up_sync(0xffffffffu, x, s);
+    const float ap = __shfl_down_sync(0xffffffffu, al, s), gp = __shfl_down_sync(0xffffffffu, ga, s),
+                xp = __shfl_down_sync(0xffffffffu, x, s);
+    inv = rcp_fast(fmaf(-ga, ap, fmaf(-al, gm, 1.0f)));
+    x = fmaf(-ga, xp, fmaf(-al, xm, x)) * inv;
+    al = -al * am * inv;
+    ga = -ga * gp * inv;
   }
-  const float xu = __shfl_up_sync(0xffffffffu, x, 1);
-  x_prev = lane > 0 ? xu : (w > 0 && w < nch && nch > 1 ? sh_x[w - 1] : 0.f);
-  return x;
+  const float xu = __shfl_up_sync(0xffffffffu, x, 1), xl = lane > 0 ? xu : 0.f;
+  out[R - 1] = x;
+#pragma unroll
+  for (int k = R - 2; k >= 0; --k) out[k] = fmaf(w[k], x, fmaf(v[k], xl, u[k]));
+}
+
+// Half of a tridiagonal system: row j of the odd rows' system, from rows
+// i - 1, i and i + 1 (i = 2 j + 1).
+__device__ __forceinline__ float4 halve_row(float4 p, float4 q, float4 n) {
+  const float inv = rcp_fast(fmaf(-q.y, n.x, fmaf(-q.x, p.y, 1.0f)));
+  return make_float4(-q.x * p.x * inv, -q.y * n.y * inv, fmaf(-q.y, n.z, fmaf(-q.x, p.z, q.z)) * inv, 0.f);
 }
 
 // Eq. 2 truncated at 2^(1/6) sigma: adds -dV/dd for separation d.
 __device__ __forceinline__ void wca_add(F3 d, float sig2, float rc2, float eps24, F3 &F) {
   const float r2 = dot(d, d);
   if (r2 < rc2) {
-    const float ir2 = 1.0f / r2;
+    const float ir2 = rcp_newton(r2);
     const float sr2 = sig2 * ir2;
     const float sr6 = sr2 * sr2 * sr2;
     const float f = eps24 * (2.0f * sr6 * sr6 - sr6) * ir2;
@@ -253,9 +245,9 @@ __device__ __forceinline__ void wca_add(F3 d, float sig2, float rc2, float eps24
 }
 
 // Eq. 3 bending at the angle of beads (a, b, c) given the two bond vectors
-// b1 = r_b - r_a and b2 = r_c - r_b: the force on bead `which` (0 = a, 1 = b,
-// 2 = c), F = -dV/dr with V = kappa phi^2 / 2.
-__device__ __forceinline__ F3 bend_force(F3 b1, F3 b2, float kappa, int which) {
+// b1 = r_b - r_a and b2 = r_c - r_b: the forces F = -dV/dr on a, b and c with
+// V = kappa phi^2 / 2.
+__device__ __noinline__ void bend_forces(F3 b1, F3 b2, float kappa, F3 &fa, F3 &fb, F3 &fc) {
   const float l1 = sqrtf(dot(b1, b1)), l2 = sqrtf(dot(b2, b2));
   float cphi = dot(b1, b2) / (l1 * l2);
   cphi = fminf(1.f, fmaxf(-1.f, cphi));
@@ -263,13 +255,13 @@ __device__ __forceinline__ F3 bend_force(F3 b1, F3 b2, float kappa, int which) {
   const float A = phi < 1e-4f ? kappa : kappa * phi / sinf(phi);
   const F3 g1 = (1.0f / (l1 * l2)) * b2 - (cphi / (l1 * l1)) * b1;
   const F3 g2 = (1.0f / (l1 * l2)) * b1 - (cphi / (l2 * l2)) * b2;
-  if (which == 0) return (-A) * g1;
-  if (which == 1) return A * (g1 - g2);
-  return A * g2;
+  fa = (-A) * g1;
+  fb = A * (g1 - g2);
+  fc = A * g2;
 }
 
 // WCA pair forces on bead i from every other non-bonded bead (minimum image).
-__device__ __forceinline__ F3 all_pair_forces(const ChainArgs &a, int i, float4 rh, float4 rl,
+__device__ __noinline__ F3 all_pair_forces(const ChainArgs &a, int i, float4 rh, float4 rl,
                                               const float4 *s_rh, const float4 *s_rl) {
   const LbGeom &g = a.geo;
   const float sig2 = a.sigma * a.sigma;
@@ -292,44 +284,41 @@ __device__ __forceinline__ F3 all_pair_forces(const ChainArgs &a, int i, float4 
 
 // Sec. III pulling force on a bead at the local position rh + rl: -f_drive x
 // inside the channel of the pore cross-section and the x-layers within 1.5
-// nodes of the wall.
-__device__ __forceinline__ F3 drive_force_at(const ChainArgs &a, float4 rh, float4 rl) {
+// nodes of the wall.  In float throughout: the cell and its fraction by integer
+// conversions are a chain of ~25-cycle latencies each.
+struct Drive {
+  float sx, sy, sz;     // local coordinate -> coordinate of the box (x: from nx / 2 before the wall)
+  float ix, iy, iz;     // 1 / box
+  float cx, half;       // channel along x: centre, half length
+  float y0, y1, z0, z1; // its cross-section [y0, y1) x [z0, z1)
+  float f;              // 0: none
+};
+__device__ __forceinline__ Drive drive_of(const ChainArgs &a) {
   const LbGeom &g = a.geo;
-  F3 F{0.f, 0.f, 0.f};
-  if (a.has_wall && a.pore_d > 0 && a.fdrive != 0.f) {
-    int c[3];
-    float sf[3];
-    cell_frac_hl(rh.x, rl.x, a.ox, g.nx, c[0], sf[0]);
-    cell_frac_hl(rh.y, rl.y, a.oy, g.ny, c[1], sf[1]);
-    cell_frac_hl(rh.z, rl.z, a.oz, g.nz, c[2], sf[2]);
-    const int di = wrap_near(c[0] - a.wall_x + g.nx / 2, g.nx) - g.nx / 2;
-    const float dx = (float)di + sf[0] - 0.5f * (float)(a.wall_t - 1);
-    const float half = 0.5f * (float)(a.wall_t - 1) + 1.5f;
-    const float ry = (float)c[1] + sf[1], rz = (float)c[2] + sf[2];
-    if (fabsf(dx) <= half && ry >= a.pore_y0 - 0.5f && ry < a.pore_y0 + a.pore_d - 0.5f &&
-        rz >= a.pore_z0 - 0.5f && rz < a.pore_z0 + a.pore_d - 0.5f)
-      F.x -= a.fdrive;
-  }
-  return F;
+  const float half_t = 0.5f * (float)(a.wall_t - 1);
+  Drive w;
+  w.sx = (float)(a.ox - a.wall_x + g.nx / 2);
+  w.sy = (float)a.oy;
+  w.sz = (float)a.oz;
+  w.ix = 1.0f / (float)g.nx;
+  w.iy = 1.0f / (float)g.ny;
+  w.iz = 1.0f / (float)g.nz;
+  w.cx = (float)(g.nx / 2) + half_t;
+  w.half = half_t + 1.5f;
+  w.y0 = (float)a.pore_y0 - 0.5f;
+  w.y1 = (float)(a.pore_y0 + a.pore_d) - 0.5f;
+  w.z0 = (float)a.pore_z0 - 0.5f;
+  w.z1 = (float)(a.pore_z0 + a.pore_d) - 0.5f;
+  w.f = a.has_wall && a.pore_d > 0 ? a.fdrive : 0.f;
+  return w;
 }
-
-// Bending (Eq. 3) and the Sec. III pulling force on bead i.
-__device__ F3 bend_drive_forces(const ChainArgs &a, int i, const float4 *s_rh, const float4 *s_rl) {
-  const int N = a.N;
-  F3 F{0.f, 0.f, 0.f};
-  if (a.kappa != 0.f && a.has_bonds) {
-    // bond vectors b_{i-2}, b_{i-1}, b_i, b_{i+1} around bead i
-    F3 bm2{0, 0, 0}, bm1{0, 0, 0}, b0{0, 0, 0}, bp1{0, 0, 0};
-    if (i >= 2) bm2 = diff_hl(s_rh[i - 1], s_rl[i - 1], s_rh[i - 2], s_rl[i - 2]);
-    if (i >= 1) bm1 = diff_hl(s_rh[i], s_rl[i], s_rh[i - 1], s_rl[i - 1]);
-    if (i + 1 < N) b0 = diff_hl(s_rh[i + 1], s_rl[i + 1], s_rh[i], s_rl[i]);
-    if (i + 2 < N) bp1 = diff_hl(s_rh[i + 2], s_rl[i + 2], s_rh[i + 1], s_rl[i + 1]);
-    if (i >= 2) F = F + bend_force(bm2, bm1, a.kappa, 2);
-    if (i >= 1 && i + 1 < N) F = F + bend_force(bm1, b0, a.kappa, 1);
-    if (i + 2 < N) F = F + bend_force(b0, bp1, a.kappa, 0);
-  }
-  // pulling force inside the channel through the pore
-  return F + drive_force_at(a, s_rh[i], s_rl[i]);
+__device__ __forceinline__ float drive_force_at(const Drive &w, const LbGeom &g, float4 rh, float4 rl) {
+  float x = (rh.x + w.sx) + rl.x, y = (rh.y + w.sy) + rl.y, z = (rh.z + w.sz) + rl.z;
+  x -= (float)g.nx * floorf(x * w.ix);  // into [0, n)
+  y -= (float)g.ny * floorf(y * w.iy);
+  z -= (float)g.nz * floorf(z * w.iz);
+  const bool in = fabsf(x - w.cx) <= w.half && y >= w.y0 && y < w.y1 && z >= w.z0 && z < w.z1;
+  return in ? -w.f : 0.f;
 }
 
 // Sum of K values over the block (every thread gets the sums).  red holds
@@ -375,8 +364,8 @@ __device__ __forceinline__ bool solid_geom(const ChainArgs &a, int x, int y, int
 }
 
 // Solid nodes around a bead within `radius` (node offsets n with
-// |n - s| < radius per axis), visited in x, y, z order.  For each solid node
-// calls fn(node coordinate in the chain's local frame).
+// |n - s| < radius per axis).  For each solid node calls fn(node coordinate in
+// the chain's local frame).
 template <typename Fn>
 __device__ __forceinline__ void for_solid_nodes(const ChainArgs &a, float4 rh, float4 rl,
                                                 float radius, Fn fn) {
@@ -385,15 +374,34 @@ __device__ __forceinline__ void for_solid_nodes(const ChainArgs &a, float4 rh, f
   int c[3];
   float sf[3];
   cell_frac_hl(rh.x, rl.x, a.ox, g.nx, c[0], sf[0]);
-  cell_frac_hl(rh.y, rl.y, a.oy, g.ny, c[1], sf[1]);
-  cell_frac_hl(rh.z, rl.z, a.oz, g.nz, c[2], sf[2]);
-  const float fx = floorf(rh.x), fy = floorf(rh.y), fz = floorf(rh.z);
   const int lo0 = (int)ceilf(sf[0] - radius), hi0 = (int)floorf(sf[0] + radius);
-  const int lo1 = (int)ceilf(sf[1] - radius), hi1 = (int)floorf(sf[1] + radius);
-  const int lo2 = (int)ceilf(sf[2] - radius), hi2 = (int)floorf(sf[2] + radius);
-  for (int ox = lo0; ox <= hi0; ++ox) {
+  const float fx = floorf(rh.x), fy = floorf(rh.y), fz = floorf(rh.z);
+  // Without y-walls only the wall layers hold solid nodes: each layer is met
+  // at one offset (the box is wider than the stencil), which is looked up.
+  // Stepping through the offsets instead had the lanes of a warp reach the
+  // layer at different steps, one scan of it behind the other (56-73 k cycles
+  // a list build, against 7 k).
+  const bool layers = !a.y_walls && g.nx > 2 * ((int)radius + 2) + a.wall_t;
+  const int steps = layers ? a.wall_t : hi0 - lo0 + 1;
+  bool ready = false;
+  int lo1 = 0, hi1 = 0, lo2 = 0, hi2 = 0;
+  for (int k = 0; k < steps; ++k) {
+    int ox = lo0 + k;
+    if (layers) {
+      ox = a.wall_x + k - c[0];
+      if (ox < lo0) ox += g.nx;
+      if (ox > hi0) ox -= g.nx;
+      if (ox < lo0 || ox > hi0) continue;
+    }
     const int x = wrap_near(c[0] + ox, g.nx);
     if (!a.y_walls && !wall_layer(a, x)) continue;  // no solid node in this layer
+    if (!ready) {  // few beads get here
+      ready = true;
+      cell_frac_hl(rh.y, rl.y, a.oy, g.ny, c[1], sf[1]);
+      cell_frac_hl(rh.z, rl.z, a.oz, g.nz, c[2], sf[2]);
+      lo1 = (int)ceilf(sf[1] - radius), hi1 = (int)floorf(sf[1] + radius);
+      lo2 = (int)ceilf(sf[2] - radius), hi2 = (int)floorf(sf[2] + radius);
+    }
     for (int oy = lo1; oy <= hi1; ++oy) {
       const int y = wrap_near(c[1] + oy, g.ny);
       for (int oz = lo2; oz <= hi2; ++oz) {
@@ -412,100 +420,267 @@ __device__ __forceinline__ void wall_add(float4 rh, float4 rl, float4 node, floa
           eps24, F);
 }
 
-// Bead i's pair forces from its shared-memory list and wall forces from its
-// solid-node list: the shared-memory copy SW (column i, entry q at SW[q N])
-// when nws >= 0, else the workspace list.
-__device__ __forceinline__ F3 list_forces(const ChainArgs &a, int i, float4 rh, float4 rl,
-                                          const float4 *s_rh, const float4 *s_rl,
-                                          const short *L, int np, const short4 *SW, int nws) {
-  const LbGeom &g = a.geo;
+// The minimum image of a separation.
+__device__ __noinline__ F3 min_image(const LbGeom &g, F3 d) {
+  const float Lx = (float)g.nx, Ly = (float)g.ny, Lz = (float)g.nz;
+  d.x -= Lx * rintf(d.x * (1.0f / Lx));
+  d.y -= Ly * rintf(d.y * (1.0f / Ly));
+  d.z -= Lz * rintf(d.z * (1.0f / Lz));
+  return d;
+}
+
+// Bead i's pair and wall forces from its own lists in the workspace
+// (kNlBead).
+__device__ __noinline__ F3 list_forces(const ChainArgs &a, int i, float4 rh, float4 rl,
+                                          const float4 *s_rh, const float4 *s_rl) {
   const float sig2 = a.sigma * a.sigma;
   const float rc = kTwoSixth * a.sigma, rc2 = rc * rc;
   const float eps24 = 24.0f * a.eps;
-  const float Lx = (float)g.nx, Ly = (float)g.ny, Lz = (float)g.nz;
-  const float iLx = 1.0f / Lx, iLy = 1.0f / Ly, iLz = 1.0f / Lz;
   F3 F{0.f, 0.f, 0.f};
+  const int np = a.nl_cnt[i], nw = a.wl_cnt[i];
+  const short *L = a.nl_list + (size_t)i * kMaxPairs;
   for (int q = 0; q < np; ++q) {
-    const int j = L[q * a.N];
-    F3 d = diff_hl(rh, rl, s_rh[j], s_rl[j]);
-    d.x -= Lx * rintf(d.x * iLx);
-    d.y -= Ly * rintf(d.y * iLy);
-    d.z -= Lz * rintf(d.z * iLz);
-    wca_add(d, sig2, rc2, eps24, F);
+    const int j = L[q] & (LBMD_MAX_BEADS - 1);
+    wca_add(min_image(a.geo, diff_hl(rh, rl, s_rh[j], s_rl[j])), sig2, rc2, eps24, F);
   }
-  if (nws >= 0) {
-#pragma unroll 4
-    for (int q = 0; q < nws; ++q) {
-      const short4 w = SW[q * a.N];
-      wall_add(rh, rl, make_float4((float)w.x, (float)w.y, (float)w.z, 0.f), sig2, rc2, eps24, F);
-    }
-    return F;
-  }
-  const int nw = a.wl_cnt[i];
   const float4 *W = a.wl_list + (size_t)i * kMaxWall;
 #pragma unroll 4
   for (int q = 0; q < nw; ++q) wall_add(rh, rl, W[q], sig2, rc2, eps24, F);
   return F;
 }
 
-// A wall node's local coordinates fit the shared-memory entry.
+// An entry of the flat force list: a bead and its partner, another bead or a
+// solid node, in 64 bits -- x: bead (10 bits), the entry's number among the
+// bead's own (5 bits, kItemTail from there on), kItemWall, and the node's x
+// coordinate in the upper half; y: the partner bead | kItemImage, or the
+// node's y and z coordinates (16-bit integers of the chain's local frame).
+constexpr unsigned kItemTail = 31u;        // summed whether it acts or not
+constexpr unsigned kItemWall = 1u << 15;   // partner is a solid node
+constexpr unsigned kItemImage = 1u << 10;  // the pair reaches across a periodic boundary
+constexpr short kPairImage = 1 << 14;      // the same in a bead's pair list
 __device__ __forceinline__ bool fits_short(float4 n) {
   return fabsf(n.x) <= 32000.f && fabsf(n.y) <= 32000.f && fabsf(n.z) <= 32000.f;
 }
 
-// Rebuild bead i's lists with cutoff r_c + skin: pair list (shared memory,
-// column i, entry q at L[q N]; copied to the workspace for the next launch)
-// and solid-node list (workspace, and its shared copy SW when not null and
-// it fits: *nws = its length, else -1).  Solid nodes are kept within the
-// sphere of radius r_c + skin (a node beyond it exerts no force while the
-// bead stays within half the skin of the build position).  Returns the pair
-// count, or -1 on overflow.
-__device__ int build_lists(const ChainArgs &a, int i, float4 rh, float4 rl, const float4 *s_rh,
-                           const float4 *s_rl, short *L, short4 *SW, int *nws) {
+// Evaluates the flat list: `who` of `of` threads share the entries.  An entry
+// within the cutoff leaves its force in s_f and a bit in its bead's mask (the
+// entry's number among the bead's own); integer ORs commute, so the result does
+// not depend on the order of the threads.
+//
+// With a list per bead the chain waited for its fullest one (a bead in the
+// pore: ~25 entries at ~200-290 cycles each, 3.5-5 k cycles of every substep).
+// Spread over the block, two entries at a time.  The low parts of the positions
+// are read only near the cutoff: they change a separation by no more than 0.1
+// while the local coordinates stay below 1e6.
+__device__ __forceinline__ void eval_items(const ChainArgs &a, const uint2 *s_item, int n, int who,
+                                           int of, const float4 *s_rh, const float4 *s_rl, float4 *s_f,
+                                           unsigned *s_mask) {
+  const float sig2 = a.sigma * a.sigma;
+  const float rc = kTwoSixth * a.sigma, rc2 = rc * rc, reach2 = (rc + 0.2f) * (rc + 0.2f);
+  const float eps24 = 24.0f * a.eps;
+#pragma unroll 1
+  for (int q0 = who; q0 < n; q0 += 2 * of) {
+    uint2 it[2];
+    float4 rh[2], oh[2];
+    it[0] = s_item[q0];
+    it[1] = s_item[min(q0 + of, n - 1)];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int i = it[k].x & (LBMD_MAX_BEADS - 1);
+      rh[k] = s_rh[i];
+      oh[k] = s_rh[(it[k].x & kItemWall) ? i : (int)(it[k].y & (LBMD_MAX_BEADS - 1))];
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int q = q0 + k * of;
+      const bool wall = (it[k].x & kItemWall) != 0;
+      const unsigned bit = (it[k].x >> 10) & 31u;
+      if (wall) {
+        oh[k].x = (float)((int)it[k].x >> 16);
+        oh[k].y = (float)(short)(it[k].y & 0xffffu);
+        oh[k].z = (float)((int)it[k].y >> 16);
+      }
+      F3 d{rh[k].x - oh[k].x, rh[k].y - oh[k].y, rh[k].z - oh[k].z};
+      const bool image = !wall && (it[k].y & kItemImage) != 0;
+      if (q < n && (dot(d, d) < reach2 || image || bit == kItemTail)) {
+        const int i = it[k].x & (LBMD_MAX_BEADS - 1);
+        const float4 rl = s_rl[i];
+        float4 ol = s_rl[wall ? i : (int)(it[k].y & (LBMD_MAX_BEADS - 1))];
+        if (wall) ol = make_float4(0.f, 0.f, 0.f, 0.f);
+        d = diff_hl(rh[k], rl, oh[k], ol);
+        if (image) d = min_image(a.geo, d);
+        const float r2 = dot(d, d);
+        const bool in = r2 < rc2;
+        const float ir2 = rcp_newton(r2);
+        const float sr2 = sig2 * ir2;
+        const float sr6 = sr2 * sr2 * sr2;
+        const float f = eps24 * (2.0f * sr6 * sr6 - sr6) * ir2;
+        if (in || bit == kItemTail) s_f[q] = in ? f4(f * d) : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (in && bit != kItemTail) atomicOr(&s_mask[i], 1u << bit);
+      }
+    }
+  }
+}
+
+// Rebuild the lists of bead i (thread i; called by the whole block, `bead`
+// false for threads without one) with cutoff r_c + skin, in the workspace: the
+// bead's pairs and solid nodes, and from them the flat list, which goes to
+// shared memory as well.  Solid nodes are kept within the sphere of radius
+// r_c + skin (a node beyond it exerts no force while the bead stays within
+// half the skin of the build position).  Returns the kind of list that holds
+// (kNl*), the same on every thread; *n_items entries of the flat one, of which
+// *cnt from s_first[i] on are the bead's.
+//
+// The chain is walked in groups of 32 consecutive beads, which lie close
+// together: a warp passes over a group whose bounding box is beyond the
+// cutoff of all its beads, and tests the others branch-free into a bit mask,
+// whose few set bits are then appended in bead order.
+__device__ __noinline__ int build_lists(const ChainArgs &a, int i, bool bead, float4 rh, float4 rl,
+                           const float4 *s_rh, const float4 *s_rl, uint2 *s_item, int *s_first,
+                           int *n_items, int *cnt) {
+  __shared__ float s_box[32][8];  // per group: centre and half extents (x, y, z)
+  __shared__ int s_sum[32];
   const LbGeom &g = a.geo;
-  const int N = a.N;
+  const int N = a.N, groups = (N + 31) >> 5, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float rlist = kTwoSixth * a.sigma + kSkin, rl2 = rlist * rlist;
   const float Lx = (float)g.nx, Ly = (float)g.ny, Lz = (float)g.nz;
   const float iLx = 1.0f / Lx, iLy = 1.0f / Ly, iLz = 1.0f / Lz;
-  short *G = a.nl_list + (size_t)i * kMaxPairs;
-  int np = 0;
-  for (int j = 0; j < N; ++j) {
-    const int dij = j - i;
-    if (dij == 0 || (a.has_bonds && (dij == 1 || dij == -1))) continue;
-    F3 d = diff_hl(rh, rl, s_rh[j], s_rl[j]);
-    d.x -= Lx * rintf(d.x * iLx);
-    d.y -= Ly * rintf(d.y * iLy);
-    d.z -= Lz * rintf(d.z * iLz);
-    if (dot(d, d) < rl2) {
-      if (np < kMaxPairs) {
-        L[np * N] = (short)j;
-        G[np] = (short)j;
-      }
-      ++np;
+  {
+    const float big = 3.0e38f;
+    F3 lo = bead ? f3(rh) : F3{big, big, big}, hi = bead ? f3(rh) : F3{-big, -big, -big};
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) {
+      lo.x = fminf(lo.x, __shfl_xor_sync(0xffffffffu, lo.x, m));
+      lo.y = fminf(lo.y, __shfl_xor_sync(0xffffffffu, lo.y, m));
+      lo.z = fminf(lo.z, __shfl_xor_sync(0xffffffffu, lo.z, m));
+      hi.x = fmaxf(hi.x, __shfl_xor_sync(0xffffffffu, hi.x, m));
+      hi.y = fmaxf(hi.y, __shfl_xor_sync(0xffffffffu, hi.y, m));
+      hi.z = fmaxf(hi.z, __shfl_xor_sync(0xffffffffu, hi.z, m));
+    }
+    if (lane == 0 && warp < groups) {
+      float *b = s_box[warp];
+      b[0] = 0.5f * (lo.x + hi.x);
+      b[1] = 0.5f * (lo.y + hi.y);
+      b[2] = 0.5f * (lo.z + hi.z);
+      b[3] = 0.5f * (hi.x - lo.x);
+      b[4] = 0.5f * (hi.y - lo.y);
+      b[5] = 0.5f * (hi.z - lo.z);
     }
   }
+  __syncthreads();
+  short *G = a.nl_list + (size_t)i * kMaxPairs;
   float4 *W = a.wl_list + (size_t)i * kMaxWall;
-  int nw = 0;
-  bool packed = SW != nullptr;
-  for_solid_nodes(a, rh, rl, rlist, [&](float4 node) {
-    const F3 d{(rh.x - node.x) + rl.x, (rh.y - node.y) + rl.y, (rh.z - node.z) + rl.z};
-    if (!(dot(d, d) < rl2)) return;
-    if (nw < kMaxWall) W[nw] = node;
-    if (packed && nw < kWallShared && fits_short(node))
-      SW[nw * N] = make_short4((short)node.x, (short)node.y, (short)node.z, 0);
-    else
-      packed = false;
-    ++nw;
-  });
-  *nws = packed ? nw : -1;
-  a.nl_cnt[i] = min(np, kMaxPairs);
-  a.wl_cnt[i] = min(nw, kMaxWall);
-  a.nl_ref[i] = rh;
-  return (np <= kMaxPairs && nw <= kMaxWall) ? np : -1;
+  int np = 0, nw = 0;
+  // a pair of the list moves by at most two half skins until the next
+  // rebuild: within this box width it keeps the image it has now
+  const float room = 2.02f * (rlist + kSkin);
+  const bool small = !(Lx > room && Ly > room && Lz > room);
+  if (warp < groups) {
+    for (int c = 0; c < groups; ++c) {
+      const float *b = s_box[c];
+      float ax = rh.x - b[0], ay = rh.y - b[1], az = rh.z - b[2];
+      ax = fmaxf(fabsf(ax - Lx * rintf(ax * iLx)) - b[3], 0.f);
+      ay = fmaxf(fabsf(ay - Ly * rintf(ay * iLy)) - b[4], 0.f);
+      az = fmaxf(fabsf(az - Lz * rintf(az * iLz)) - b[5], 0.f);
+      // beyond the cutoff with room for rounding; a NaN goes on to the test
+      const bool far = !bead || ax * ax + ay * ay + az * az > 1.01f * rl2 + 0.01f;
+      if (__all_sync(0xffffffffu, far)) continue;
+      const int j0 = c << 5, nj = min(32, N - j0);
+      unsigned mask = 0u;
+#pragma unroll 4
+      for (int jj = 0; jj < nj; ++jj) {
+        F3 d = diff_hl(rh, rl, s_rh[j0 + jj], s_rl[j0 + jj]);
+        d.x -= Lx * rintf(d.x * iLx);
+        d.y -= Ly * rintf(d.y * iLy);
+        d.z -= Lz * rintf(d.z * iLz);
+        if (dot(d, d) < rl2) mask |= 1u << jj;
+      }
+      // not the bead itself, nor its bonded neighbours
+      const int own = i - j0, reach = a.has_bonds ? 1 : 0;
+      for (int k = own - reach; k <= own + reach; ++k)
+        if (k >= 0 && k < 32) mask &= ~(1u << k);
+      if (!bead) mask = 0u;
+      while (mask) {
+        const int j = j0 + __ffs(mask) - 1;
+        mask &= mask - 1u;
+        const F3 d = diff_hl(rh, rl, s_rh[j], s_rl[j]);
+        const bool image = small || rintf(d.x * iLx) != 0.f || rintf(d.y * iLy) != 0.f ||
+                           rintf(d.z * iLz) != 0.f;
+        if (np < kMaxPairs) G[np] = (short)(j | (image ? kPairImage : 0));
+        ++np;
+      }
+    }
+  }
+  bool fit = true;
+  if (bead) {
+    for_solid_nodes(a, rh, rl, rlist, [&](float4 node) {
+      const F3 d{(rh.x - node.x) + rl.x, (rh.y - node.y) + rl.y, (rh.z - node.z) + rl.z};
+      if (!(dot(d, d) < rl2)) return;
+      if (nw < kMaxWall) W[nw] = node;
+      fit = fit && fits_short(node);
+      ++nw;
+    });
+    a.nl_cnt[i] = min(np, kMaxPairs);
+    a.wl_cnt[i] = min(nw, kMaxWall);
+    a.nl_ref[i] = rh;
+  }
+  const int held = __syncthreads_and(np <= kMaxPairs && nw <= kMaxWall);
+  if (!held) return kNlNone;
+  // entries before this bead's: sums over the warp, then over the warps
+  int upto = np + nw;
+#pragma unroll
+  for (int m = 1; m < 32; m <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, upto, m);
+    if (lane >= m) upto += t;
+  }
+  if (lane == 31) s_sum[warp] = upto;
+  __syncthreads();
+  int before = 0, total = 0;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+    if (w < warp) before += s_sum[w];
+    total += s_sum[w];
+  }
+  if (!__syncthreads_and(fit && total <= item_cap(N))) return kNlBead;
+  if (bead) {
+    const int q = before + upto - (np + nw);
+    s_first[i] = q;
+    a.it_first[i] = q | (np + nw) << 16;
+    const auto tag = [&](int e) { return (unsigned)i | min((unsigned)e, kItemTail) << 10; };
+    const auto put = [&](int e, uint2 it) {
+      s_item[q + e] = it;
+      a.items[q + e] = it;
+    };
+    // read back what this thread has just written, in wide or several loads
+    for (int k0 = 0; k0 < np; k0 += 8) {
+      const uint4 g8 = reinterpret_cast<const uint4 *>(G)[k0 >> 3];
+      const unsigned g2[4] = {g8.x, g8.y, g8.z, g8.w};
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const unsigned v = g2[k >> 1] >> (16 * (k & 1));
+        if (k0 + k < np)
+          put(k0 + k, make_uint2(tag(k0 + k), (v & (LBMD_MAX_BEADS - 1)) | ((v & kPairImage) ? kItemImage : 0u)));
+      }
+    }
+    for (int k0 = 0; k0 < nw; k0 += 8) {
+      float4 v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (k0 + k < nw) v[k] = W[k0 + k];
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (k0 + k < nw)
+          put(np + k0 + k, make_uint2(tag(np + k0 + k) | kItemWall | ((unsigned)(int)v[k].x << 16),
+                                      ((unsigned)(int)v[k].y & 0xffffu) | ((unsigned)(int)v[k].z << 16)));
+    }
+  }
+  *n_items = total;
+  *cnt = np + nw;
+  __syncthreads();
+  return kNlFlat;
 }
 
 // Without lists (overflow): wall forces by scanning the stencil.
-__device__ F3 wall_stencil_forces(const ChainArgs &a, float4 rh, float4 rl) {
+__device__ __noinline__ F3 wall_stencil_forces(const ChainArgs &a, float4 rh, float4 rl) {
   const float sig2 = a.sigma * a.sigma;
   const float rc = kTwoSixth * a.sigma, rc2 = rc * rc;
   const float eps24 = 24.0f * a.eps;
@@ -592,95 +767,224 @@ __device__ __forceinline__ void spread_finalize(const ChainArgs &a, int e) {
 }
 
 // (2) the M MD substeps of one chain, one thread per bead, and (5) the
-// bookkeeping; `a` may live in parameter or shared memory.
-template <bool WS>
+// bookkeeping; `a` may live in parameter or shared memory.  BLOCK is the
+// register class (512 or 1024 threads).
+//
+// One chain is one block, so a substep is a chain of dependent phases and its
+// bound is their latency.  The positions of a substep are final after SHAKE, so
+// the next substep's forces, bond vectors and noise are found by the bead
+// warps while one warp solves RATTLE; what is left in line is: velocities and
+// the sum of the acting forces, one barrier, two Newton iterations (rows and
+// vote, solve, barrier), a last vote, positions and RATTLE's rows, one vote, the
+// solve, one barrier.  A thread keeps its own and its successor's displacement,
+// both updated by the same operations, so the Newton iterations exchange
+// nothing but the rows and the solution.
+template <int BLOCK>
 __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
   extern __shared__ float4 smem4[];
   const int N = a.N;
   const int i = threadIdx.x;  // bead of this thread
   const bool bead = i < N;
-  float4 *s_rh = smem4;       // positions, hi part (start of the substep)
-  float4 *s_rl = s_rh + N;    // positions, lo part
-  float4 *s_t = s_rl + N;     // displacement of the substep
-  float4 *s_b = s_t + N;      // bond vectors
-  float4 *s_v = s_b + N;      // velocities (RATTLE)
-  float *s_lam = (float *)(s_v + N);  // N: SHAKE multipliers of the last substep
-  short *s_nl = (short *)(s_lam + N);  // [kMaxPairs][N] pair lists, column per bead
-  // [kWallShared][N] wall lists, column per bead (WS: chains of <= 512 beads)
-  short4 *s_w = WS ? (short4 *)((char *)smem4 + md_smem_head(N)) : nullptr;
-  int nws = -1;  // length of this bead's shared wall list, -1: read the workspace
+  // the warp of the tridiagonal solves: the last one, or the first of a block
+  // without a spare one
+  const bool spare = (int)blockDim.x > bead_threads(N);
+  const bool solves = spare ? i >= bead_threads(N) : i < 32;
+  const int rows = 32 * solve_rows(N);
+  float4 *s_row = smem4;         // rows of the tridiagonal system to solve
+  float4 *s_full = s_row + rows; // halved rows: the whole system, two buffers
+  float4 *s_rh = s_full + (BLOCK > 512 ? 2 * (N + 1) : 0);  // positions, hi part (start of the substep)
+  float4 *s_rl = s_rh + N;       // positions, lo part
+  float4 *s_b = s_rl + N;        // bond vectors, start of the substep
+  float4 *s_t = s_b + N;         // unconstrained displacement of the substep
+  float4 *s_d = s_t + N;         // bond vectors at the end of the substep
+  float *s_x = (float *)(s_d + N);                 // solution of the tridiagonal system
+  float *s_lam = s_x + rows;                       // SHAKE multipliers of the last substep
+  unsigned *s_mask = (unsigned *)(s_lam + N);      // acting entries of the bead's flat list
+  float4 *s_f = (float4 *)((char *)smem4 + md_smem_head(N));  // their forces
+  uint2 *s_item = (uint2 *)(s_f + item_cap(N));               // the flat list
+  __shared__ int s_first[BLOCK];                              // a bead's first entry
 
-  const long long step = a.status->step;
-  int nl_ok = a.status->nl_ok && a.status->nl_builds > 0;
+  const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int q = (BLOCK > 512 ? (N - 1) / 2 : max(N - 1, 0)) + i; q < rows; q += blockDim.x) s_row[q] = none;
+  if (BLOCK > 512 && i < 2) s_full[i * (N + 1) + N - 1] = none;  // the row after the last
+
+  const DevStatus *st0 = a.status;
+  const long long step = st0->step;
+  const int max_trans0 = st0->max_trans, state0 = st0->state;
+  const bool lists = a.eps != 0.f;
+  int nl_ok = st0->nl_builds > 0 ? st0->nl_ok : kNlNone, n_items = st0->nl_items, n_own = 0;
   float4 rh = make_float4(0, 0, 0, 0), rl = rh, ref = rh;
   F3 v{0.f, 0.f, 0.f}, ui{0.f, 0.f, 0.f};
-  int np = 0;  // length of this bead's pair list
+  double b0 = 1.0;
   if (bead) {
     rh = a.pos[i];
     rl = a.pos_lo[i];
     ref = a.nl_ref[i];
     v = f3(a.vel[i]);
-    ui = f3(a.ui[i]);  // (1) interpolated by k_gather, frozen for the M substeps
+    const float lam0 = a.lam[i];
+    const int own = a.it_first[i];
+    if (i < N - 1 && a.has_bonds) b0 = a.b0[i];
     s_rh[i] = rh;
     s_rl[i] = rl;
-    s_lam[i] = a.lam[i];
-    if (nl_ok) {
-      np = a.nl_cnt[i];
-      const short *G = a.nl_list + (size_t)i * kMaxPairs;
-      for (int q = 0; q < np; ++q) s_nl[q * N + i] = G[q];
-      if (WS) {
-        // this launch's substeps read the wall list from shared memory
-        const int nw = a.wl_cnt[i];
-        if (nw <= kWallShared) {
-          const float4 *W = a.wl_list + (size_t)i * kMaxWall;
-          bool fit = true;
-#pragma unroll 4
-          for (int q = 0; q < nw; ++q) {
-            const float4 node = W[q];
-            fit = fit && fits_short(node);
-            s_w[q * N + i] = make_short4((short)node.x, (short)node.y, (short)node.z, 0);
-          }
-          nws = fit ? nw : -1;
-        }
-      }
-    }
+    s_lam[i] = lam0;
+    s_mask[i] = 0u;
+    s_first[i] = own & 0xffff;
+    n_own = own >> 16;
   }
+  if (nl_ok == kNlFlat)
+    for (int q = i; q < n_items; q += 4 * blockDim.x) {  // four loads in flight
+      uint2 it[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (q + k * (int)blockDim.x < n_items) it[k] = a.items[q + k * blockDim.x];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (q + k * (int)blockDim.x < n_items) s_item[q + k * blockDim.x] = it[k];
+    }
+  // Noise of every substep: a loop of its own, whose instructions stay in
+  // the instruction cache over its turns (in the substep they do not: the
+  // substep's code then exceeds it and is fetched anew each time).
+#pragma unroll 1
+  for (int k = 0; k < a.M; ++k)
+    if (bead) {
+      const float3 xi = gauss3(a.seed, (uint32_t)i, step, (uint32_t)k, 0u);
+      a.noise[(size_t)k * N + i] = make_float4(xi.x, xi.y, xi.z, 0.f);
+    }
   const float half_skin2 = 0.25f * kSkin * kSkin;
   auto moved = [&]() {
     const float dx = rh.x - ref.x, dy = rh.y - ref.y, dz = rh.z - ref.z;
     return !(dx * dx + dy * dy + dz * dz <= half_skin2);
   };
-  int rebuild = __syncthreads_or(bead && (!nl_ok || moved()));
+  int rebuild = __syncthreads_or(bead && (nl_ok == kNlNone || moved()));
   F3 J{0.f, 0.f, 0.f};
   const float dt = a.dt, m = a.mass, im = 1.0f / a.mass, idt = 1.0f / a.dt;
   const float sig_r = sqrtf(2.0f * m * a.gamma * a.kT / dt);
-  const double b0 = (bead && i < N - 1 && a.has_bonds) ? a.b0[i] : 1.0;
+  const float b02 = (float)(b0 * b0);
   const float tol = fmaxf(a.shake_tol, 5e-7f);
+  const bool bond = a.has_bonds && i < N - 1;  // bond (i, i + 1)
+  const bool bends = a.kappa != 0.f && a.has_bonds;
+  const Drive drive = drive_of(a);
   int shake_bad = 0, newton_total = 0, builds = 0;
+  // A row of the tridiagonal system, the solve (between two block barriers)
+  // and an unknown of it.  With halved rows the rows of successive solves take
+  // two buffers in turn: a thread may still look up an even unknown while
+  // another writes its next row.
+  constexpr bool HALF = BLOCK > 512;
+  int turn = 0;
+  auto put_row = [&](float4 r) { (HALF ? s_full + turn * (N + 1) : s_row)[i] = r; };
+  auto solve = [&]() {
+    const int n = N - 1;
+    if (HALF) {
+      const float4 *f = s_full + turn * (N + 1);
+      turn ^= 1;
+      if ((i & 1) && i < n) s_row[i >> 1] = halve_row(f[i - 1], f[i], f[i + 1]);
+      __syncthreads();
+      if (!solves) return;
+      if (n / 2 <= 32 * 13)
+        tri_solve_warp<13>(n / 2, s_row, s_x);
+      else
+        tri_solve_warp<17>(n / 2, s_row, s_x);
+      return;
+    }
+    if (!solves) return;
+    if (n <= 32 * 5)
+      tri_solve_warp<5>(n, s_row, s_x);
+    else if (n <= 32 * 13)
+      tri_solve_warp<13>(n, s_row, s_x);
+    else
+      tri_solve_warp<17>(n, s_row, s_x);
+  };
+  auto unknown = [&](int j) {  // x_j of the last solve, 0 <= j < N - 1
+    if (!HALF) return s_x[j];
+    if (j & 1) return s_x[j >> 1];
+    const float4 r = s_full[(turn ^ 1) * (N + 1) + j];
+    const float xm = j > 0 ? s_x[(j >> 1) - 1] : 0.f, xp = j + 1 < N - 1 ? s_x[j >> 1] : 0.f;
+    return fmaf(-r.y, xp, fmaf(-r.x, xm, r.z));
+  };
+  // What the coming substep k needs of the positions now in s_rh, s_rl (every
+  // thread has passed a barrier since they were written; another follows
+  // before the results are read): noise, the force on this bead from the
+  // drive and from bending (the shares of its angle on the neighbours left
+  // in s_d and in the unused components of s_rh, s_rl and s_b), its bond
+  // vector and the entries of the flat list.
+  float4 xi = make_float4(0.f, 0.f, 0.f, 0.f);
+  F3 Fp{0.f, 0.f, 0.f};
+  auto prepare = [&](int k) {
+    if (lists && nl_ok == kNlFlat && !(spare && solves))
+      eval_items(a, s_item, n_items, i, spare ? bead_threads(N) : (int)blockDim.x, s_rh, s_rl, s_f,
+                 s_mask);
+    if (!bead) return;
+    xi = a.noise[(size_t)k * N + i];  // this thread wrote it
+    F3 sb{0.f, 0.f, 0.f};
+    Fp = F3{0.f, 0.f, 0.f};
+    if (bond) sb = diff_hl(s_rh[i + 1], s_rl[i + 1], rh, rl);
+    float4 keep = f4(sb);
+    if (bends) {
+      F3 fa{0.f, 0.f, 0.f}, fc = fa;
+      if (i >= 1 && i + 1 < N)
+        bend_forces(diff_hl(rh, rl, s_rh[i - 1], s_rl[i - 1]), sb, a.kappa, fa, Fp, fc);
+      s_d[i] = f4(fc);
+      keep.w = fa.x;
+      s_rh[i].w = fa.y;
+      s_rl[i].w = fa.z;
+    }
+    if (bond || bends) s_b[i] = keep;
+    // pulling force inside the channel through the pore
+    Fp.x += drive_force_at(drive, a.geo, rh, rl);
+  };
+  F3 D1{0.f, 0.f, 0.f};  // displacement of bead i + 1
+  F3 d{0.f, 0.f, 0.f};   // bond vector i at the end of the substep
+  F3 dm{0.f, 0.f, 0.f};  // bond vector i - 1 there
 
-  for (int k = 0; k < a.M; ++k) {  // (2) M MD substeps
-    if (rebuild && a.eps != 0.f) {
+  // (2) M MD substeps.  One turn ends substep k - 1 (RATTLE) and takes substep
+  // k up to its positions, so that every phase stands in the code once.
+  for (int k = 0;; ++k) {
+    if (rebuild && lists && k < a.M) {
       // neighbour lists: pairs and solid nodes within r_c + skin
-      int cnt = 0;
-      if (bead) {
-        cnt = build_lists(a, i, rh, rl, s_rh, s_rl, s_nl + i, WS ? s_w + i : nullptr, &nws);
-        ref = rh;
-      }
-      nl_ok = __syncthreads_and(cnt >= 0);
-      np = cnt < 0 ? 0 : cnt;
+      nl_ok = build_lists(a, i, bead, rh, rl, s_rh, s_rl, s_item, s_first, &n_items, &n_own);
+      ref = rh;
       ++builds;
     }
-    F3 D{0.f, 0.f, 0.f};
+    if (a.has_bonds && k > 0) solve();
+    if (k < a.M) prepare(k);
+    __syncthreads();
+    if (a.has_bonds && bead && k > 0) {
+      if (bond) v = axpy(unknown(i) * im, d, v);
+      if (i > 0) v = axpy(-(unknown(i - 1) * im), dm, v);
+    }
+    if (k == a.M) break;
+    if (k == 0) {
+      // (1) interpolated by k_gather, beside which this block may have
+      // started; frozen for the M substeps
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      if (bead) ui = f3(a.ui[i]);
+    }
+    // bond vectors s_{i-1}, s_i, s_{i+1} around the bead
+    F3 sm{0.f, 0.f, 0.f}, sb{0.f, 0.f, 0.f}, sp{0.f, 0.f, 0.f}, D{0.f, 0.f, 0.f};
+    float lam = 0.f;  // multiplier of bond i
     if (bead) {
-      F3 Fc = bend_drive_forces(a, i, s_rh, s_rl);
-      if (a.eps != 0.f) {
-        if (nl_ok)
-          Fc = Fc + list_forces(a, i, rh, rl, s_rh, s_rl, s_nl + i, np, WS ? s_w + i : nullptr,
-                                WS ? nws : -1);
-        else
-          Fc = Fc + all_pair_forces(a, i, rh, rl, s_rh, s_rl) + wall_stencil_forces(a, rh, rl);
+      F3 Fc = Fp;
+      if (bends) {
+        Fc = F3{0.f, 0.f, 0.f};
+        if (i >= 2) Fc = Fc + f3(s_d[i - 1]);
+        Fc = Fc + Fp;
+        if (i + 2 < N) Fc = Fc + F3{s_b[i + 1].w, s_rh[i + 1].w, s_rl[i + 1].w};
       }
-      const float3 xi = gauss3(a.seed, (uint32_t)i, step, (uint32_t)k, 0u);
+      if (lists) {
+        F3 F{0.f, 0.f, 0.f};
+        if (nl_ok == kNlFlat) {
+          const float4 *f = s_f + s_first[i];
+          unsigned mask = s_mask[i];
+          s_mask[i] = 0u;
+          for (; mask; mask &= mask - 1u) F = F + f3(f[__ffs(mask) - 1]);
+          for (int q = (int)kItemTail; q < n_own; ++q) F = F + f3(f[q]);
+        } else if (nl_ok == kNlBead) {
+          F = list_forces(a, i, rh, rl, s_rh, s_rl);
+        } else {
+          F = all_pair_forces(a, i, rh, rl, s_rh, s_rl) + wall_stencil_forces(a, rh, rl);
+        }
+        Fc = Fc + F;
+      }
       const F3 fdrag = (-m * a.gamma) * (v - ui);
       const F3 fr = sig_r * F3{xi.x, xi.y, xi.z};
       v = v + (dt * im) * (Fc + fdrag + fr);
@@ -690,98 +994,85 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
     if (a.has_bonds) {
       // SHAKE on displacements: D_i = dt v_i + (lam_i s_i - lam_{i-1} s_{i-1}) / m
       // with the old bond vectors s_b; Newton on G_b = |s_b + D_{b+1} - D_b|^2 - b0^2.
-      // The residual is evaluated in double (old bond from the double-float
-      // positions); the Jacobian and the corrections stay in float.
+      // Old bonds come from the double-float positions; the rows are divided
+      // by their diagonals -4 d_b . s_b / m.
       // Warm start: the multipliers of the previous substep applied along the
       // new old-bond vectors (the constraint forces change slowly).
-      float lam = 0.f;
-      F3 sb{0.f, 0.f, 0.f};
       if (bead) {
-        F3 sm{0.f, 0.f, 0.f};
-        if (i > 0) sm = diff_hl(rh, rl, s_rh[i - 1], s_rl[i - 1]);
-        if (i < N - 1) {
-          sb = diff_hl(s_rh[i + 1], s_rl[i + 1], rh, rl);
-          s_b[i] = f4(sb);
+        if (bond) {
+          sb = f3(s_b[i]);
           lam = s_lam[i];
-          D = D + (lam * im) * sb;
+          D = axpy(lam * im, sb, D);
         }
-        if (i > 0) D = D - (s_lam[i - 1] * im) * sm;
+        if (i > 0) {
+          sm = f3(s_b[i - 1]);
+          D = axpy(-(s_lam[i - 1] * im), sm, D);
+        }
+        if (i < N - 2) sp = f3(s_b[i + 1]);
         s_t[i] = f4(D);
       }
       __syncthreads();
-      const float b02 = (float)(b0 * b0);
+      if (bond) D1 = f3(s_t[i + 1]);
       for (int it = 0;; ++it) {
-        float G = 0.f, diag = 1.f, sub = 0.f, sup = 0.f;
+        float G = 0.f;
         bool ok = true;
-        if (i < N - 1) {
+        if (bond) {
           // old bond from the double-float positions, displacements small: the
           // float residual is good to ~1e-7 of b0^2
-          const F3 d = sb + (f3(s_t[i + 1]) - f3(s_t[i]));
+          d = sb + (D1 - D);
           G = dot(d, d) - b02;
           ok = fabsf(G) <= tol * b02;
-          diag = -4.0f * im * dot(d, sb);
-          if (i > 0) sub = 2.0f * im * dot(d, f3(s_b[i - 1]));
-          if (i < N - 2) sup = 2.0f * im * dot(d, f3(s_b[i + 1]));
+          const float q = rcp_fast(dot(d, sb)), h = -0.5f * q;
+          put_row(make_float4(i > 0 ? h * dot(d, sm) : 0.f, i < N - 2 ? h * dot(d, sp) : 0.f,
+                              0.25f * m * q * G, 0.f));
+          s_d[i] = f4(d);
         }
         if (__syncthreads_and(ok)) break;
         if (it >= a.shake_maxit) {
-          const bool bad = (i < N - 1) && !(fabsf(G) <= 1e-3f * b02);
+          const bool bad = bond && !(fabsf(G) <= 1e-3f * b02);
           if (__syncthreads_or(bad)) shake_bad = 1;
           break;
         }
         ++newton_total;
-        float xm;
-        const float x = spike_tri_solve(N - 1, sub, diag, sup, -G, xm);
+        solve();
+        __syncthreads();
         if (bead) {
-          F3 dd = f3(s_t[i]);
-          if (i < N - 1) {
-            dd = dd + (x * im) * f3(s_b[i]);
+          // own and next bead's displacement, by the same operations on both
+          // threads that hold it
+          const float x = bond ? unknown(i) : 0.f, xm = i > 0 ? unknown(i - 1) : 0.f;
+          if (bond) {
+            D = axpy(x * im, sb, D);
+            if (i < N - 2) D1 = axpy(unknown(i + 1) * im, sp, D1);
+            D1 = axpy(-(x * im), sb, D1);
             lam += x;
           }
-          if (i > 0) dd = dd - (xm * im) * f3(s_b[i - 1]);
-          s_t[i] = f4(dd);
+          if (i > 0) D = axpy(-(xm * im), sm, D);
         }
-        __syncthreads();
       }
-      if (i < N - 1) s_lam[i] = lam;  // read again only after later barriers
-      if (bead) D = f3(s_t[i]);
+      if (bond) s_lam[i] = lam;  // read again only after later barriers
     }
+    // every read of s_rh / s_rl of this substep precedes a barrier of the
+    // constraint solves; without constraints one barrier is needed here
+    if (!a.has_bonds) __syncthreads();
     if (bead) {
       // v = (r' - r) / dt evaluated as D / dt (no cancellation); r' = r + D
       v = idt * D;
       two_sum_add(rh.x, rl.x, D.x);
       two_sum_add(rh.y, rl.y, D.y);
       two_sum_add(rh.z, rl.z, D.z);
-    }
-    if (a.has_bonds) {
-      // RATTLE: v_i += (mu_i d_i - mu_{i-1} d_{i-1}) / m with the new bond
-      // vectors d_b = s_b + D_{b+1} - D_b, so that d_b . (v_{b+1} - v_b) = 0.
-      if (bead) s_v[i] = f4(v);
-      F3 dnew{0.f, 0.f, 0.f};
-      if (i < N - 1) dnew = f3(s_b[i]) + (f3(s_t[i + 1]) - f3(s_t[i]));
-      __syncthreads();  // s_v complete; every read of s_b / s_t above done
-      if (i < N - 1) s_b[i] = f4(dnew);
-      __syncthreads();
-      float rhs = 0.f, diag = 1.f, sub = 0.f, sup = 0.f;
-      if (i < N - 1) {
-        rhs = dot(dnew, f3(s_v[i + 1]) - v);
-        diag = -2.0f * im * dot(dnew, dnew);
-        if (i > 0) sub = im * dot(dnew, f3(s_b[i - 1]));
-        if (i < N - 2) sup = im * dot(dnew, f3(s_b[i + 1]));
-      }
-      float mum;
-      const float mu = spike_tri_solve(N - 1, sub, diag, sup, -rhs, mum);
-      if (bead) {
-        if (i < N - 1) v = v + (mu * im) * f3(s_b[i]);
-        if (i > 0) v = v - (mum * im) * f3(s_b[i - 1]);
-      }
-    }
-    // every read of s_rh / s_rl of this substep precedes a barrier of the
-    // constraint solves; without constraints one barrier is needed here
-    if (!a.has_bonds) __syncthreads();
-    if (bead) {
       s_rh[i] = rh;
       s_rl[i] = rl;
+    }
+    if (a.has_bonds && bead) {
+      // RATTLE: v_i += (mu_i d_i - mu_{i-1} d_{i-1}) / m with the new bond
+      // vectors d_b = s_b + D_{b+1} - D_b, so that d_b . (v_{b+1} - v_b) = 0;
+      // rows divided by their diagonals -2 d_b . d_b / m.
+      if (i > 0) dm = f3(s_d[i - 1]);
+      if (bond) {
+        const float q = rcp_fast(dot(d, d)), h = -0.5f * q;
+        put_row(make_float4(i > 0 ? h * dot(d, dm) : 0.f, i < N - 2 ? h * dot(d, f3(s_d[i + 1])) : 0.f,
+                            0.5f * m * q * dot(d, idt * D1 - v), 0.f));
+      }
     }
     rebuild = __syncthreads_or(bead && moved());
   }
@@ -803,13 +1094,15 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
   const int bad = __syncthreads_or(shake_bad);
   if (i == 0) {
     DevStatus *st = a.status;
+    const int max_trans = max(max_trans0, nt);  // read at the start: no load here
     st->n_trans = nt;
-    if (nt > st->max_trans) st->max_trans = nt;
+    st->max_trans = max_trans;
     if (bad) st->shake_fail += 1;
     st->newton_iters = newton_total;
-    st->nl_builds += builds;
+    if (builds) st->nl_builds += builds;
     st->nl_ok = nl_ok;
-    if (st->state == LBMD_RUNNING) {
+    st->nl_items = n_items;
+    if (state0 == LBMD_RUNNING) {
       if (nan)
         st->state = LBMD_NAN;
       else if (bad)
@@ -818,7 +1111,7 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
         if (nt == N) {
           st->state = LBMD_TRANSLOCATED;
           st->t_transloc = step + 1;
-        } else if (st->max_trans >= 1 && out) {
+        } else if (max_trans >= 1 && out) {
           st->state = LBMD_RETRACTED;
         }
       }
@@ -839,9 +1132,9 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
     const float it = nt > 0 ? 1.0f / (float)nt : 0.f, iu = nu > 0 ? 1.0f / (float)nu : 0.f;
     const F3 dt_{r.x - c[0] * it, r.y - c[1] * it, r.z - c[2] * it};
     const F3 du_{r.x - c[3] * iu, r.y - c[4] * iu, r.z - c[5] * iu};
-    const F3 fd = bead ? drive_force_at(a, rh, rl) : F3{0.f, 0.f, 0.f};
+    const float fd = bead ? drive_force_at(drive, a.geo, rh, rl) : 0.f;
     float q[5] = {tr ? dot(dt_, dt_) : 0.f, un ? dot(du_, du_) : 0.f, bead ? dot(v, ui) : 0.f,
-                  dot(fd, v), bead ? dot(v, v) : 0.f};
+                  fd * v.x, bead ? dot(v, v) : 0.f};
     block_sum<5>(q, s_red);
     if (i == 0) {
       DevStatus *st = a.status;
@@ -865,14 +1158,14 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
 }
 
 template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK) k_md_cycle(ChainArgs a) {
-  md_cycle_body<BLOCK <= kWallSharedMaxN>(a);
+__global__ void __launch_bounds__(BLOCK, 1) k_md_cycle(ChainArgs a) {
+  md_cycle_body<BLOCK>(a);
 }
 
 // Ensemble variant: block b runs chain chains[b] if its realisation is live.
 // The chain's arguments are copied to shared memory once.
 template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK)
+__global__ void __launch_bounds__(BLOCK, 1)
     k_ens_md_cycle(const EnsMember *__restrict__ mem, const int *__restrict__ chains,
                    const int *__restrict__ live) {
   __shared__ ChainArgs s_a;
@@ -883,7 +1176,7 @@ __global__ void __launch_bounds__(BLOCK)
   int *dst = reinterpret_cast<int *>(&s_a);
   for (int k = threadIdx.x; k < (int)(sizeof(ChainArgs) / sizeof(int)); k += blockDim.x) dst[k] = src[k];
   __syncthreads();
-  md_cycle_body<BLOCK <= kWallSharedMaxN>(s_a);
+  md_cycle_body<BLOCK>(s_a);
 }
 
 // Stage (1) for (bead, corner) pair e = 8 i + k handled by one thread; the
@@ -960,6 +1253,7 @@ __device__ F3 gather_pair(const ChainArgs &a, const void *f, int e, bool valid) 
 
 template <int S>
 __global__ void __launch_bounds__(256) k_gather(ChainArgs a) {
+  asm volatile("griddepcontrol.launch_dependents;");  // the MD block may be placed
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   const bool valid = e < 8 * a.N;
   const F3 u = gather_pair<S>(a, a.f, e, valid);
@@ -984,8 +1278,10 @@ __global__ void __launch_bounds__(256)
 }
 
 cudaError_t md_prepare() {
-  const int s512 = (int)md_smem_bytes(kWallSharedMaxN), s1024 = (int)md_smem_bytes(LBMD_MAX_BEADS);
+  const int s512 = (int)md_smem_bytes(512), s768 = (int)md_smem_bytes(768), s1024 = (int)md_smem_bytes(LBMD_MAX_BEADS);
   cudaError_t e;
+  if ((e = cudaFuncSetAttribute(k_md_cycle<768>, cudaFuncAttributeMaxDynamicSharedMemorySize, s768)) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(k_ens_md_cycle<768>, cudaFuncAttributeMaxDynamicSharedMemorySize, s768)) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(k_md_cycle<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, s512)) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(k_md_cycle<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, s1024)) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(k_ens_md_cycle<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, s512)) != cudaSuccess) return e;
@@ -1006,7 +1302,11 @@ cudaError_t launch_gather(int storage, const ChainArgs &a, cudaStream_t s) {
 
 // The MD block is launched at the highest stream priority so that, when it
 // and the stream-collide become ready together, its block is placed first.
-cudaError_t launch_md_cycle(const ChainArgs &a, int priority, cudaStream_t s) {
+// beside: the kernel before it on `s` is the gather of the same step, which lets
+// this one start beside it (programmatic dependent launch): the block then
+// reads its state and lists, draws its noise and finds its first forces while
+// the gather runs, and waits for it before it takes u_i.
+cudaError_t launch_md_cycle(const ChainArgs &a, int priority, bool beside, cudaStream_t s) {
   if (a.N <= 0) return cudaSuccess;
   const int threads = md_threads(a.N);
   cudaLaunchConfig_t cfg = {};
@@ -1014,12 +1314,15 @@ cudaError_t launch_md_cycle(const ChainArgs &a, int priority, cudaStream_t s) {
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = md_smem_bytes(a.N);
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributePriority;
   attr[0].val.priority = priority;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = beside ? 2 : 1;
   if (threads <= 512) return cudaLaunchKernelEx(&cfg, k_md_cycle<512>, a);
+  if (threads <= 768) return cudaLaunchKernelEx(&cfg, k_md_cycle<768>, a);
   return cudaLaunchKernelEx(&cfg, k_md_cycle<1024>, a);
 }
 
@@ -1216,6 +1519,7 @@ cudaError_t launch_ens_md_cycle(const EnsMember *mem, const int *chains, int cou
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   if (threads <= 512) return cudaLaunchKernelEx(&cfg, k_ens_md_cycle<512>, mem, chains, live);
+  if (threads <= 768) return cudaLaunchKernelEx(&cfg, k_ens_md_cycle<768>, mem, chains, live);
   return cudaLaunchKernelEx(&cfg, k_ens_md_cycle<1024>, mem, chains, live);
 }
 
