@@ -20,7 +20,11 @@ using namespace lbmd;
 
 namespace {
 
-constexpr int kEnsSide = 4;     // side streams for the MD groups
+// Side streams for the MD groups, one per block size there is
+// (md_group_threads), so that no group waits for another: with a group per
+// warp count on four streams, 32 chains of 120 - 400 beads ran ten launches, up
+// to three of them one behind the other (step 437 us, stream-collide 186 us).
+constexpr int kEnsSide = 9;
 constexpr int kEnsBlock = 16;   // steps per long graph
 const int kEnsGraphSteps[3] = {1, 2, kEnsBlock};
 
@@ -528,9 +532,9 @@ int lbmd_ensemble_create(const lbmd_params *members, int32_t count, void *dev_wo
     const int N = members[m].n_beads, Np = (N + 3) / 4 * 4;
     for (int i = 0; i < Np; ++i) beads.push_back(i < N ? make_int2(m, i) : make_int2(-1, 0));
   }
-  // MD groups: chains with the same block size (one thread per bead, whole warps)
+  // MD groups: chains with the same block size
   std::map<int, std::vector<int>> by_threads;
-  for (int m = 0; m < count; ++m) by_threads[md_threads(members[m].n_beads)].push_back(m);
+  for (int m = 0; m < count; ++m) by_threads[md_group_threads(members[m].n_beads)].push_back(m);
   std::vector<int> chains;
   for (auto &kv : by_threads) {
     Group g{kv.first, 0, (int)chains.size(), (int)kv.second.size()};

@@ -165,6 +165,7 @@ struct __align__(16) EnsTile {
 
 size_t md_smem_bytes(int N);
 int md_threads(int N);
+int md_group_threads(int N);
 int md_item_cap(int N);  // entries the flat force list has room for
 // Opt the MD kernels into the dynamic shared memory of the longest chain.
 cudaError_t md_prepare();

@@ -53,6 +53,13 @@ int md_threads(int N) {
   const int t = bead_threads(N);
   return t == 512 || t == 768 || t == LBMD_MAX_BEADS ? t : t + 32;
 }
+// The block of an ensemble's chains: sizes in steps of 64 threads up to 512,
+// then the register classes, so that few launches take chains of every length
+// (nine at most; warps without beads wait at the barriers).
+int md_group_threads(int N) {
+  const int t = md_threads(N);
+  return t <= 512 ? (t + 63) / 64 * 64 : t <= 768 ? 768 : LBMD_MAX_BEADS;
+}
 
 // Chains of more than 512 beads halve their system before the solve: the
 // threads of the odd rows eliminate the even rows beside them (all at once),
@@ -785,10 +792,10 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
   const int N = a.N;
   const int i = threadIdx.x;  // bead of this thread
   const bool bead = i < N;
-  // the warp of the tridiagonal solves: the last one, or the first of a block
-  // without a spare one
+  // the warp of the tridiagonal solves: the one after the beads', or the first
+  // of a block without a spare one
   const bool spare = (int)blockDim.x > bead_threads(N);
-  const bool solves = spare ? i >= bead_threads(N) : i < 32;
+  const bool solves = (i >> 5) == (spare ? bead_threads(N) >> 5 : 0);
   const int rows = 32 * solve_rows(N);
   float4 *s_row = smem4;         // rows of the tridiagonal system to solve
   float4 *s_full = s_row + rows; // halved rows: the whole system, two buffers
@@ -910,7 +917,7 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
   float4 xi = make_float4(0.f, 0.f, 0.f, 0.f);
   F3 Fp{0.f, 0.f, 0.f};
   auto prepare = [&](int k) {
-    if (lists && nl_ok == kNlFlat && !(spare && solves))
+    if (lists && nl_ok == kNlFlat && (!spare || i < bead_threads(N)))
       eval_items(a, s_item, n_items, i, spare ? bead_threads(N) : (int)blockDim.x, s_rh, s_rl, s_f,
                  s_mask);
     if (!bead) return;
