@@ -489,6 +489,8 @@ int lbmd_ensemble_create(const lbmd_params *members, int32_t count, void *dev_wo
   for (cudaEvent_t *ev : {&e->ev_in, &e->ev_out, &e->ev_fork})
     if ((err = cudaEventCreateWithFlags(ev, cudaEventDisableTiming)) != cudaSuccess) return bail(err, "event");
 
+  size_t traffic = 0;  // bytes of a step of all realisations
+  for (int m = 0; m < count; ++m) traffic += 2 * 19 * (size_t)E.L[m].Vp * store_bytes(members[0].storage);
   // every realisation as a single box in its slice (synchronises per member)
   e->inst.resize(count);
   e->hmem.resize(count);
@@ -511,12 +513,12 @@ int lbmd_ensemble_create(const lbmd_params *members, int32_t count, void *dev_wo
     const LbGeom &g = e->inst[m].geo;
     D.pop[0] = M.pop[0];
     D.pop[1] = M.pop[1];
-    D.lmask = g.lmask;
-    D.tile_near = g.tile_near;
     D.nx = g.nx;
     D.ny = g.ny;
     D.nz = g.nz;
-    D.ntx = g.ntx;
+    D.wall = g.wall;
+    D.fill_solid = fill_solid(members[m], traffic);
+    D.lmask = g.lmask;
     D.Vp = (int)g.Vp;
     D.inv_nx = 1.0f / (float)g.nx;
     D.omega = M.ph.omega;

@@ -29,28 +29,24 @@ namespace lbmd {
 template <int S, int FORCING, typename I, bool ODD, bool FLUCT>
 __device__ __forceinline__ void aa_node(const LbGeom &g, const LbPhys &ph,
                                         typename Store<S>::T *buf, int x, int y, int z,
-                                        bool near) {
+                                        uint32_t bb) {
   using St = Store<S>;
   const int nx = g.nx, ny = g.ny;
   const I self = ((I)z * ny + y) * nx + x;
-  const I Vp = (I)g.Vp;
-  uint32_t bb = 0u;  // link mask; constant zero away from solid nodes
-  if (near) {
-    bb = __ldg(&g.lmask[self]);
-    if (bb & 1u) return;  // solid node
-  }
+  const I st = pop_stride<S, I>((I)g.Vp);
+  if (bb & 1u) return;  // solid node
   float h[kQ];
   if (!ODD) {
 #pragma unroll
-    for (int p = 0; p < kQ; ++p) h[p] = St::load_plain(buf + (I)p * Vp + self);
+    for (int p = 0; p < kQ; ++p) h[p] = St::load_plain(buf + (I)p * st + pop_base<S, I>(self));
     collide19<FORCING, FLUCT>(h, ph, (uint32_t)self);
     // The store addresses are the load addresses permuted; hiding the base
     // behind an empty asm makes the compiler recompute them after the
     // collision instead of keeping 19 of them live across it (which spills).
-    typename Store<S>::T *out = buf + self;
+    typename Store<S>::T *out = buf + pop_base<S, I>(self);
     asm volatile("" : "+l"(out));
 #pragma unroll
-    for (int p = 0; p < kQ; ++p) St::store(out + (I)opp(p) * Vp, h[p]);
+    for (int p = 0; p < kQ; ++p) St::store(out + (I)opp(p) * st, h[p]);
     return;
   }
   const int xm = wrap_m1(x, nx), xp = wrap_p1(x, nx);
@@ -62,8 +58,8 @@ __device__ __forceinline__ void aa_node(const LbGeom &g, const LbPhys &ph,
     const int sx = cx(p) == 1 ? xm : (cx(p) == -1 ? xp : x);
     const int sy = cy(p) == 1 ? ym : (cy(p) == -1 ? yp : y);
     const int sz = cz(p) == 1 ? zm : (cz(p) == -1 ? zp : z);
-    const I sidx = (I)opp(p) * Vp + ((I)sz * ny + sy) * nx + sx;
-    const I bidx = (I)p * Vp + self;
+    const I sidx = (I)opp(p) * st + pop_base<S, I>(((I)sz * ny + sy) * nx + sx);
+    const I bidx = (I)p * st + pop_base<S, I>(self);
     h[p] = St::load_plain(buf + (((bb >> p) & 1u) ? bidx : sidx));
   }
   collide19<FORCING, FLUCT>(h, ph, (uint32_t)self);
@@ -83,8 +79,8 @@ __device__ __forceinline__ void aa_node(const LbGeom &g, const LbPhys &ph,
     const int tx = cx(p) == 1 ? oxp : (cx(p) == -1 ? oxm : ox);
     const int ty = cy(p) == 1 ? oyp : (cy(p) == -1 ? oym : oy);
     const int tz = cz(p) == 1 ? ozp : (cz(p) == -1 ? ozm : oz);
-    const I didx = (I)p * Vp + ((I)tz * ny + ty) * nx + tx;
-    const I bidx = (I)opp(p) * Vp + oself;
+    const I didx = (I)p * st + pop_base<S, I>(((I)tz * ny + ty) * nx + tx);
+    const I bidx = (I)opp(p) * st + pop_base<S, I>(oself);
     St::store(out + (((bb >> opp(p)) & 1u) ? bidx : didx), h[p]);
   }
 }
@@ -101,7 +97,9 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock, FLUCT ? 1 : (ODD ? 5 : 6))
   const int z = blockIdx.z;
   if (bump != nullptr && x == 0 && y == 0 && z == 0) bump->step += 1;
   if (x >= g.nx || y >= g.ny) return;
-  aa_node<S, FORCING, I, ODD, FLUCT>(g, ph, buf, x, y, z, tile_is_near(g, x, y, z));
+  uint32_t bb = 0u;  // link mask; zero away from solid nodes
+  if (beside_wall(g, x, y)) bb = __ldg(&g.lmask[((size_t)z * g.ny + y) * g.nx + x]);
+  aa_node<S, FORCING, I, ODD, FLUCT>(g, ph, buf, x, y, z, bb);
 }
 
 template <int S, typename I, bool FLUCT>

@@ -20,8 +20,7 @@ namespace lbmd {
 // not a multiple of 32).  With CPT = 3 (16-bit storage) a thread takes two
 // x-adjacent nodes instead, whose deviations share a 32-bit word (pair_node),
 // and a tile is 64 x ROWS consecutive nodes of one plane (every member's nx
-// is even, so a pair never straddles a row).  A warp takes the bounce-back checks if any of its
-// nodes needs them.  WARPS is the occupancy the register budget is sized for:
+// is even, so a pair never straddles a row).  WARPS is the occupancy the register budget is sized for:
 // 48 warps per SM (40 registers, a little spilling) or 32 (64 registers,
 // none); population offsets are 32-bit.
 template <int S, int FORCING, int ROWS, int WARPS, int CPT>
@@ -49,11 +48,13 @@ __global__ void __launch_bounds__(32 * ROWS, WARPS / ROWS)
     g.nx = d.nx;
     g.ny = d.ny;
     g.nz = d.nz;
-    g.ntx = d.ntx;
+    g.wall = d.wall;
+    g.fill_solid = d.fill_solid;
+    g.ntx = 0;
     g.V = 0;
     g.Vp = d.Vp;
     g.solid = nullptr;  // the link mask replaces the bitfield here
-    g.tile_near = d.tile_near;
+    g.tile_near = nullptr;
     g.lmask = d.lmask;
     LbPhys ph;
     ph.omega = d.omega;
@@ -81,16 +82,11 @@ __global__ void __launch_bounds__(32 * ROWS, WARPS / ROWS)
     T *dst = (T *)(cur ? d.pop[0] : d.pop[1]);
     if constexpr (CPT == 3) {
       using T2 = typename std::conditional<S == LBMD_STORE_F16, __half2, __nv_bfloat162>::type;
-      const bool near = __any_sync(0xffffffffu, active && tile_is_near(g, x, y, w.y));
-      if (active)
-        pair_node<T2, FORCING>(g, ph, (const uint32_t *)src, (uint32_t *)dst, x >> 1, y, w.y, near);
+      if (active) pair_node<T2, FORCING>(g, ph, (const uint32_t *)src, (uint32_t *)dst, x >> 1, y, w.y);
     } else if (CPT == 2 && w.w == 2) {
-      const bool near = __any_sync(0xffffffffu, active && (tile_is_near(g, x, y, w.y) ||
-                                                            tile_is_near(g, x, y, w.y + 1)));
-      if (active) stream_collide_node2<S, FORCING>(g, ph, src, dst, x, y, w.y, near);
+      if (active) stream_collide_node2<S, FORCING>(g, ph, src, dst, x, y, w.y);
     } else {
-      const bool near = __any_sync(0xffffffffu, active && tile_is_near(g, x, y, w.y));
-      if (active) stream_collide_node<S, FORCING, int>(g, ph, src, dst, x, y, w.y, near);
+      if (active) stream_collide_node<S, FORCING, int>(g, ph, src, dst, x, y, w.y);
     }
   }
 }

@@ -16,7 +16,7 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock)
   const int y = blockIdx.y * kRowsPerBlock + threadIdx.y;
   const int z = blockIdx.z;
   if (x >= g.nx || y >= g.ny) return;
-  stream_collide_node<S, FORCING, I, true>(g, ph, src, dst, x, y, z, tile_is_near(g, x, y, z));
+  stream_collide_node<S, FORCING, I, true>(g, ph, src, dst, x, y, z);
 }
 
 template <int S, typename I>

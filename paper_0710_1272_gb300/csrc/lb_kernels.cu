@@ -1,7 +1,8 @@
 // lb_kernels.cu -- D3Q19 BGK stream-collide (Eq. 5 with the Eq. 6 equilibrium
 // and the body-force source), population initialisation and field read-outs.
 //
-// Layout: structure of arrays, h[p][z][y][x] with population stride Vp, every
+// Layout: h[p][z][y][x] with population stride Vp (FP32), or blocks of 64
+// consecutive nodes with their 19 populations (16-bit storage, pop_base), every
 // entry the deviation h = f - w_p rho0 in the storage type.  One thread per
 // node; a warp covers 32 consecutive x of one (y, z) row so that every one of
 // the 19 loads and 19 stores of a warp is a contiguous 128-byte (fp32) or
@@ -23,7 +24,7 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock, 6)
   const int z = blockIdx.z;
   if (bump != nullptr && x == 0 && y == 0 && z == 0) bump->step += 1;
   if (x >= g.nx || y >= g.ny) return;
-  stream_collide_node<S, FORCING, I>(g, ph, src, dst, x, y, z, tile_is_near(g, x, y, z));
+  stream_collide_node<S, FORCING, I>(g, ph, src, dst, x, y, z);
 }
 
 // 16-bit storage: one thread per pair of x-adjacent nodes (pair_node).  A
@@ -39,7 +40,7 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock, FORCING == kForcingNone ? 
   const int z = blockIdx.z;
   if (bump != nullptr && xw == 0 && y == 0 && z == 0) bump->step += 1;
   if (xw >= (g.nx >> 1) || y >= g.ny) return;
-  pair_node<T2, FORCING>(g, ph, src, dst, xw, y, z, tile_is_near(g, 2 * xw, y, z));
+  pair_node<T2, FORCING>(g, ph, src, dst, xw, y, z);
 }
 
 template <typename T2>
@@ -175,10 +176,10 @@ __global__ void k_init(LbGeom g, float rho0, const float *rho, const float *u, f
   const int z = blockIdx.z;
   if (x >= g.nx || y >= g.ny) return;
   const size_t self = ((size_t)z * g.ny + y) * g.nx + x;
-  const size_t Vp = (size_t)g.Vp;
+  const size_t st = pop_stride<S, size_t>((size_t)g.Vp), at = pop_base<S, size_t>(self);
   if (solid_at(g.solid, g.ntx, g.ny, x, y, z)) {
 #pragma unroll
-    for (int q = 0; q < kQ; ++q) St::store(dst + q * Vp + self, 0.f);
+    for (int q = 0; q < kQ; ++q) St::store(dst + q * st + at, 0.f);
     return;
   }
   float r0, ux0, uy0, uz0;
@@ -196,7 +197,7 @@ __global__ void k_init(LbGeom g, float rho0, const float *rho, const float *u, f
     } else {
       v = feq_dev(opp(q), r0, rho0, ux0, uy0, uz0);
     }
-    St::store(dst + q * Vp + self, v);
+    St::store(dst + q * st + at, v);
   }
 }
 
@@ -233,14 +234,14 @@ __global__ void k_init_local(LbGeom g, float rho0, const float *rho, const float
   const int z = z0 + blockIdx.z;
   if (x >= g.nx || y >= g.ny) return;
   const size_t self = ((size_t)z * g.ny + y) * g.nx + x;
-  const size_t Vp = (size_t)g.Vp;
+  const size_t st = pop_stride<S, size_t>((size_t)g.Vp), at = pop_base<S, size_t>(self);
   float r = rho0, ux = 0.f, uy = 0.f, uz = 0.f;
   const bool solid = solid_at(g.solid, g.ntx, g.ny, x, y, z);
   if (!solid)
     fields_at(x, y, ((size_t)blockIdx.z * g.ny + y) * g.nx + x, ustride, g, rho0, rho, u, tg_amp, r,
               ux, uy, uz);
 #pragma unroll
-  for (int q = 0; q < kQ; ++q) St::store(dst + q * Vp + self, solid ? 0.f : feq_dev(q, r, rho0, ux, uy, uz));
+  for (int q = 0; q < kQ; ++q) St::store(dst + q * st + at, solid ? 0.f : feq_dev(q, r, rho0, ux, uy, uz));
 }
 
 cudaError_t launch_init_local(int storage, const LbGeom &g, float rho0, const float *rho,

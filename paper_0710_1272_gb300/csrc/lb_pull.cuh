@@ -26,17 +26,52 @@ __device__ __forceinline__ void pull19_mask(const LbGeom &g,
   const int ym = wrap_m1(y, ny), yp = wrap_p1(y, ny);
   const int zm = wrap_m1(z, nz), zp = wrap_p1(z, nz);
   const I self = ((I)z * ny + y) * nx + x;
-  const I Vp = (I)g.Vp;
+  const I st = pop_stride<S, I>((I)g.Vp);
 #pragma unroll
   for (int p = 0; p < kQ; ++p) {
     // source node x - c_p
     const int sx = cx(p) == 1 ? xm : (cx(p) == -1 ? xp : x);
     const int sy = cy(p) == 1 ? ym : (cy(p) == -1 ? yp : y);
     const int sz = cz(p) == 1 ? zm : (cz(p) == -1 ? zp : z);
-    const I sidx = (I)(SWAP ? opp(p) : p) * Vp + ((I)sz * ny + sy) * nx + sx;
-    const I bidx = (I)(SWAP ? p : opp(p)) * Vp + self;
+    const I sidx = (I)(SWAP ? opp(p) : p) * st + pop_base<S, I>(((I)sz * ny + sy) * nx + sx);
+    const I bidx = (I)(SWAP ? p : opp(p)) * st + pop_base<S, I>(self);
     h[p] = St::load(src + (((bb >> p) & 1u) ? bidx : sidx));
   }
+}
+
+// Whether node (x, y) or, with W > 1, one of the W nodes from x on may have a
+// solid node within one node: it is in or beside a wall layer or a solid row.
+// (In the pore's opening such a node's link mask is zero.)
+//
+// Computed, so that the few nodes beside a wall read their mask word while the
+// populations are on their way.  The stream-collides used to read a flag per
+// 32-node tile and, in tiles next to a solid node, the mask before they could
+// load a population (a quarter of the tiles of the 256x128x128 box with one
+// wall layer, each waiting for two more memory latencies: FP32 100.4 us a step
+// against 94.6 without the wall).  The mask itself is not computed: the bits of
+// 18 directions cost the 16-bit kernel, bound by instructions, more than the
+// load (70.7 us against 61.5).
+template <int W = 1>
+__device__ __forceinline__ bool beside_wall(const LbGeom &g, int x, int y) {
+  const WallGeom &w = g.wall;
+  int dx = x - w.wall_x;  // layers after the first one, around the box
+  if (dx < 0) dx += g.nx;
+  return (w.wall_x >= 0 && (dx <= w.wall_t || dx >= g.nx - W)) ||
+         (w.y_walls && (y <= 1 || y >= g.ny - 2));
+}
+
+// The bounce-back of pull19_mask after the fact: h holds the values of every
+// source x - c_p, solid or not; those of the solid ones (bits of `bb`) are
+// replaced by the node's own reversed populations.
+template <int S, typename I = size_t>
+__device__ __forceinline__ void bounce19(const LbGeom &g, const typename Store<S>::T *__restrict__ src,
+                                         I self, uint32_t bb, float h[kQ]) {
+  using St = Store<S>;
+  const I st = pop_stride<S, I>((I)g.Vp);
+  const typename St::T *own = src + pop_base<S, I>(self);
+#pragma unroll
+  for (int p = 1; p < kQ; ++p)
+    if ((bb >> p) & 1u) h[p] = St::load(own + (I)opp(p) * st);
 }
 
 __device__ __forceinline__ bool tile_is_near(const LbGeom &g, int x, int y, int z) {
@@ -54,7 +89,7 @@ __device__ __forceinline__ void fetch19(const LbGeom &g, const typename Store<S>
   const I self = ((I)z * g.ny + y) * g.nx + x;
   if (mode == kPopAALocal) {
 #pragma unroll
-    for (int p = 0; p < kQ; ++p) h[p] = St::load(src + (I)p * (I)g.Vp + self);
+    for (int p = 0; p < kQ; ++p) h[p] = St::load(src + (I)p * pop_stride<S, I>((I)g.Vp) + pop_base<S, I>(self));
     return;
   }
   const uint32_t bb = tile_is_near(g, x, y, z) ? __ldg(&g.lmask[self]) : 0u;

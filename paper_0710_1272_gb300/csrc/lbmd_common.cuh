@@ -61,6 +61,24 @@ template <> struct Store<LBMD_STORE_BF16> {
   static __device__ __forceinline__ void add(T *p, float v) { atomicAdd(p, __float2bfloat16_rn(v)); }
 };
 
+// Where population p of node n (z, y, x row-major) is held: at
+// pop_base(n) + p pop_stride.
+//   FP32: structure of arrays, stride Vp.
+//   16-bit: blocks of 64 consecutive nodes, a block holding its 19 populations
+//   one after the other (128 bytes each).  The 19 populations a kernel stores
+//   per node, and those it loads from one node, then differ by constant
+//   offsets: one address instead of nineteen.  The 16-bit stream-collide is
+//   bound by instructions, not by HBM; with a stride of Vp two fifths of
+//   them were address arithmetic.
+constexpr int kBlockNodes = 64;
+template <int S, typename I> __host__ __device__ __forceinline__ I pop_base(I n) {
+  if (S == LBMD_STORE_F32) return n;
+  return n + (n >> 6) * (I)((kQ - 1) * kBlockNodes);  // 2^6 nodes a block
+}
+template <int S, typename I> __host__ __device__ __forceinline__ I pop_stride(I Vp) {
+  return S == LBMD_STORE_F32 ? Vp : (I)kBlockNodes;
+}
+
 // ---------------------------------------------------------------------------
 // Geometry helpers
 // ---------------------------------------------------------------------------

@@ -377,6 +377,9 @@ cudaError_t init_instance(const lbmd_params &p, const Layout &L, char *ws, cudaS
   g.ntx = L.ntx;
   g.V = (long long)p.nx * p.ny * p.nz;
   g.Vp = L.Vp;
+  g.wall = WallGeom{p.wall_x, p.wall_thickness, p.wall_x >= 0 ? p.pore_d : 0, 0, 0, p.y_walls};
+  if (p.wall_x >= 0) pore_origin(p, g.wall.pore_y0, g.wall.pore_z0);
+  g.fill_solid = fill_solid(p, 2 * 19 * (size_t)L.Vp * store_bytes(p.storage));
   g.solid = (const uint32_t *)(ws + L.solid);
   g.tile_near = (const uint8_t *)(ws + L.tile);
   g.lmask = (const uint32_t *)(ws + L.lmask);

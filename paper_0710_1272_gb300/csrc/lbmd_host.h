@@ -41,6 +41,11 @@ Layout make_layout(const lbmd_params &p, bool single_box);
 size_t stage_floats_for(const lbmd_params &p);
 long long chunk_cells_for(const lbmd_params &p);
 
+// LbGeom::fill_solid of a box stepped with `traffic` bytes of populations per
+// step: beyond the 129 MB L2, and a wall of up to a sector's eight floats.
+inline int fill_solid(const lbmd_params &p, size_t traffic) {
+  return p.wall_x >= 0 && p.wall_thickness <= 8 && traffic > (size_t)129 << 20;
+}
 int validate(const lbmd_params *p);
 bool params_have_bonds(const lbmd_params &p);
 

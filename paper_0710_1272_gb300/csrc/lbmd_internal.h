@@ -42,9 +42,19 @@ struct DevDiag {
 constexpr int kMaxPairs = 48;
 constexpr int kMaxWall = 128;
 
+// Sec. III geometry: wall layers wall_x .. wall_x + wall_t - 1 (wall_x < 0: no
+// wall) minus the pore_d x pore_d pore, and the rows y = 0 and y = ny - 1 with
+// y_walls -- the rule the solid bitfield and the link masks are built from.
+struct WallGeom {
+  int wall_x, wall_t, pore_d, pore_y0, pore_z0, y_walls;
+};
+
 // Lattice geometry as the kernels see it.
 struct LbGeom {
   int nx, ny, nz;
+  WallGeom wall;
+  int fill_solid;               // stream-collides write zeros to solid nodes: a thin
+                                // wall in a box beyond the L2 cache
   int ntx;                      // x-tiles of 32 nodes = words per bitfield row
   long long V;                  // nx * ny * nz
   long long Vp;                 // population stride (V rounded up to 64)
@@ -142,12 +152,13 @@ struct EnsMember {
 };
 
 // What the ensemble stream-collide needs of one realisation, 16-byte aligned
-// so that a block reads it with six vector loads.
+// so that a block reads it with seven vector loads.
 struct __align__(16) EnsLb {
   void *pop[2];                 // post-collision populations, swapped every step
   const uint32_t *lmask;        // as LbGeom::lmask
-  const uint8_t *tile_near;     // as LbGeom::tile_near
-  int nx, ny, nz, ntx;
+  int nx, ny, nz;
+  WallGeom wall;
+  int fill_solid;               // as LbGeom's, for the realisations together
   int Vp;                       // population stride (19 Vp < 2^31)
   float inv_nx;                 // 1 / nx, for the row of a node in its plane
   float omega, rho0;

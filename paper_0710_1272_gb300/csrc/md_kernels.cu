@@ -1380,7 +1380,7 @@ __global__ void __launch_bounds__(256)
     if (node < 0) return;  // not an owner
     F = F3{v.x, v.y, v.z};
   }
-  const size_t Vp = (size_t)g.Vp;
+  const size_t st = pop_stride<S, size_t>((size_t)g.Vp), own = pop_base<S, size_t>((size_t)node);
   uint32_t bb = 0u;
   int x = 0, y = 0, z = 0;
   if (mode == kPopAALocal) {
@@ -1396,9 +1396,9 @@ __global__ void __launch_bounds__(256)
     if (mode == kPopAALocal) {
       const size_t t = ((size_t)wrapi(z + cz(p), g.nz) * g.ny + wrapi(y + cy(p), g.ny)) * g.nx +
                        wrapi(x + cx(p), g.nx);
-      at[p] = ((bb >> opp(p)) & 1u) ? (size_t)opp(p) * Vp + node : (size_t)p * Vp + t;
+      at[p] = ((bb >> opp(p)) & 1u) ? (size_t)opp(p) * st + own : (size_t)p * st + pop_base<S, size_t>(t);
     } else {
-      at[p] = (size_t)(mode == kPopAASwap ? opp(p) : p) * Vp + node;
+      at[p] = (size_t)(mode == kPopAASwap ? opp(p) : p) * st + own;
     }
   }
   if (S == LBMD_STORE_F32) {
@@ -1469,19 +1469,19 @@ __global__ void __launch_bounds__(256)
     const int node = a.sp_node[e2];
     if (node >= 0 && a.owner[node] == e2) {  // the owner converts its node's sum
       const F3 F = spread_take(a, node, e2);
-      typename St::T *dst = (typename St::T *)mem[mi.x].pop[cur ^ 1];
-      const size_t Vp = (size_t)a.geo.Vp;
+      const size_t st = pop_stride<S, size_t>((size_t)a.geo.Vp);
+      typename St::T *dst = (typename St::T *)mem[mi.x].pop[cur ^ 1] + pop_base<S, size_t>((size_t)node);
       if (S == LBMD_STORE_F32) {
 #pragma unroll
         for (int p = 1; p < kQ; ++p)
-          St::add(dst + (size_t)p * Vp + node, 3.0f * wq(p) * (cx(p) * F.x + cy(p) * F.y + cz(p) * F.z));
+          St::add(dst + (size_t)p * st, 3.0f * wq(p) * (cx(p) * F.x + cy(p) * F.y + cz(p) * F.z));
       } else {
         float hv[kQ];
 #pragma unroll
-        for (int p = 1; p < kQ; ++p) hv[p] = St::load_plain(dst + (size_t)p * Vp + node);
+        for (int p = 1; p < kQ; ++p) hv[p] = St::load_plain(dst + (size_t)p * st);
 #pragma unroll
         for (int p = 1; p < kQ; ++p)
-          St::store(dst + (size_t)p * Vp + node,
+          St::store(dst + (size_t)p * st,
                     hv[p] + 3.0f * wq(p) * (cx(p) * F.x + cy(p) * F.y + cz(p) * F.z));
       }
     }
