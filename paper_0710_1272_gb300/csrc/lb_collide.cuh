@@ -26,46 +26,6 @@ __host__ __device__ constexpr int mode_row(int k, int p) {
        : k == 17 ? (2 * c2 - 3) * (3 * x * x - c2) : (2 * c2 - 3) * (y * y - z * z);
 }
 
-// Thermal source F_p of Eq. 5 (fluctuating LB, Adhikari et al. 2005, in the
-// mode form of Duenweg, Schiller and Ladd 2007) at node `node`, density rho:
-//   xi_p = w_p sum_{k=4}^{18} e_kp a_k sqrt(rho) r_k,
-//   a_k = sqrt((kT / c_s^2) (1 - (1 - omega)^2) / b_k)   (ph.fl_amp[k - 4]),
-// with fifteen standard normals r_k from Box-Muller on four Philox blocks,
-// counter (node, step lo, step hi, block | 2 << 8), key (seed lo, seed hi).
-// The noise touches only non-conserved modes: mass and momentum are exact.
-__device__ __forceinline__ void thermal_source(const LbPhys &ph, uint32_t node, float rho,
-                                               float xi[kQ]) {
-  const long long step = *ph.step;
-  float r[16];
-#pragma unroll
-  for (uint32_t j = 0; j < 4; ++j) {
-    const U4 c{node, (uint32_t)(unsigned long long)step, (uint32_t)((unsigned long long)step >> 32),
-               j | (2u << 8)};
-    const U4 x = philox4x32_10(c, (uint32_t)ph.seed, (uint32_t)(ph.seed >> 32));
-    const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const float rad = sqrtf(-2.0f * logf(uniform23(xs[2 * h])));
-      float sn, cs;
-      sincospif(2.0f * uniform23(xs[2 * h + 1]), &sn, &cs);
-      r[4 * j + 2 * h] = rad * cs;
-      r[4 * j + 2 * h + 1] = rad * sn;
-    }
-  }
-  const float sr = sqrtf(rho);
-  float t[15];
-#pragma unroll
-  for (int k = 0; k < 15; ++k) t[k] = ph.fl_amp[k] * sr * r[k];
-#pragma unroll
-  for (int p = 0; p < kQ; ++p) {
-    float acc = 0.f;
-#pragma unroll
-    for (int k = 4; k < kQ; ++k)
-      if (mode_row(k, p) != 0) acc = fmaf((float)mode_row(k, p), t[k - 4], acc);
-    xi[p] = wq(p) * acc;
-  }
-}
-
 // Arithmetic of the collision, on one node (Ops1: float) or on two nodes at
 // once (Ops2: float2, the paired FP32 instructions of sm_100 and later).  A
 // paired operation is two independent correctly rounded operations, so both
@@ -75,6 +35,9 @@ __device__ __forceinline__ void thermal_source(const LbPhys &ph, uint32_t node, 
 // identically.
 struct Ops1 {
   using V = float;
+  static constexpr int N = 1;  // nodes
+  static __device__ __forceinline__ V pack(const float *v) { return v[0]; }
+  static __device__ __forceinline__ void unpack(V v, float *o) { o[0] = v; }
   static __device__ __forceinline__ V add(V a, V b) { return __fadd_rn(a, b); }
   static __device__ __forceinline__ V sub(V a, V b) { return __fadd_rn(a, -b); }
   static __device__ __forceinline__ V mul(V a, V b) { return __fmul_rn(a, b); }
@@ -86,6 +49,12 @@ struct Ops1 {
 };
 struct Ops2 {
   using V = float2;
+  static constexpr int N = 2;
+  static __device__ __forceinline__ V pack(const float *v) { return make_float2(v[0], v[1]); }
+  static __device__ __forceinline__ void unpack(V v, float *o) {
+    o[0] = v.x;
+    o[1] = v.y;
+  }
   static __device__ __forceinline__ V neg(V a) { return make_float2(-a.x, -a.y); }
   static __device__ __forceinline__ V add(V a, V b) { return __fadd2_rn(a, b); }
   static __device__ __forceinline__ V sub(V a, V b) { return __fadd2_rn(a, neg(b)); }
@@ -95,6 +64,165 @@ struct Ops2 {
   static __device__ __forceinline__ V rcp(V a) { return make_float2(__frcp_rn(a.x), __frcp_rn(a.y)); }
   static __device__ __forceinline__ bool finite(V a) { return isfinite(a.x) && isfinite(a.y); }
 };
+
+// Uniforms in (0, 1) as uniform23 gives them: 1 + k 2^-23 by its bits, less
+// 1 - 2^-24, both exact.
+template <class O>
+__device__ __forceinline__ typename O::V uniform23_t(const uint32_t *x) {
+  float f[O::N];
+#pragma unroll
+  for (int n = 0; n < O::N; ++n) f[n] = __uint_as_float((x[n] >> 9) | 0x3f800000u);
+  return O::add(O::pack(f), O::splat(-0.99999994f));
+}
+
+// Two standard normals per node by Box and Muller, sqrt(-2 ln u1) times the
+// cosine and sine of 2 pi u2, on operations that take one or two nodes at once
+// (the library functions take one, and were two fifths of the kernel).
+//   ln u = e ln 2 + ln(1 + f), 2^e (1 + f) = u, sqrt(1/2) <= 1 + f < sqrt(2):
+//     f - f^2/2 + f^3 Q(f), Q the minimax polynomial of degree 7 (6e-9);
+//   the angle is reduced to +-pi/4 exactly (2 u2 less a multiple of 1/2), sine
+//     and cosine there by minimax polynomials in r^2 (3e-9, 6e-11);
+//   the root from the hardware's reciprocal root and one Newton step.
+// Against 64 bits over all 2^23 values of u1: rms 4.39e-8 relative for the normals,
+// largest error 1.7e-7 of the radius (library functions 4.38e-8, 1.7e-7).
+template <class O>
+__device__ __forceinline__ void box_muller_t(typename O::V u1, typename O::V u2, typename O::V &n1,
+                                             typename O::V &n2) {
+  using V = typename O::V;
+  float u[O::N], m[O::N], ef[O::N];
+  O::unpack(u1, u);
+#pragma unroll
+  for (int n = 0; n < O::N; ++n) {
+    // k >> 23 = 64 + e: less sqrt(1/2)'s bits
+    const uint32_t i = __float_as_uint(u[n]) + 0x20000000u, k = i - 0x3f3504f3u;
+    m[n] = __uint_as_float(i - (k & 0xff800000u));
+    ef[n] = __uint_as_float(0x4b400000u | (k >> 23));  // 1.5 2^23 + 64 + e
+  }
+  const V e = O::add(O::pack(ef), O::splat(-12582976.0f));
+  const V f = O::add(O::pack(m), O::splat(-1.0f));
+  V q = O::splat(-0.07634429633617401f);
+  q = O::fma(q, f, O::splat(0.12761549651622772f));
+  q = O::fma(q, f, O::splat(-0.131601944565773f));
+  q = O::fma(q, f, O::splat(0.14201761782169342f));
+  q = O::fma(q, f, O::splat(-0.16623356938362122f));
+  q = O::fma(q, f, O::splat(0.20001226663589478f));
+  q = O::fma(q, f, O::splat(-0.250008225440979f));
+  q = O::fma(q, f, O::splat(0.3333333134651184f));
+  q = O::mul(f, O::fma(q, f, O::splat(-0.5f)));  // ln(1 + f) = f + f (f (Q f - 1/2))
+  q = O::fma(e, O::splat(-2.1219444e-4f), O::fma(f, q, f));  // ln 2 = 0.693359375 - 2.12e-4
+  const V L = O::mul(O::splat(-2.0f), O::fma(e, O::splat(0.693359375f), q));
+  float l[O::N];
+  O::unpack(L, l);
+#pragma unroll
+  for (int n = 0; n < O::N; ++n) asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(l[n]) : "f"(l[n]));
+  const V y = O::pack(l), s0 = O::mul(L, y);
+  const V rad = O::fma(O::mul(O::splat(0.5f), y), O::fma(O::neg(s0), s0, L), s0);
+  const V t = O::fma(u2, O::splat(4.0f), O::splat(12582912.0f));  // quadrant in its low bits
+  const V r = O::fma(O::add(t, O::splat(-12582912.0f)), O::splat(-0.5f), O::add(u2, u2));
+  const V r2 = O::mul(r, r);
+  V s = O::fma(r2, O::splat(-0.5890786647796631f), O::splat(2.549767255783081f));
+  s = O::fma(r2, s, O::splat(-5.167707920074463f));
+  // the leading coefficient in two parts, the large one in the last, once rounded operation
+  s = O::fma(O::splat(3.1415927410125732f), r, O::mul(r, O::fma(r2, s, O::splat(-9.707896709e-08f))));
+  V c = O::fma(r2, O::splat(0.23142953217029572f), O::splat(-1.3350584506988525f));
+  c = O::fma(r2, c, O::splat(4.0587077140808105f));
+  c = O::fma(r2, c, O::splat(-4.934802055358887f));
+  c = O::fma(r2, c, O::splat(1.0f));
+  float k[O::N], sn[O::N], cs[O::N];
+  O::unpack(t, k);
+  O::unpack(s, sn);
+  O::unpack(c, cs);
+#pragma unroll
+  for (int n = 0; n < O::N; ++n) {
+    const int a = __float_as_int(k[n]);
+    const float v = (a & 1) ? cs[n] : sn[n], w = (a & 1) ? sn[n] : cs[n];
+    sn[n] = __int_as_float(__float_as_int(v) ^ ((a & 2) << 30));
+    cs[n] = __int_as_float(__float_as_int(w) ^ (((a + 1) & 2) << 30));
+  }
+  n1 = O::mul(rad, O::pack(cs));
+  n2 = O::mul(rad, O::pack(sn));
+}
+
+// Thermal source F_p of Eq. 5 (fluctuating LB, Adhikari et al. 2005, in the
+// mode form of Duenweg, Schiller and Ladd 2007) at the nodes `node`, density
+// rho:
+//   xi_p = w_p sum_{k=4}^{18} e_kp a_k sqrt(rho) r_k,
+//   a_k = sqrt((kT / c_s^2) (1 - (1 - omega)^2) / b_k)   (ph.fl_amp[k - 4]),
+// with fifteen standard normals r_k from Box-Muller on four Philox blocks,
+// counter (node, step lo, step hi, block | 2 << 8), key (seed lo, seed hi).
+// The noise touches only non-conserved modes: mass and momentum are exact.
+// Returns v_p = xi_p / w_p.  The sum over modes (mode_row) is taken by the parity of the modes and of the
+// directions: 55 additions in place of 238 products.
+template <class O>
+__device__ __forceinline__ void thermal_normals_t(const LbPhys &ph, const uint32_t *node,
+                                                  typename O::V r[16]) {
+  const long long step = *ph.step;
+#pragma unroll
+  for (uint32_t j = 0; j < 4; ++j) {
+    uint32_t xs[4][O::N];
+#pragma unroll
+    for (int n = 0; n < O::N; ++n) {
+      const U4 c{node[n], (uint32_t)(unsigned long long)step,
+                 (uint32_t)((unsigned long long)step >> 32), j | (2u << 8)};
+      const U4 x = philox4x32_10(c, (uint32_t)ph.seed, (uint32_t)(ph.seed >> 32));
+      xs[0][n] = x.x;
+      xs[1][n] = x.y;
+      xs[2][n] = x.z;
+      xs[3][n] = x.w;
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      box_muller_t<O>(uniform23_t<O>(xs[2 * h]), uniform23_t<O>(xs[2 * h + 1]), r[4 * j + 2 * h],
+                      r[4 * j + 2 * h + 1]);
+  }
+}
+template <class O>
+__device__ __forceinline__ void thermal_source_t(const LbPhys &ph, const typename O::V r[16],
+                                                 typename O::V rho, typename O::V v[kQ]) {
+  using V = typename O::V;
+  float rr[O::N];
+  O::unpack(rho, rr);
+#pragma unroll
+  for (int n = 0; n < O::N; ++n) rr[n] = sqrtf(rr[n]);
+  const V sr = O::pack(rr);
+  // Products that meet a sum are written as fused operations: paired products
+  // (unlike __fmul_rn) are contracted with a sum that follows, and one and two
+  // nodes at a time must round alike.
+  const auto a = [&](int k) { return O::mul(O::splat(ph.fl_amp[k - 4]), sr); };
+  const auto n = [&](int k) { return r[k - 4]; };
+  const V two = O::splat(2.0f);
+  // directions +-: even part of the modes, plus or minus the odd part
+  const auto pair = [&](int p, V even, V odd) {
+    v[p] = O::add(even, odd);
+    v[p + 1] = O::sub(even, odd);
+  };
+  const auto axis = [&](int p, V even, int k) {
+    const V c = O::mul(O::splat(-2.0f), a(k));
+    v[p] = O::fma(c, n(k), even);
+    v[p + 1] = O::fma(O::neg(c), n(k), even);
+  };
+  const V t16 = O::mul(a(16), n(16)), t17 = O::mul(a(17), n(17)), t18 = O::mul(a(18), n(18));
+  const V m16 = O::mul(O::splat(-2.0f), t16);
+  v[0] = O::fma(O::neg(a(4)), n(4), t16);
+  const V a5 = O::fma(a(5), n(5), O::neg(t17)), b5 = O::fma(a(5), n(5), t17);
+  const V a6 = O::fma(a(6), n(6), O::neg(t18)), b6 = O::fma(a(6), n(6), t18);
+  const V b0 = O::fma(a(4), n(4), t16);
+  axis(1, O::fma(two, a5, m16), 10);
+  axis(3, O::add(O::sub(a6, a5), m16), 11);
+  axis(5, O::sub(m16, O::add(a5, a6)), 12);
+  const V t13 = O::mul(a(13), n(13)), t14 = O::mul(a(14), n(14)), t15 = O::mul(a(15), n(15));
+  const V xp = O::fma(a(10), n(10), t13), xm = O::fma(a(10), n(10), O::neg(t13));
+  const V yp = O::fma(a(11), n(11), t14), ym = O::fma(a(11), n(11), O::neg(t14));
+  const V zp = O::fma(a(12), n(12), t15), zm = O::fma(a(12), n(12), O::neg(t15));
+  const V bxy = O::add(b0, O::add(b5, b6)), bxz = O::add(b0, O::sub(b5, b6)),
+          byz = O::fma(O::splat(-2.0f), b5, b0);
+  pair(7, O::fma(a(7), n(7), bxy), O::add(xp, ym));
+  pair(9, O::fma(O::neg(a(7)), n(7), bxy), O::sub(xp, ym));
+  pair(11, O::fma(a(9), n(9), bxz), O::add(xm, zp));
+  pair(13, O::fma(O::neg(a(9)), n(9), bxz), O::sub(xm, zp));
+  pair(15, O::fma(a(8), n(8), byz), O::add(yp, zm));
+  pair(17, O::fma(O::neg(a(8)), n(8), byz), O::sub(yp, zm));
+}
 
 // rho - rho0 and j = sum_p h_p c_p, each a sum in the population order, the
 // momentum components as signed sums (no products with c_p).
@@ -131,15 +259,16 @@ __device__ __forceinline__ typename O::V cdotu_t(int p, typename O::V ux, typena
 //   paper forcing: S_p = 3 w_p c_p . g;
 //   Guo forcing:   u = (j + g/2)/rho, S_p = (1 - omega/2) w_p [3 (c - u) + 9 (c.u) c] . g;
 //   kForcingNone (g = 0): u = j/rho, S_p = 0;
-//   FLUCT (Ops1 only): plus the thermal source F_p of Eq. 5 (thermal_source).
+//   FLUCT: plus the thermal source F_p of Eq. 5 (thermal_source_t) of the
+//   node's (nodes') fifteen normals.
 // Opposite directions p, opp(p) = p + 1 (odd p) share c.u up to the sign, so
 // heq splits into the even part w_p [(rho - rho0) - 3/2 rho u.u + 9/2 rho (c.u)^2]
 // and the odd part +-3 w_p rho c.u, computed once per pair.  A node whose
 // density is not finite (a population is not) sets *ph.nonfinite.
 template <class O, int FORCING, bool FLUCT = false>
-__device__ __forceinline__ void collide_t(typename O::V h[kQ], const LbPhys &ph, uint32_t node = 0) {
+__device__ __forceinline__ void collide_t(typename O::V h[kQ], const LbPhys &ph,
+                                          const typename O::V *normals = nullptr) {
   using V = typename O::V;
-  static_assert(!FLUCT || sizeof(V) == sizeof(float), "thermal source: one node per call");
   V drho, jx, jy, jz;
   moments_t<O>(h, drho, jx, jy, jz);
   const V rho = O::add(O::splat(ph.rho0), drho);
@@ -176,10 +305,10 @@ __device__ __forceinline__ void collide_t(typename O::V h[kQ], const LbPhys &ph,
     if (FORCING == LBMD_FORCING_PAPER) return O::add(v, O::splat(__fmul_rn(3.0f * wq(p), cg)));
     return v;
   };
-  float xi[kQ];
-  if constexpr (FLUCT) thermal_source(ph, node, rho, xi);
+  V xi[kQ];  // F_p / w_p
+  if constexpr (FLUCT) thermal_source_t<O>(ph, normals, rho, xi);
   h[0] = add_source(0, O::splat(0.f), O::fma(O::splat(__fmul_rn(om, wq(0))), A, O::mul(vom1, h[0])));
-  if constexpr (FLUCT) h[0] = O::add(h[0], xi[0]);
+  if constexpr (FLUCT) h[0] = O::fma(O::splat(wq(0)), xi[0], h[0]);
 #pragma unroll
   for (int p = 1; p < kQ; p += 2) {
     const V cu = cdotu_t<O>(p, ux, uy, uz);  // c_opp(p) . u = -cu
@@ -188,15 +317,17 @@ __device__ __forceinline__ void collide_t(typename O::V h[kQ], const LbPhys &ph,
     h[p] = add_source(p, cu, O::fma(ow, O::fma(r3, cu, even), O::mul(vom1, h[p])));
     h[p + 1] = add_source(p + 1, O::neg(cu), O::fma(ow, O::fma(O::neg(r3), cu, even), O::mul(vom1, h[p + 1])));
     if constexpr (FLUCT) {
-      h[p] = O::add(h[p], xi[p]);
-      h[p + 1] = O::add(h[p + 1], xi[p + 1]);
+      h[p] = O::fma(O::splat(wq(p)), xi[p], h[p]);
+      h[p + 1] = O::fma(O::splat(wq(p)), xi[p + 1], h[p + 1]);
     }
   }
 }
 
 template <int FORCING, bool FLUCT = false>
 __device__ __forceinline__ void collide19(float h[kQ], const LbPhys &ph, uint32_t node = 0) {
-  collide_t<Ops1, FORCING, FLUCT>(h, ph, node);
+  float r[16];
+  if constexpr (FLUCT) thermal_normals_t<Ops1>(ph, &node, r);
+  collide_t<Ops1, FORCING, FLUCT>(h, ph, r);
 }
 
 __device__ __forceinline__ void zero19(float h[kQ]) {
@@ -214,7 +345,7 @@ __device__ __forceinline__ bool solid_is_left_out(const LbGeom &g, int y) {
 }
 
 // Stream and collide node (x, y, z) of one box: pull, Eq. 5 collision, store.
-template <int S, int FORCING, typename I, bool FLUCT = false>
+template <int S, int FORCING, typename I>
 __device__ __forceinline__ void stream_collide_node(const LbGeom &g, const LbPhys &ph,
                                                     const typename Store<S>::T *__restrict__ src,
                                                     typename Store<S>::T *__restrict__ dst, int x,
@@ -233,7 +364,7 @@ __device__ __forceinline__ void stream_collide_node(const LbGeom &g, const LbPhy
   } else {
     pull19_mask<S, I>(g, src, x, y, z, 0u, h);  // constant mask: no selects
   }
-  collide19<FORCING, FLUCT>(h, ph, (uint32_t)self);
+  collide19<FORCING>(h, ph);
   if (bb & 1u) zero19(h);
   const I st = pop_stride<S, I>((I)g.Vp), at = pop_base<S, I>(self);
 #pragma unroll

@@ -8,23 +8,64 @@
 
 namespace lbmd {
 
+// Two nodes per thread, on consecutive z-planes, for the paired FP32
+// instructions: the noise is bound by instructions (~1300 per node with the
+// library's logarithm, sine and root one node at a time, 780 now; two fifths
+// of the FMA pipe's time are Philox products).  The normals are drawn before
+// the 38 loads are issued, so that both fit 96 registers: five blocks of 128
+// threads.  128^3, FP32: 92 us a step before, 71 now; 74 with six blocks (80
+// registers, spills), 77 with the loads first and 16 warps per SM.  An odd last
+// plane is taken alone.
+constexpr int kFluctRows = 4;
 template <int S, int FORCING, typename I>
-__global__ void __launch_bounds__(32 * kRowsPerBlock)
+__global__ void __launch_bounds__(32 * kFluctRows, 5)
     k_stream_collide_fluct(LbGeom g, LbPhys ph, const typename Store<S>::T *__restrict__ src,
                            typename Store<S>::T *__restrict__ dst) {
+  using St = Store<S>;
   const int x = blockIdx.x * 32 + threadIdx.x;
-  const int y = blockIdx.y * kRowsPerBlock + threadIdx.y;
-  const int z = blockIdx.z;
+  const int y = blockIdx.y * kFluctRows + threadIdx.y;
+  const int za = 2 * blockIdx.z, zb = min(za + 1, g.nz - 1);
   if (x >= g.nx || y >= g.ny) return;
-  stream_collide_node<S, FORCING, I, true>(g, ph, src, dst, x, y, z);
+  const I na = ((I)za * g.ny + y) * g.nx + x, nb = ((I)zb * g.ny + y) * g.nx + x;
+  uint32_t ma = 0u, mb = 0u;
+  if (beside_wall(g, x, y)) {
+    ma = __ldg(&g.lmask[na]);
+    mb = __ldg(&g.lmask[nb]);
+  }
+  if (ma & mb & 1u) return;
+  const uint32_t node[2] = {(uint32_t)na, (uint32_t)nb};
+  float2 r[16];
+  thermal_normals_t<Ops2>(ph, node, r);
+  float ha[kQ], hb[kQ];
+  pull19_mask<S, I>(g, src, x, y, za, 0u, ha);
+  pull19_mask<S, I>(g, src, x, y, zb, 0u, hb);
+  if (ma) bounce19<S, I>(g, src, na, ma, ha);
+  if (mb) bounce19<S, I>(g, src, nb, mb, hb);
+  if (ma & 1u) zero19(ha);  // harmless inputs: not written
+  if (mb & 1u) zero19(hb);
+  float2 h[kQ];
+#pragma unroll
+  for (int p = 0; p < kQ; ++p) h[p] = make_float2(ha[p], hb[p]);
+  collide_t<Ops2, FORCING, true>(h, ph, r);
+  const I st = pop_stride<S, I>((I)g.Vp);
+  if (!(ma & 1u)) {
+    typename St::T *out = dst + pop_base<S, I>(na);
+#pragma unroll
+    for (int p = 0; p < kQ; ++p) St::store(out + (I)p * st, h[p].x);
+  }
+  if (zb != za && !(mb & 1u)) {
+    typename St::T *out = dst + pop_base<S, I>(nb);
+#pragma unroll
+    for (int p = 0; p < kQ; ++p) St::store(out + (I)p * st, h[p].y);
+  }
 }
 
 template <int S, typename I>
 static cudaError_t fluct_launch(const LbGeom &g, const LbPhys &ph, const void *src, void *dst,
                                 cudaStream_t s) {
   using T = typename Store<S>::T;
-  dim3 block(32, kRowsPerBlock);
-  dim3 grid(g.ntx, (g.ny + kRowsPerBlock - 1) / kRowsPerBlock, g.nz);
+  dim3 block(32, kFluctRows);
+  dim3 grid(g.ntx, (g.ny + kFluctRows - 1) / kFluctRows, (g.nz + 1) / 2);
   if (ph.g[0] == 0.f && ph.g[1] == 0.f && ph.g[2] == 0.f)
     k_stream_collide_fluct<S, kForcingNone, I><<<grid, block, 0, s>>>(g, ph, (const T *)src, (T *)dst);
   else if (ph.forcing == LBMD_FORCING_GUO)
