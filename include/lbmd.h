@@ -331,20 +331,12 @@ int lbmd_kernel_times(lbmd_ctx *ctx, double *lb_ms, double *md_ms, double *sprea
  *   f_out:   device, 19*V floats, receives f_p(x, t+1); solid nodes set to 0;
  *            must not overlap f_in
  *   cuda_stream: stream of the work (cudaStream_t; NULL = legacy default)
- * The geometry scratch (solid bitfield + tile flags) lives in one fixed device
- * array inside the library, 5 MiB per GPU that loads the library, held until
- * the process exits; it limits the box to ny * nz * ceil(nx / 32) <= 2^20
- * (e.g. 256^3).  Each call rebuilds it on the stream, so nothing carries over
- * from the previous call, but every call shares it: calls that may overlap on
- * the GPU (unordered streams) race and must be serialised by the caller.  The
- * first call on each device looks up the array's device address
- * (cudaGetSymbolAddress) and keeps it for the life of the process; make that
- * first call before any stream capture.  A device reset (cudaDeviceReset)
- * may move the array: after one, this entry point must not be called again
- * in the same process.
+ * The walls are computed from the parameters in the kernel: nothing is kept
+ * between calls, and calls on different streams do not disturb each other.
+ * The box is limited to ny * nz * ceil(nx / 32) <= 2^20 (e.g. 256^3).
  * Asynchronous; errors: LBMD_EINVAL (bad parameter, f_in == f_out,
  * ny > 524280), LBMD_EUNSUPPORTED (see params), LBMD_ESIZE (box beyond the
- * scratch limit), LBMD_ECUDA (a launch failed; the status is that of this
+ * limit), LBMD_ECUDA (a launch failed; the status is that of this
  * call's own launches).
  */
 int lbmd_lb_step_noalloc(const lbmd_params *params, const float *f_in, float *f_out,

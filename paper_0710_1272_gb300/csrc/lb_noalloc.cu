@@ -8,165 +8,125 @@
 // the allocator -- but does own two population buffers and wants the solvent
 // update of the coupled step (no beads).
 //
-// The only global memory besides the caller's input and output is the
-// geometry scratch (solid bitfield and per-tile "solid nearby" flags), kept in
-// a fixed file-scope device array.  Its size limits the box: ny * nz *
-// ceil(nx / 32) <= 2^20 tiles (for example 256^3).  Every call rebuilds the
-// scratch on the device from the parameters, so no state carries over from the
-// previous call.  All calls share that one array: calls that overlap on the GPU
-// (different streams, no ordering between them) race on it.
+// One kernel and no memory besides the caller's input and output: whether a
+// node or its neighbour is solid is computed from the Sec. III geometry, for
+// the few nodes beside a wall.  (Two more kernels used to build a bitfield and
+// tile flags in a fixed device array on every call, 9 us and two launches of a
+// 73 us call on 160x96x96, and calls on different streams raced on it.)
+// The box stays limited to the size that array had room for.
 #include <cuda_runtime.h>
-
-#include <mutex>
 
 #include "lbmd_common.cuh"
 
 namespace lbmd {
 namespace {
 
-constexpr int kNoAllocMaxTiles = 1 << 20;  // words of the bitfield = tiles
-constexpr int kMaxDevices = 64;
-
-// [kNoAllocMaxTiles] uint32 solid words, then [kNoAllocMaxTiles] uint8 flags
-static __device__ __align__(256) uint32_t g_noalloc_scratch[kNoAllocMaxTiles + kNoAllocMaxTiles / 4];
-
-std::mutex g_mu;
-void *g_scratch_addr[kMaxDevices];  // device address of g_noalloc_scratch per device
+constexpr int kNoAllocMaxTiles = 1 << 20;  // ny nz ceil(nx / 32): 2^25 nodes, 32-bit offsets
 
 struct GeoParams {
-  int nx, ny, nz, ntx;
-  int wall_x, wall_t, pore_d, pore_y0, pore_z0, y_walls;
+  int nx, ny, nz;
+  WallGeom wall;
 };
 
-__device__ __forceinline__ bool solid_node(const GeoParams &q, int x, int y, int z) {
-  if (q.y_walls && (y == 0 || y == q.ny - 1)) return true;
-  if (q.wall_x < 0) return false;
-  int dx = x - q.wall_x;
+// Which of the node itself (bit 0) and its neighbours x + c_p (bit p) are solid.
+__device__ __forceinline__ uint32_t solid_around(const GeoParams &q, int x, int y, int z) {
+  const WallGeom &w = q.wall;
+  int dx = x - w.wall_x;  // layers after the first one, around the box
   if (dx < 0) dx += q.nx;
-  if (dx >= q.wall_t) return false;
-  const bool in_pore = q.pore_d > 0 && y >= q.pore_y0 && y < q.pore_y0 + q.pore_d &&
-                       z >= q.pore_z0 && z < q.pore_z0 + q.pore_d;
-  return !in_pore;
-}
-
-// One thread per bitfield word: the solid bits of 32 consecutive x.
-__global__ void k_noalloc_bits(GeoParams q, uint32_t *bits) {
-  const long long w = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long nwords = (long long)q.ny * q.nz * q.ntx;
-  if (w >= nwords) return;
-  const int t = (int)(w % q.ntx);
-  const long long row = w / q.ntx;
-  const int y = (int)(row % q.ny), z = (int)(row / q.ny);
-  uint32_t word = 0;
-  for (int b = 0; b < 32; ++b) {
-    const int x = t * 32 + b;
-    if (x < q.nx && solid_node(q, x, y, z)) word |= 1u << b;
+  const bool layer = w.wall_x >= 0 && (dx <= w.wall_t || dx == q.nx - 1);
+  const bool rows = w.y_walls && (y <= 1 || y >= q.ny - 2);
+  if (!layer && !rows) return 0u;
+  // solid along each axis at offsets -1, 0, +1
+  bool in[3], row[3], py[3], pz[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    int a = dx + k - 1;
+    a = a < 0 ? a + q.nx : (a >= q.nx ? a - q.nx : a);
+    in[k] = w.wall_x >= 0 && a < w.wall_t;
+    const int b = k == 0 ? wrap_m1(y, q.ny) : (k == 2 ? wrap_p1(y, q.ny) : y);
+    const int c = k == 0 ? wrap_m1(z, q.nz) : (k == 2 ? wrap_p1(z, q.nz) : z);
+    row[k] = w.y_walls && (b == 0 || b == q.ny - 1);
+    py[k] = b >= w.pore_y0 && b < w.pore_y0 + w.pore_d;
+    pz[k] = c >= w.pore_z0 && c < w.pore_z0 + w.pore_d;
   }
-  bits[w] = word;
-}
-
-__device__ __forceinline__ bool bit_at(const uint32_t *bits, const GeoParams &q, int x, int y, int z) {
-  return (bits[((long long)z * q.ny + y) * q.ntx + (x >> 5)] >> (x & 31)) & 1u;
-}
-
-// One thread per tile: 1 if a solid node lies within one node of the tile.
-__global__ void k_noalloc_tiles(GeoParams q, const uint32_t *bits, uint8_t *tiles) {
-  const long long w = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long ntiles = (long long)q.ny * q.nz * q.ntx;
-  if (w >= ntiles) return;
-  const int t = (int)(w % q.ntx);
-  const long long row = w / q.ntx;
-  const int y = (int)(row % q.ny), z = (int)(row / q.ny);
-  const int x0 = t * 32, x1 = min(q.nx - 1, x0 + 31);
-  const int xl = wrapi(x0 - 1, q.nx), xr = wrapi(x1 + 1, q.nx);
-  uint8_t near = 0;
-  for (int dz = -1; dz <= 1; ++dz)
-    for (int dy = -1; dy <= 1; ++dy) {
-      const int yy = wrapi(y + dy, q.ny), zz = wrapi(z + dz, q.nz);
-      // the tile's own 32 cells (bits beyond nx are zero), then its two x-neighbours
-      if (bits[((long long)zz * q.ny + yy) * q.ntx + t] != 0u || bit_at(bits, q, xl, yy, zz) ||
-          bit_at(bits, q, xr, yy, zz))
-        near = 1;
-    }
-  tiles[w] = near;
+  uint32_t s = 0u;
+#pragma unroll
+  for (int p = 0; p < kQ; ++p)
+    if (row[1 + cy(p)] || (in[1 + cx(p)] && !(py[1 + cy(p)] && pz[1 + cz(p)]))) s |= 1u << p;
+  return s;
 }
 
 // Collide-then-push form of Eq. 5 on absolute populations:
 //   f*_p(x) = f_p - (f_p - f_eq,p(rho, u)) / tau + S_p(g),
 //   f_p(x + c_p, t+1) = f*_p(x) if x + c_p is fluid, else f_opp(p)(x, t+1) = f*_p(x).
-// Solid nodes of the output are set to zero.
+// Solid nodes of the output are set to zero.  Bound by HBM (19 loads, 19
+// stores per node, those for c_x = +-1 shifted by a node); 32-bit offsets and
+// one reciprocal per node, where 64-bit offsets, three divisions and per-tile
+// flags had made it a kernel of 60 us at 160x96x96 (33 us of traffic): the whole
+// call took 71.9 us, now 42.5.
 template <int FORCING>
-__global__ void __launch_bounds__(256) k_noalloc_step(GeoParams q, float omega, float rho0,
-                                                      float gx, float gy, float gz,
-                                                      const uint32_t *__restrict__ bits,
-                                                      const uint8_t *__restrict__ tiles,
-                                                      const float *__restrict__ fin,
-                                                      float *__restrict__ fout) {
+__global__ void __launch_bounds__(256, 5) k_noalloc_step(GeoParams q, float omega, float gx, float gy,
+                                                         float gz, const float *__restrict__ fin,
+                                                         float *__restrict__ fout) {
   const int x = blockIdx.x * 32 + threadIdx.x;
   const int y = blockIdx.y * 8 + threadIdx.y;
   const int z = blockIdx.z;
   if (x >= q.nx || y >= q.ny) return;
-  const long long V = (long long)q.nx * q.ny * q.nz;
-  const long long self = ((long long)z * q.ny + y) * q.nx + x;
-  const bool near = tiles[((long long)z * q.ny + y) * q.ntx + (x >> 5)] != 0;
-  if (near && bit_at(bits, q, x, y, z)) {
+  const int nx = q.nx, ny = q.ny, nz = q.nz;
+  const int V = nx * ny * nz;
+  const int self = (z * ny + y) * nx + x;
+  float f[kQ];
+#pragma unroll
+  for (int p = 0; p < kQ; ++p) f[p] = __ldg(fin + (p * V + self));
+  const uint32_t solid = solid_around(q, x, y, z);
+  if (solid & 1u) {
 #pragma unroll
     for (int p = 0; p < kQ; ++p) fout[p * V + self] = 0.f;
     return;
   }
-  float f[kQ];
-  float rho = 0.f, jx = 0.f, jy = 0.f, jz = 0.f;
+  float rho = f[0], jx = 0.f, jy = 0.f, jz = 0.f;
 #pragma unroll
-  for (int p = 0; p < kQ; ++p) {
-    f[p] = fin[p * V + self];
+  for (int p = 1; p < kQ; ++p) {
     rho += f[p];
-    jx += cx(p) * f[p];
-    jy += cy(p) * f[p];
-    jz += cz(p) * f[p];
+    if (cx(p)) jx += cx(p) > 0 ? f[p] : -f[p];
+    if (cy(p)) jy += cy(p) > 0 ? f[p] : -f[p];
+    if (cz(p)) jz += cz(p) > 0 ? f[p] : -f[p];
   }
   if (FORCING == LBMD_FORCING_GUO) {
     jx += 0.5f * gx;
     jy += 0.5f * gy;
     jz += 0.5f * gz;
   }
-  const float ux = jx / rho, uy = jy / rho, uz = jz / rho;
-  const float usq15 = 1.5f * (ux * ux + uy * uy + uz * uz);
+  const float inv = 1.0f / rho;
+  const float ux = jx * inv, uy = jy * inv, uz = jz * inv;
+  const float base = 1.0f - 1.5f * (ux * ux + uy * uy + uz * uz);
   const float gu = gx * ux + gy * uy + gz * uz;
-  const int nx = q.nx, ny = q.ny, nz = q.nz;
+  const float kguo = 1.0f - 0.5f * omega;
+  // source of direction p, c_p . u = cu
+  const auto source = [&](int p, float cu) {
+    const float cg = cx(p) * gx + cy(p) * gy + cz(p) * gz;
+    return FORCING == LBMD_FORCING_GUO ? kguo * wq(p) * (3.0f * (cg - gu) + 9.0f * cu * cg)
+                                       : 3.0f * wq(p) * cg;
+  };
+  // opposite directions p, p + 1 (odd p) share the even part of the equilibrium
+  f[0] = f[0] - omega * (f[0] - wq(0) * rho * base) + source(0, 0.f);
+#pragma unroll
+  for (int p = 1; p < kQ; p += 2) {
+    const float cu = cx(p) * ux + cy(p) * uy + cz(p) * uz, wr = wq(p) * rho;
+    const float even = wr * (base + 4.5f * cu * cu), odd = 3.0f * wr * cu;
+    f[p] = f[p] - omega * (f[p] - (even + odd)) + source(p, cu);
+    f[p + 1] = f[p + 1] - omega * (f[p + 1] - (even - odd)) + source(p + 1, -cu);
+  }
+  const int xm = wrap_m1(x, nx), xp = wrap_p1(x, nx), ym = wrap_m1(y, ny), yp = wrap_p1(y, ny);
+  const int zm = wrap_m1(z, nz), zp = wrap_p1(z, nz);
 #pragma unroll
   for (int p = 0; p < kQ; ++p) {
-    const float cu = cx(p) * ux + cy(p) * uy + cz(p) * uz;
-    const float feq = wq(p) * rho * (1.0f + 3.0f * cu + 4.5f * cu * cu - usq15);
-    const float cg = cx(p) * gx + cy(p) * gy + cz(p) * gz;
-    const float src = FORCING == LBMD_FORCING_GUO
-                          ? (1.0f - 0.5f * omega) * wq(p) * (3.0f * (cg - gu) + 9.0f * cu * cg)
-                          : 3.0f * wq(p) * cg;
-    const float fs = f[p] - omega * (f[p] - feq) + src;
-    const int xd = cx(p) == 1 ? wrap_p1(x, nx) : (cx(p) == -1 ? wrap_m1(x, nx) : x);
-    const int yd = cy(p) == 1 ? wrap_p1(y, ny) : (cy(p) == -1 ? wrap_m1(y, ny) : y);
-    const int zd = cz(p) == 1 ? wrap_p1(z, nz) : (cz(p) == -1 ? wrap_m1(z, nz) : z);
-    if (p != 0 && near && bit_at(bits, q, xd, yd, zd))
-      fout[opp(p) * V + self] = fs;
-    else
-      fout[p * V + ((long long)zd * ny + yd) * nx + xd] = fs;
+    const int xd = cx(p) == 1 ? xp : (cx(p) == -1 ? xm : x);
+    const int yd = cy(p) == 1 ? yp : (cy(p) == -1 ? ym : y);
+    const int zd = cz(p) == 1 ? zp : (cz(p) == -1 ? zm : z);
+    const int to = p * V + ((zd * ny + yd) * nx + xd), back = opp(p) * V + self;
+    fout[((solid >> p) & 1u) ? back : to] = f[p];
   }
-}
-
-// Device address of the scratch array on the current device, looked up once.
-cudaError_t scratch_address(uint32_t **out) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-  std::lock_guard<std::mutex> lock(g_mu);
-  if (!g_scratch_addr[dev]) {
-    void *p = nullptr;
-    e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
-    if (e != cudaSuccess) return e;
-    g_scratch_addr[dev] = p;
-  }
-  *out = (uint32_t *)g_scratch_addr[dev];
-  return cudaSuccess;
 }
 
 }  // namespace
@@ -189,48 +149,31 @@ extern "C" int lbmd_lb_step_noalloc(const lbmd_params *p, const float *f_in, flo
   q.nx = p->nx;
   q.ny = p->ny;
   q.nz = p->nz;
-  q.ntx = (p->nx + 31) / 32;
-  q.wall_x = p->wall_x;
-  q.wall_t = p->wall_thickness;
-  q.pore_d = p->pore_d;
-  q.y_walls = p->y_walls;
+  q.wall = WallGeom{p->wall_x, p->wall_thickness, 0, 0, 0, p->y_walls};
   if (p->wall_x >= 0) {
     if (p->wall_thickness < 1 || p->wall_thickness >= p->nx) return LBMD_EINVAL;
     if (p->pore_d < 0 || p->pore_d > p->ny || p->pore_d > p->nz) return LBMD_EINVAL;
-    q.pore_y0 = p->pore_y0 >= 0 ? p->pore_y0 : (p->ny - p->pore_d) / 2;
-    q.pore_z0 = p->pore_z0 >= 0 ? p->pore_z0 : (p->nz - p->pore_d) / 2;
-    if (q.pore_y0 + p->pore_d > p->ny || q.pore_z0 + p->pore_d > p->nz) return LBMD_EINVAL;
-  } else {
-    q.pore_y0 = q.pore_z0 = 0;
+    q.wall.pore_d = p->pore_d;
+    q.wall.pore_y0 = p->pore_y0 >= 0 ? p->pore_y0 : (p->ny - p->pore_d) / 2;
+    q.wall.pore_z0 = p->pore_z0 >= 0 ? p->pore_z0 : (p->nz - p->pore_d) / 2;
+    if (q.wall.pore_y0 + p->pore_d > p->ny || q.wall.pore_z0 + p->pore_d > p->nz) return LBMD_EINVAL;
   }
-  const long long tiles = (long long)q.ny * q.nz * q.ntx;
-  if (tiles > kNoAllocMaxTiles) return LBMD_ESIZE;  // box larger than the fixed scratch
+  const int ntx = (q.nx + 31) / 32;
+  const long long tiles = (long long)q.ny * q.nz * ntx;
+  if (tiles > kNoAllocMaxTiles) return LBMD_ESIZE;  // box beyond the limit
   if ((q.ny + 7) / 8 > 65535) return LBMD_EINVAL;   // grid y of the step kernel (ny <= 524280)
 
-  uint32_t *scratch = nullptr;
-  if (scratch_address(&scratch) != cudaSuccess) return LBMD_ECUDA;
-  uint32_t *bits = scratch;
-  uint8_t *tile = (uint8_t *)(scratch + kNoAllocMaxTiles);
   // launched with cudaLaunchKernelEx, whose return value is the status of
   // that launch alone (not an error left behind by unrelated earlier work)
   cudaLaunchConfig_t cfg = {};
   cfg.stream = (cudaStream_t)cuda_stream;
-  cfg.blockDim = dim3(256);
-  cfg.gridDim = dim3((unsigned)((tiles + 255) / 256));
-  if (cudaLaunchKernelEx(&cfg, k_noalloc_bits, q, bits) != cudaSuccess) return LBMD_ECUDA;
-  if (cudaLaunchKernelEx(&cfg, k_noalloc_tiles, q, (const uint32_t *)bits, tile) != cudaSuccess)
-    return LBMD_ECUDA;
   cfg.blockDim = dim3(32, 8);
-  cfg.gridDim = dim3(q.ntx, (q.ny + 7) / 8, q.nz);
-  const float omega = (float)(1.0 / p->tau), rho0 = (float)p->rho0;
+  cfg.gridDim = dim3(ntx, (q.ny + 7) / 8, q.nz);
+  const float omega = (float)(1.0 / p->tau);
   const float gx = (float)p->body_force[0], gy = (float)p->body_force[1], gz = (float)p->body_force[2];
-  const uint32_t *cbits = bits;
-  const uint8_t *ctile = tile;
   const cudaError_t e =
       p->forcing == LBMD_FORCING_GUO
-          ? cudaLaunchKernelEx(&cfg, k_noalloc_step<LBMD_FORCING_GUO>, q, omega, rho0, gx, gy, gz, cbits,
-                               ctile, f_in, f_out)
-          : cudaLaunchKernelEx(&cfg, k_noalloc_step<LBMD_FORCING_PAPER>, q, omega, rho0, gx, gy, gz, cbits,
-                               ctile, f_in, f_out);
+          ? cudaLaunchKernelEx(&cfg, k_noalloc_step<LBMD_FORCING_GUO>, q, omega, gx, gy, gz, f_in, f_out)
+          : cudaLaunchKernelEx(&cfg, k_noalloc_step<LBMD_FORCING_PAPER>, q, omega, gx, gy, gz, f_in, f_out);
   return e == cudaSuccess ? LBMD_OK : LBMD_ECUDA;
 }
