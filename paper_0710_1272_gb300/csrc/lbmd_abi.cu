@@ -122,11 +122,9 @@ cudaError_t enqueue_step(lbmd_ctx *c, int src) {
   if (c->N > 0) {
     // (1) gather from the pre-step populations, and the MD cycle on the
     // high-priority side stream while the stream-collide runs on the main
-    // one.  Where the stream-collide sets the step, the gather runs on the
-    // side stream too, so the stream-collide starts at once (FP32 benchmark
-    // box: 113.5 -> 111.5 us); where the MD branch sets it, the gather runs
-    // first, before the stream-collide takes the SMs (FP16: 83.7 against
-    // 85.6 us the other way).
+    // one.  Where the stream-collide sets the step, it starts at once; where
+    // the MD branch sets it, the gather runs first, before the
+    // stream-collide takes the SMs (figures at spread_take_in_apply).
     ChainArgs a = c->chain;
     a.f = A;
     a.f_mode = pop_mode(c, src);

@@ -244,12 +244,14 @@ constexpr int kOwnerFree = 0x7f7f7f7f;
 cudaError_t launch_spread_sum(const ChainArgs &a, bool records, cudaStream_t s);
 // Single box: true when the apply should convert the sums itself (the MD
 // branch sets the step), false when the stream-collide sets it -- taken as a
-// stream-collide moving 480 MB or more per step (~70 us at the HBM rate, about
-// the MD branch of a 400-bead chain beside it): FP32 populations of 3.2 M
-// nodes or more.
+// stream-collide moving 240 MB or more per step (~40 us at the HBM rate, about
+// the MD branch of a 400-bead chain beside it).  The gather follows the same
+// rule (enqueue_step).  Step of a 400-bead chain, us, true against false:
+// 144x80x80 FP32 (140 MB) 47.7 / 54.5, FP16 44.2 / 47.1; 256x128x128 FP16
+// (318 MB) 73.3 / 69.1, FP32 (637 MB) 105.3 / 101.6.
 inline bool spread_take_in_apply(int storage, long long nodes) {
   const long long bytes = 2LL * 19 * nodes * (storage == LBMD_STORE_F32 ? 4 : 2);
-  return bytes < 480000000LL;
+  return bytes < 240000000LL;
 }
 // `take`: the owners' forces from their fixed-point sums (the sum ran with
 // records == false), else from the records.  `bump` (may be null):

@@ -1084,6 +1084,7 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
     rebuild = __syncthreads_or(bead && moved());
   }
 
+  asm volatile("griddepcontrol.launch_dependents;");  // the spread's sum may be placed
   if (bead) {
     a.pos[i] = rh;
     a.pos_lo[i] = rl;
@@ -1335,11 +1336,13 @@ cudaError_t launch_md_cycle(const ChainArgs &a, int priority, bool beside, cudaS
 
 // The sum of the spread as two kernels, one thread per (bead, corner) entry.
 __global__ void __launch_bounds__(256) k_spread_accum(ChainArgs a) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // the MD cycle's impulses
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= 8 * a.N) return;
-  spread_add(a, e, a.J[e >> 3]);
+  if (e < 8 * a.N) spread_add(a, e, a.J[e >> 3]);
+  asm volatile("griddepcontrol.launch_dependents;");
 }
 __global__ void __launch_bounds__(256) k_spread_finalize(ChainArgs a) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // every share
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= 8 * a.N) return;
   spread_finalize(a, e);
@@ -1418,10 +1421,20 @@ __global__ void __launch_bounds__(256)
 
 cudaError_t launch_spread_sum(const ChainArgs &a, bool records, cudaStream_t s) {
   if (a.N <= 0) return cudaSuccess;
-  const int blocks = (8 * a.N + 255) / 256;
-  k_spread_accum<<<blocks, 256, 0, s>>>(a);
-  if (records) k_spread_finalize<<<blocks, 256, 0, s>>>(a);
-  return cudaGetLastError();
+  // both may be placed while the kernel before them ends (programmatic
+  // dependent launch; they wait for its results first)
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((8 * a.N + 255) / 256);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_spread_accum, a);
+  if (e != cudaSuccess || !records) return e;
+  return cudaLaunchKernelEx(&cfg, k_spread_finalize, a);
 }
 
 template <int S>
