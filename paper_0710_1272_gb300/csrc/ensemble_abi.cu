@@ -29,7 +29,7 @@ constexpr int kEnsBlock = 16;   // steps per long graph
 const int kEnsGraphSteps[3] = {1, 2, kEnsBlock};
 
 struct EnsLayout {
-  size_t mem, lbd, tiles, n_tiles, beads, live, cap, chains, stage;
+  size_t mem, lbd, tiles, n_tiles, beads, live, cap, chains, status, stage;
   size_t stage_floats;
   size_t max_tiles;  // tile capacity (rows = 4, every realisation)
   int nb;            // padded bead slots
@@ -96,6 +96,7 @@ EnsLayout make_ens_layout(const lbmd_params *m, int32_t count) {
   E.live = take(2 * (size_t)count * sizeof(int));
   E.cap = take(sizeof(long long));
   E.chains = take((size_t)count * sizeof(int));
+  E.status = take((size_t)count * sizeof(DevStatus));
   E.stage = take(E.stage_floats * sizeof(float));
   E.off.resize(count);
   E.L.resize(count);
@@ -128,6 +129,7 @@ struct lbmd_ensemble {
   int *d_n_tiles, *d_live, *d_chains;
   int2 *d_beads;
   long long *d_cap;
+  DevStatus *d_status;  // [count] the realisations' status words, gathered for a read-out
   float *stage;
   int rows, warps, claim, cpt, grid, sms;
   long long G;        // ensemble steps enqueued so far
@@ -226,13 +228,14 @@ cudaError_t read_live(lbmd_ensemble *e, std::vector<int> &live) {
   return cudaStreamSynchronize(e->own);
 }
 
+// One gather and one copy: a copy per realisation took ~10 us each.
 cudaError_t read_status(lbmd_ensemble *e, std::vector<DevStatus> &st) {
   st.resize(e->count);
-  cudaError_t err;
-  for (int m = 0; m < e->count; ++m)
-    if ((err = cudaMemcpyAsync(&st[m], e->inst[m].status, sizeof(DevStatus), cudaMemcpyDeviceToHost,
-                               e->own)) != cudaSuccess)
-      return err;
+  cudaError_t err = launch_ens_status(e->d_mem, e->count, e->d_status, e->own);
+  if (err != cudaSuccess) return err;
+  if ((err = cudaMemcpyAsync(st.data(), e->d_status, e->count * sizeof(DevStatus), cudaMemcpyDeviceToHost,
+                             e->own)) != cudaSuccess)
+    return err;
   return cudaStreamSynchronize(e->own);
 }
 
@@ -458,6 +461,7 @@ int lbmd_ensemble_create(const lbmd_params *members, int32_t count, void *dev_wo
   e->d_beads = (int2 *)(e->ws + E.beads);
   e->d_live = (int *)(e->ws + E.live);
   e->d_cap = (long long *)(e->ws + E.cap);
+  e->d_status = (DevStatus *)(e->ws + E.status);
   e->d_chains = (int *)(e->ws + E.chains);
   e->stage = (float *)(e->ws + E.stage);
   e->rows = 8;
@@ -645,19 +649,17 @@ int lbmd_ensemble_read_beads(lbmd_ensemble *e, int32_t member, double *pos, doub
   const ChainArgs &a = e->inst[member].chain;
   const int N = a.N;
   if (!pos && !vel) return LBMD_OK;
-  EK(e, cudaEventRecord(e->ev_in, e->user));
-  EK(e, cudaStreamWaitEvent(e->own, e->ev_in, 0));
   double *dx = pos, *dy = vel;
   if (!dst_is_device) {
     dx = pos ? (double *)e->stage : nullptr;
     dy = vel ? (double *)e->stage + 3 * N : nullptr;
   }
-  EK(e, launch_read_beads(a.pos, a.pos_lo, a.vel, N, a.ox, a.oy, a.oz, dx, dy, e->own));
+  EK(e, launch_read_beads(a.pos, a.pos_lo, a.vel, N, a.ox, a.oy, a.oz, dx, dy, e->user));
   if (!dst_is_device) {
-    if (pos) EK(e, cudaMemcpyAsync(pos, dx, 3 * N * sizeof(double), cudaMemcpyDeviceToHost, e->own));
-    if (vel) EK(e, cudaMemcpyAsync(vel, dy, 3 * N * sizeof(double), cudaMemcpyDeviceToHost, e->own));
+    if (pos) EK(e, cudaMemcpyAsync(pos, dx, 3 * N * sizeof(double), cudaMemcpyDeviceToHost, e->user));
+    if (vel) EK(e, cudaMemcpyAsync(vel, dy, 3 * N * sizeof(double), cudaMemcpyDeviceToHost, e->user));
   }
-  EK(e, cudaStreamSynchronize(e->own));
+  EK(e, cudaStreamSynchronize(e->user));
   return LBMD_OK;
 }
 
@@ -666,18 +668,15 @@ int lbmd_ensemble_read_populations(lbmd_ensemble *e, int32_t member, float *f, i
   if (rc) return rc;
   if (member < 0 || member >= e->count) return fail(LBMD_EINVAL, "member out of range");
   if (!f) return fail(LBMD_EINVAL, "f is NULL");
-  EK(e, cudaEventRecord(e->ev_in, e->user));
-  EK(e, cudaStreamWaitEvent(e->own, e->ev_in, 0));
-  DevStatus st;
-  EK(e, cudaMemcpyAsync(&st, e->inst[member].status, sizeof(st), cudaMemcpyDeviceToHost, e->own));
-  EK(e, cudaStreamSynchronize(e->own));
   const Instance &in = e->inst[member];
   const LbGeom &g = in.geo;
   const float rho0 = (float)e->p[member].rho0;
-  const void *src = in.pop[st.out_buf & 1];
+  // the buffer of the last step is found on the device; the caller's stream is
+  // already behind every step enqueued so far
+  const void *src0 = in.pop[0], *src1 = in.pop[1];
   if (dst_is_device) {
-    EK(e, launch_read_pulled(e->storage, g, rho0, src, kPopPull, 0, g.nz, f, g.V, e->own));
-    EK(e, cudaStreamSynchronize(e->own));
+    EK(e, launch_read_pulled(e->storage, g, rho0, src0, src1, in.status, kPopPull, 0, g.nz, f, g.V, e->user));
+    EK(e, cudaStreamSynchronize(e->user));
     return LBMD_OK;
   }
   const long long plane = (long long)g.nx * g.ny;
@@ -685,12 +684,12 @@ int lbmd_ensemble_read_populations(lbmd_ensemble *e, int32_t member, float *f, i
   for (long long z0 = 0; z0 < g.nz; z0 += nzc_max) {
     const long long nzc = std::min(nzc_max, (long long)g.nz - z0);
     const long long cells = nzc * plane;
-    EK(e, launch_read_pulled(e->storage, g, rho0, src, kPopPull, z0, nzc, e->stage, cells, e->own));
+    EK(e, launch_read_pulled(e->storage, g, rho0, src0, src1, in.status, kPopPull, z0, nzc, e->stage, cells, e->user));
     for (int q = 0; q < 19; ++q)
       EK(e, cudaMemcpyAsync(f + q * g.V + z0 * plane, e->stage + q * cells, cells * 4,
-                            cudaMemcpyDeviceToHost, e->own));
+                            cudaMemcpyDeviceToHost, e->user));
   }
-  EK(e, cudaStreamSynchronize(e->own));
+  EK(e, cudaStreamSynchronize(e->user));
   return LBMD_OK;
 }
 

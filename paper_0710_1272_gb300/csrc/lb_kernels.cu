@@ -302,8 +302,10 @@ __global__ void k_read_moments(LbGeom g, LbPhys ph, const typename Store<S>::T *
 }
 
 template <int S>
-__global__ void k_read_pulled(LbGeom g, float rho0, const typename Store<S>::T *__restrict__ src,
-                              int mode, int z0, float *f, long long fstride) {
+__global__ void k_read_pulled(LbGeom g, float rho0, const typename Store<S>::T *src0,
+                              const typename Store<S>::T *src1, const DevStatus *st, int mode, int z0,
+                              float *f, long long fstride) {
+  const typename Store<S>::T *__restrict__ src = st != nullptr && (st->out_buf & 1) ? src1 : src0;
   const int x = blockIdx.x * 32 + threadIdx.x;
   const int y = blockIdx.y * kRowsPerBlock + threadIdx.y;
   const int z = z0 + blockIdx.z;
@@ -342,19 +344,19 @@ cudaError_t launch_read_moments(int storage, const LbGeom &g, const LbPhys &ph, 
 }
 
 cudaError_t launch_read_pulled(int storage, const LbGeom &g, float rho0, const void *src,
-                               int mode, long long z0, long long nzc, float *f,
-                               long long fstride, cudaStream_t s) {
+                               const void *src1, const DevStatus *st, int mode, long long z0,
+                               long long nzc, float *f, long long fstride, cudaStream_t s) {
   dim3 block(32, kRowsPerBlock);
   dim3 grid(g.ntx, (g.ny + kRowsPerBlock - 1) / kRowsPerBlock, (unsigned)nzc);
   switch (storage) {
     case LBMD_STORE_F32:
-      k_read_pulled<LBMD_STORE_F32><<<grid, block, 0, s>>>(g, rho0, (const float *)src, mode, (int)z0, f, fstride);
+      k_read_pulled<LBMD_STORE_F32><<<grid, block, 0, s>>>(g, rho0, (const float *)src, (const float *)src1, st, mode, (int)z0, f, fstride);
       break;
     case LBMD_STORE_F16:
-      k_read_pulled<LBMD_STORE_F16><<<grid, block, 0, s>>>(g, rho0, (const __half *)src, mode, (int)z0, f, fstride);
+      k_read_pulled<LBMD_STORE_F16><<<grid, block, 0, s>>>(g, rho0, (const __half *)src, (const __half *)src1, st, mode, (int)z0, f, fstride);
       break;
     case LBMD_STORE_BF16:
-      k_read_pulled<LBMD_STORE_BF16><<<grid, block, 0, s>>>(g, rho0, (const __nv_bfloat16 *)src, mode, (int)z0, f, fstride);
+      k_read_pulled<LBMD_STORE_BF16><<<grid, block, 0, s>>>(g, rho0, (const __nv_bfloat16 *)src, (const __nv_bfloat16 *)src1, st, mode, (int)z0, f, fstride);
       break;
     default:
       return cudaErrorInvalidValue;

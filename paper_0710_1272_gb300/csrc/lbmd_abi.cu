@@ -511,7 +511,8 @@ int lbmd_read_populations(lbmd_ctx *c, float *f, int dst_is_device) {
   const void *src = c->pop[c->cur];
   const int mode = pop_mode(c, c->cur);
   if (dst_is_device) {
-    CK(c, launch_read_pulled(c->p.storage, g, (float)c->p.rho0, src, mode, 0, g.nz, f, g.V, c->user));
+    CK(c, launch_read_pulled(c->p.storage, g, (float)c->p.rho0, src, nullptr, nullptr, mode, 0, g.nz, f,
+                             g.V, c->user));
     return LBMD_OK;
   }
   const long long plane = (long long)g.nx * g.ny;
@@ -519,8 +520,8 @@ int lbmd_read_populations(lbmd_ctx *c, float *f, int dst_is_device) {
   for (long long z0 = 0; z0 < g.nz; z0 += nzc_max) {
     const long long nzc = std::min(nzc_max, (long long)g.nz - z0);
     const long long cells = nzc * plane;
-    CK(c, launch_read_pulled(c->p.storage, g, (float)c->p.rho0, src, mode, z0, nzc, c->stage, cells,
-                             c->user));
+    CK(c, launch_read_pulled(c->p.storage, g, (float)c->p.rho0, src, nullptr, nullptr, mode, z0, nzc,
+                             c->stage, cells, c->user));
     for (int q = 0; q < 19; ++q)
       CK(c, cudaMemcpyAsync(f + q * g.V + z0 * plane, c->stage + q * cells, cells * 4,
                             cudaMemcpyDeviceToHost, c->user));

@@ -216,9 +216,12 @@ cudaError_t launch_lb_aa_fluct(int storage, const LbGeom &g, const LbPhys &ph, v
 cudaError_t launch_read_moments(int storage, const LbGeom &g, const LbPhys &ph,
                                 const void *src, int mode, long long z0, long long nzc,
                                 float *rho, float *u, long long ustride, cudaStream_t s);
+// st (may be null): the populations are in src1 if st->out_buf is odd.
 cudaError_t launch_read_pulled(int storage, const LbGeom &g, float rho0, const void *src,
-                               int mode, long long z0, long long nzc, float *f,
-                               long long fstride, cudaStream_t s);
+                               const void *src1, const DevStatus *st, int mode, long long z0,
+                               long long nzc, float *f, long long fstride, cudaStream_t s);
+// Status words of `count` realisations, side by side into `out`.
+cudaError_t launch_ens_status(const EnsMember *mem, int count, DevStatus *out, cudaStream_t s);
 cudaError_t launch_gather(int storage, const ChainArgs &a, cudaStream_t s);
 cudaError_t launch_md_cycle(const ChainArgs &a, int priority, bool beside, cudaStream_t s);
 // Spread of the bead impulses (stage 3), independent of the order of

@@ -1579,6 +1579,16 @@ cudaError_t launch_ens_spread(int storage, const EnsMember *mem, const int2 *bea
   return cudaGetLastError();
 }
 
+__global__ void k_ens_status(const EnsMember *__restrict__ mem, int count, DevStatus *__restrict__ out) {
+  const int m = blockIdx.x * blockDim.x + threadIdx.x;
+  if (m < count) out[m] = *mem[m].a.status;
+}
+
+cudaError_t launch_ens_status(const EnsMember *mem, int count, DevStatus *out, cudaStream_t s) {
+  k_ens_status<<<(count + 127) / 128, 128, 0, s>>>(mem, count, out);
+  return cudaGetLastError();
+}
+
 __global__ void k_read_beads(const float4 *pos, const float4 *pos_lo, const float4 *vel, int N,
                              int ox, int oy, int oz, double *dpos, double *dvel) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
