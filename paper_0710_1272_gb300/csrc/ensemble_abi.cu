@@ -521,6 +521,7 @@ int lbmd_ensemble_create(const lbmd_params *members, int32_t count, void *dev_wo
     D.ny = g.ny;
     D.nz = g.nz;
     D.wall = g.wall;
+    D.pitch = g.pitch;
     D.fill_solid = fill_solid(members[m], traffic);
     D.lmask = g.lmask;
     D.Vp = (int)g.Vp;

@@ -32,14 +32,15 @@ __device__ __forceinline__ void aa_node(const LbGeom &g, const LbPhys &ph,
                                         uint32_t bb) {
   using St = Store<S>;
   const int nx = g.nx, ny = g.ny;
-  const I self = ((I)z * ny + y) * nx + x;
+  const int pitch = row_pitch<S>(g);
+  const I node = ((I)z * ny + y) * nx + x, self = ((I)z * ny + y) * pitch + x;
   const I st = pop_stride<S, I>((I)g.Vp);
   if (bb & 1u) return;  // solid node
   float h[kQ];
   if (!ODD) {
 #pragma unroll
     for (int p = 0; p < kQ; ++p) h[p] = St::load_plain(buf + (I)p * st + pop_base<S, I>(self));
-    collide19<FORCING, FLUCT>(h, ph, (uint32_t)self);
+    collide19<FORCING, FLUCT>(h, ph, (uint32_t)node);
     // The store addresses are the load addresses permuted; hiding the base
     // behind an empty asm makes the compiler recompute them after the
     // collision instead of keeping 19 of them live across it (which spills).
@@ -58,11 +59,11 @@ __device__ __forceinline__ void aa_node(const LbGeom &g, const LbPhys &ph,
     const int sx = cx(p) == 1 ? xm : (cx(p) == -1 ? xp : x);
     const int sy = cy(p) == 1 ? ym : (cy(p) == -1 ? yp : y);
     const int sz = cz(p) == 1 ? zm : (cz(p) == -1 ? zp : z);
-    const I sidx = (I)opp(p) * st + pop_base<S, I>(((I)sz * ny + sy) * nx + sx);
+    const I sidx = (I)opp(p) * st + pop_base<S, I>(((I)sz * ny + sy) * pitch + sx);
     const I bidx = (I)p * st + pop_base<S, I>(self);
     h[p] = St::load_plain(buf + (((bb >> p) & 1u) ? bidx : sidx));
   }
-  collide19<FORCING, FLUCT>(h, ph, (uint32_t)self);
+  collide19<FORCING, FLUCT>(h, ph, (uint32_t)node);
   // As in the even step: the store offsets equal the load offsets of the
   // opposite directions, so the coordinates are hidden behind an empty asm
   // and the offsets recomputed rather than kept live across the collision.
@@ -72,14 +73,14 @@ __device__ __forceinline__ void aa_node(const LbGeom &g, const LbPhys &ph,
   const int oxm = wrap_m1(ox, nx), oxp = wrap_p1(ox, nx);
   const int oym = wrap_m1(oy, ny), oyp = wrap_p1(oy, ny);
   const int ozm = wrap_m1(oz, g.nz), ozp = wrap_p1(oz, g.nz);
-  const I oself = ((I)oz * ny + oy) * nx + ox;
+  const I oself = ((I)oz * ny + oy) * pitch + ox;
 #pragma unroll
   for (int p = 0; p < kQ; ++p) {
     // destination node x + c_p; bit opp(p) of the mask: x + c_p is solid
     const int tx = cx(p) == 1 ? oxp : (cx(p) == -1 ? oxm : ox);
     const int ty = cy(p) == 1 ? oyp : (cy(p) == -1 ? oym : oy);
     const int tz = cz(p) == 1 ? ozp : (cz(p) == -1 ? ozm : oz);
-    const I didx = (I)p * st + pop_base<S, I>(((I)tz * ny + ty) * nx + tx);
+    const I didx = (I)p * st + pop_base<S, I>(((I)tz * ny + ty) * pitch + tx);
     const I bidx = (I)opp(p) * st + pop_base<S, I>(oself);
     St::store(out + (((bb >> opp(p)) & 1u) ? bidx : didx), h[p]);
   }

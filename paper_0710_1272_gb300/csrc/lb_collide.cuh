@@ -366,7 +366,8 @@ __device__ __forceinline__ void stream_collide_node(const LbGeom &g, const LbPhy
   }
   collide19<FORCING>(h, ph);
   if (bb & 1u) zero19(h);
-  const I st = pop_stride<S, I>((I)g.Vp), at = pop_base<S, I>(self);
+  const I st = pop_stride<S, I>((I)g.Vp);
+  const I at = pop_base<S, I>(((I)z * g.ny + y) * row_pitch<S>(g) + x);
 #pragma unroll
   for (int p = 0; p < kQ; ++p) St::store(dst + (I)p * st + at, h[p]);
 }
@@ -389,24 +390,26 @@ __device__ __forceinline__ void stream_collide_node2(const LbGeom &g, const LbPh
   }
   pull19_mask<S, int>(g, src, x, y, z, 0u, ha);  // constant masks: no selects
   pull19_mask<S, int>(g, src, x, y, z + 1, 0u, hb);
-  if (ma) bounce19<S, int>(g, src, self_a, ma, ha);
-  if (mb) bounce19<S, int>(g, src, self_b, mb, hb);
+  const int own_a = (z * g.ny + y) * row_pitch<S>(g) + x, own_b = own_a + row_pitch<S>(g) * g.ny;
+  if (ma) bounce19<S, int>(g, src, own_a, ma, ha);
+  if (mb) bounce19<S, int>(g, src, own_b, mb, hb);
   const int st = pop_stride<S, int>((int)g.Vp);
   if (!(ma & 1u)) {  // a solid node is pulled but not written
     collide19<FORCING>(ha, ph);
 #pragma unroll
-    for (int p = 0; p < kQ; ++p) St::store(dst + p * st + pop_base<S, int>(self_a), ha[p]);
+    for (int p = 0; p < kQ; ++p) St::store(dst + p * st + pop_base<S, int>(own_a), ha[p]);
   }
   if (!(mb & 1u)) {
     collide19<FORCING>(hb, ph);
 #pragma unroll
-    for (int p = 0; p < kQ; ++p) St::store(dst + p * st + pop_base<S, int>(self_b), hb[p]);
+    for (int p = 0; p < kQ; ++p) St::store(dst + p * st + pop_base<S, int>(own_b), hb[p]);
   }
 }
 
 // 16-bit storage, two x-adjacent nodes (2 xw, 2 xw + 1) of one box per
-// call: their deviations of one population share a 32-bit word (nx even, so
-// a pair never straddles a row).  Every population is one 32-bit load for
+// call: their deviations of one population share a 32-bit word (rows are held
+// at an even length, so a pair never straddles a row; the second node of an odd
+// row's last pair is padding).  Every population is one 32-bit load for
 // c_x = 0 and two for c_x = +-1 (the neighbouring word supplies the shifted
 // half; one byte permute assembles the pair), one 32-bit store, and the
 // collision runs once for both nodes on float2 with the paired FP32
@@ -437,7 +440,8 @@ __device__ __forceinline__ void pair_node(const LbGeom &g, const LbPhys &ph,
                                           const uint32_t *__restrict__ src,
                                           uint32_t *__restrict__ dst, int xw, int y, int z) {
   using P = Pair16<T2>;
-  const int wpr = g.nx >> 1;  // words per row
+  const int wpr = g.pitch >> 1;  // words per row
+  const bool odd = g.nx & 1, lone = odd && xw == wpr - 1;
   // a word w of the node pairs' row-major order, population p: words of
   // pop_base's blocks (32 words a population)
   constexpr int kW = kBlockNodes / 2;
@@ -449,7 +453,11 @@ __device__ __forceinline__ void pair_node(const LbGeom &g, const LbPhys &ph,
   const int xl = xw == 0 ? wpr - 1 : xw - 1, xr = xw == wpr - 1 ? 0 : xw + 1;
   // link masks of the two nodes (bit 0: solid; bit p: the pull source is solid)
   uint2 bb = make_uint2(0u, 0u);
-  if (beside_wall<2>(g, 2 * xw, y)) bb = __ldg(reinterpret_cast<const uint2 *>(g.lmask) + self);
+  if (beside_wall<2>(g, 2 * xw, y)) {
+    const uint32_t *m = g.lmask + ((z * ny + y) * g.nx + 2 * xw);
+    bb.x = __ldg(m);
+    if (!lone) bb.y = __ldg(m + 1);
+  }
   float2 h[kQ];
 #pragma unroll
   for (int p = 0; p < kQ; ++p) {
@@ -459,10 +467,15 @@ __device__ __forceinline__ void pair_node(const LbGeom &g, const LbPhys &ph,
     const int row = (sz * ny + sy) * wpr;
     const uint32_t w0 = __ldg(word(src, row + xw) + p * kW);
     uint32_t w = w0;
-    if (cx(p) == 1) w = __byte_perm(__ldg(word(src, row + xl) + p * kW), w0, 0x5432);   // (x - 1, x)
-    if (cx(p) == -1) w = __byte_perm(w0, __ldg(word(src, row + xr) + p * kW), 0x5432);  // (x + 1, x + 2)
+    // (x - 1, x): node nx - 1 of an odd row is the first of its word
+    if (cx(p) == 1) w = __byte_perm(__ldg(word(src, row + xl) + p * kW), w0, odd && xw == 0 ? 0x5410 : 0x5432);
+    // (x + 1, x + 2): behind the last node of an odd row comes the first one
+    if (cx(p) == -1) w = __byte_perm(w0, __ldg(word(src, row + xr) + p * kW), lone ? 0x5454 : 0x5432);
     h[p] = P::unpack(w);
   }
+  if (lone)  // padding: harmless inputs
+#pragma unroll
+    for (int p = 0; p < kQ; ++p) h[p].y = 0.f;
   if (bb.x | bb.y) {
     // halfway bounce-back: a population whose source is solid comes back as
     // the node's own post-collision opposite population

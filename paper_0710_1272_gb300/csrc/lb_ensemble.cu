@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(32 * ROWS, WARPS / ROWS)
     g.nz = d.nz;
     g.wall = d.wall;
     g.fill_solid = d.fill_solid;
+    g.pitch = d.pitch;
     g.ntx = 0;
     g.V = 0;
     g.Vp = d.Vp;

@@ -39,8 +39,9 @@ __global__ void __launch_bounds__(32 * kFluctRows, 5)
   float ha[kQ], hb[kQ];
   pull19_mask<S, I>(g, src, x, y, za, 0u, ha);
   pull19_mask<S, I>(g, src, x, y, zb, 0u, hb);
-  if (ma) bounce19<S, I>(g, src, na, ma, ha);
-  if (mb) bounce19<S, I>(g, src, nb, mb, hb);
+  const I oa = ((I)za * g.ny + y) * row_pitch<S>(g) + x, ob = ((I)zb * g.ny + y) * row_pitch<S>(g) + x;
+  if (ma) bounce19<S, I>(g, src, oa, ma, ha);
+  if (mb) bounce19<S, I>(g, src, ob, mb, hb);
   if (ma & 1u) zero19(ha);  // harmless inputs: not written
   if (mb & 1u) zero19(hb);
   float2 h[kQ];
@@ -49,12 +50,12 @@ __global__ void __launch_bounds__(32 * kFluctRows, 5)
   collide_t<Ops2, FORCING, true>(h, ph, r);
   const I st = pop_stride<S, I>((I)g.Vp);
   if (!(ma & 1u)) {
-    typename St::T *out = dst + pop_base<S, I>(na);
+    typename St::T *out = dst + pop_base<S, I>(oa);
 #pragma unroll
     for (int p = 0; p < kQ; ++p) St::store(out + (I)p * st, h[p].x);
   }
   if (zb != za && !(mb & 1u)) {
-    typename St::T *out = dst + pop_base<S, I>(nb);
+    typename St::T *out = dst + pop_base<S, I>(ob);
 #pragma unroll
     for (int p = 0; p < kQ; ++p) St::store(out + (I)p * st, h[p].y);
   }

@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock, FORCING == kForcingNone ? 
   const int y = blockIdx.y * kRowsPerBlock + threadIdx.y;
   const int z = blockIdx.z;
   if (bump != nullptr && xw == 0 && y == 0 && z == 0) bump->step += 1;
-  if (xw >= (g.nx >> 1) || y >= g.ny) return;
+  if (xw >= (g.pitch >> 1) || y >= g.ny) return;
   pair_node<T2, FORCING>(g, ph, src, dst, xw, y, z);
 }
 
@@ -47,7 +47,7 @@ template <typename T2>
 static cudaError_t lb_launch_pair(const LbGeom &g, const LbPhys &ph, const void *src, void *dst,
                                   DevStatus *bump, cudaStream_t s) {
   dim3 block(32, kRowsPerBlock);
-  dim3 grid((g.nx / 2 + 31) / 32, (g.ny + kRowsPerBlock - 1) / kRowsPerBlock, g.nz);
+  dim3 grid((g.pitch / 2 + 31) / 32, (g.ny + kRowsPerBlock - 1) / kRowsPerBlock, g.nz);
   const uint32_t *a = (const uint32_t *)src;
   uint32_t *b = (uint32_t *)dst;
   if (ph.g[0] == 0.f && ph.g[1] == 0.f && ph.g[2] == 0.f)
@@ -79,8 +79,8 @@ static cudaError_t lb_launch(const LbGeom &g, const LbPhys &ph, const void *src,
                              DevStatus *bump, cudaStream_t s) {
   // 32-bit offsets when every population index fits
   const bool small = (long long)kQ * g.Vp < 0x7fffffffLL;
-  // 16-bit storage with an even row length: two nodes per thread
-  if (small && g.nx % 2 == 0) {
+  // 16-bit storage: two nodes per thread (rows of an even length, LbGeom::pitch)
+  if (small && g.pitch % 2 == 0) {
     if (S == LBMD_STORE_F16) return lb_launch_pair<__half2>(g, ph, src, dst, bump, s);
     if (S == LBMD_STORE_BF16) return lb_launch_pair<__nv_bfloat162>(g, ph, src, dst, bump, s);
   }
@@ -176,7 +176,8 @@ __global__ void k_init(LbGeom g, float rho0, const float *rho, const float *u, f
   const int z = blockIdx.z;
   if (x >= g.nx || y >= g.ny) return;
   const size_t self = ((size_t)z * g.ny + y) * g.nx + x;
-  const size_t st = pop_stride<S, size_t>((size_t)g.Vp), at = pop_base<S, size_t>(self);
+  const size_t st = pop_stride<S, size_t>((size_t)g.Vp);
+  const size_t at = pop_base<S, size_t>(((size_t)z * g.ny + y) * row_pitch<S>(g) + x);
   if (solid_at(g.solid, g.ntx, g.ny, x, y, z)) {
 #pragma unroll
     for (int q = 0; q < kQ; ++q) St::store(dst + q * st + at, 0.f);
@@ -234,7 +235,8 @@ __global__ void k_init_local(LbGeom g, float rho0, const float *rho, const float
   const int z = z0 + blockIdx.z;
   if (x >= g.nx || y >= g.ny) return;
   const size_t self = ((size_t)z * g.ny + y) * g.nx + x;
-  const size_t st = pop_stride<S, size_t>((size_t)g.Vp), at = pop_base<S, size_t>(self);
+  const size_t st = pop_stride<S, size_t>((size_t)g.Vp);
+  const size_t at = pop_base<S, size_t>(((size_t)z * g.ny + y) * row_pitch<S>(g) + x);
   float r = rho0, ux = 0.f, uy = 0.f, uz = 0.f;
   const bool solid = solid_at(g.solid, g.ntx, g.ny, x, y, z);
   if (!solid)

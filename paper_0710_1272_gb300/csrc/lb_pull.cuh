@@ -16,16 +16,28 @@ namespace lbmd {
 // (SWAP = false, kPopPull) or at [opp(q)][y] (SWAP = true, kPopAASwap).  I is
 // the index type of the population offsets: int when 19 Vp < 2^31 (cheaper
 // address arithmetic), size_t otherwise.
+// Row length of the populations of storage S (pad: see LbGeom::pitch).
+template <int S>
+__device__ __forceinline__ int row_pitch(const LbGeom &g) {
+  return S == LBMD_STORE_F32 ? g.nx : g.pitch;
+}
+// Index of the population row-major order from that of the nodes.
+template <int S, typename I>
+__device__ __forceinline__ I pop_node(const LbGeom &g, I node) {
+  if (S == LBMD_STORE_F32 || g.pitch == g.nx) return node;
+  return node + (I)((unsigned)node / (unsigned)g.nx);  // one padding element per row
+}
+
 template <int S, typename I = size_t, bool SWAP = false>
 __device__ __forceinline__ void pull19_mask(const LbGeom &g,
                                             const typename Store<S>::T *__restrict__ src, int x,
                                             int y, int z, uint32_t bb, float h[kQ]) {
   using St = Store<S>;
-  const int nx = g.nx, ny = g.ny, nz = g.nz;
+  const int nx = g.nx, ny = g.ny, nz = g.nz, pitch = row_pitch<S>(g);
   const int xm = wrap_m1(x, nx), xp = wrap_p1(x, nx);
   const int ym = wrap_m1(y, ny), yp = wrap_p1(y, ny);
   const int zm = wrap_m1(z, nz), zp = wrap_p1(z, nz);
-  const I self = ((I)z * ny + y) * nx + x;
+  const I self = ((I)z * ny + y) * pitch + x;
   const I st = pop_stride<S, I>((I)g.Vp);
 #pragma unroll
   for (int p = 0; p < kQ; ++p) {
@@ -33,7 +45,7 @@ __device__ __forceinline__ void pull19_mask(const LbGeom &g,
     const int sx = cx(p) == 1 ? xm : (cx(p) == -1 ? xp : x);
     const int sy = cy(p) == 1 ? ym : (cy(p) == -1 ? yp : y);
     const int sz = cz(p) == 1 ? zm : (cz(p) == -1 ? zp : z);
-    const I sidx = (I)(SWAP ? opp(p) : p) * st + pop_base<S, I>(((I)sz * ny + sy) * nx + sx);
+    const I sidx = (I)(SWAP ? opp(p) : p) * st + pop_base<S, I>(((I)sz * ny + sy) * pitch + sx);
     const I bidx = (I)(SWAP ? p : opp(p)) * st + pop_base<S, I>(self);
     h[p] = St::load(src + (((bb >> p) & 1u) ? bidx : sidx));
   }
@@ -62,7 +74,8 @@ __device__ __forceinline__ bool beside_wall(const LbGeom &g, int x, int y) {
 
 // The bounce-back of pull19_mask after the fact: h holds the values of every
 // source x - c_p, solid or not; those of the solid ones (bits of `bb`) are
-// replaced by the node's own reversed populations.
+// replaced by the node's own reversed populations (self: its index in the
+// populations' rows).
 template <int S, typename I = size_t>
 __device__ __forceinline__ void bounce19(const LbGeom &g, const typename Store<S>::T *__restrict__ src,
                                          I self, uint32_t bb, float h[kQ]) {
@@ -88,8 +101,9 @@ __device__ __forceinline__ void fetch19(const LbGeom &g, const typename Store<S>
   using St = Store<S>;
   const I self = ((I)z * g.ny + y) * g.nx + x;
   if (mode == kPopAALocal) {
+    const I own = ((I)z * g.ny + y) * row_pitch<S>(g) + x;
 #pragma unroll
-    for (int p = 0; p < kQ; ++p) h[p] = St::load(src + (I)p * pop_stride<S, I>((I)g.Vp) + pop_base<S, I>(self));
+    for (int p = 0; p < kQ; ++p) h[p] = St::load(src + (I)p * pop_stride<S, I>((I)g.Vp) + pop_base<S, I>(own));
     return;
   }
   const uint32_t bb = tile_is_near(g, x, y, z) ? __ldg(&g.lmask[self]) : 0u;

@@ -41,6 +41,14 @@ Layout make_layout(const lbmd_params &p, bool single_box);
 size_t stage_floats_for(const lbmd_params &p);
 long long chunk_cells_for(const lbmd_params &p);
 
+// Row length of the populations: 16-bit ones start every row at a word, so that
+// two x-adjacent nodes share one whatever the box (not where the padding would
+// take the offsets beyond 32 bits).
+inline int pop_pitch(const lbmd_params &p) {
+  const int even = p.nx + (p.nx & 1);
+  const bool fits = 19LL * ((long long)even * p.ny * p.nz + 64) < 0x7fffffffLL;
+  return p.storage == LBMD_STORE_F32 || !fits ? p.nx : even;
+}
 // LbGeom::fill_solid of a box stepped with `traffic` bytes of populations per
 // step: beyond the 129 MB L2, and a wall of up to a sector's eight floats.
 inline int fill_solid(const lbmd_params &p, size_t traffic) {

@@ -55,9 +55,11 @@ struct LbGeom {
   WallGeom wall;
   int fill_solid;               // stream-collides write zeros to solid nodes: a thin
                                 // wall in a box beyond the L2 cache
+  int pitch;                    // row length of the populations: nx, or nx + 1 if nx
+                                // is odd and they are held in 16 bits
   int ntx;                      // x-tiles of 32 nodes = words per bitfield row
   long long V;                  // nx * ny * nz
-  long long Vp;                 // population stride (V rounded up to 64)
+  long long Vp;                 // population stride (pitch * ny * nz rounded up to 64)
   const uint32_t *solid;        // [nz][ny][ntx] words, bit x & 31 of word x >> 5
   const uint8_t *tile_near;     // [nz][ny][ntx]: 1 if a solid node is within one
                                 // node of the tile's 32 cells (incl. themselves)
@@ -159,6 +161,7 @@ struct __align__(16) EnsLb {
   int nx, ny, nz;
   WallGeom wall;
   int fill_solid;               // as LbGeom's, for the realisations together
+  int pitch;                    // as LbGeom's
   int Vp;                       // population stride (19 Vp < 2^31)
   float inv_nx;                 // 1 / nx, for the row of a node in its plane
   float omega, rho0;

@@ -1383,7 +1383,7 @@ __global__ void __launch_bounds__(256)
     if (node < 0) return;  // not an owner
     F = F3{v.x, v.y, v.z};
   }
-  const size_t st = pop_stride<S, size_t>((size_t)g.Vp), own = pop_base<S, size_t>((size_t)node);
+  const size_t st = pop_stride<S, size_t>((size_t)g.Vp), own = pop_base<S, size_t>(pop_node<S, size_t>(g, (size_t)node));
   uint32_t bb = 0u;
   int x = 0, y = 0, z = 0;
   if (mode == kPopAALocal) {
@@ -1397,7 +1397,7 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
   for (int p = 1; p < kQ; ++p) {
     if (mode == kPopAALocal) {
-      const size_t t = ((size_t)wrapi(z + cz(p), g.nz) * g.ny + wrapi(y + cy(p), g.ny)) * g.nx +
+      const size_t t = ((size_t)wrapi(z + cz(p), g.nz) * g.ny + wrapi(y + cy(p), g.ny)) * row_pitch<S>(g) +
                        wrapi(x + cx(p), g.nx);
       at[p] = ((bb >> opp(p)) & 1u) ? (size_t)opp(p) * st + own : (size_t)p * st + pop_base<S, size_t>(t);
     } else {
@@ -1483,7 +1483,8 @@ __global__ void __launch_bounds__(256)
     if (node >= 0 && a.owner[node] == e2) {  // the owner converts its node's sum
       const F3 F = spread_take(a, node, e2);
       const size_t st = pop_stride<S, size_t>((size_t)a.geo.Vp);
-      typename St::T *dst = (typename St::T *)mem[mi.x].pop[cur ^ 1] + pop_base<S, size_t>((size_t)node);
+      typename St::T *dst = (typename St::T *)mem[mi.x].pop[cur ^ 1] +
+                              pop_base<S, size_t>(pop_node<S, size_t>(a.geo, (size_t)node));
       if (S == LBMD_STORE_F32) {
 #pragma unroll
         for (int p = 1; p < kQ; ++p)
