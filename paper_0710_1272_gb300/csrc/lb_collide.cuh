@@ -435,10 +435,11 @@ template <> struct Pair16<__nv_bfloat162> {
   }
 };
 
-template <typename T2, int FORCING>
-__device__ __forceinline__ void pair_node(const LbGeom &g, const LbPhys &ph,
-                                          const uint32_t *__restrict__ src,
-                                          uint32_t *__restrict__ dst, int xw, int y, int z) {
+// pair_pull: the pre-collision deviations h of both nodes (zero for a solid one
+// and for padding); returns their link masks.
+template <typename T2>
+__device__ __forceinline__ uint2 pair_pull(const LbGeom &g, const uint32_t *__restrict__ src, int xw,
+                                           int y, int z, float2 h[kQ]) {
   using P = Pair16<T2>;
   const int wpr = g.pitch >> 1;  // words per row
   const bool odd = g.nx & 1, lone = odd && xw == wpr - 1;
@@ -458,7 +459,6 @@ __device__ __forceinline__ void pair_node(const LbGeom &g, const LbPhys &ph,
     bb.x = __ldg(m);
     if (!lone) bb.y = __ldg(m + 1);
   }
-  float2 h[kQ];
 #pragma unroll
   for (int p = 0; p < kQ; ++p) {
     // source row of x - c_p; the pair's sources are x - c_x, x - c_x + 1
@@ -496,6 +496,18 @@ __device__ __forceinline__ void pair_node(const LbGeom &g, const LbPhys &ph,
 #pragma unroll
       for (int p = 0; p < kQ; ++p) h[p].y = 0.f;
   }
+  return bb;
+}
+
+template <typename T2, int FORCING>
+__device__ __forceinline__ void pair_node(const LbGeom &g, const LbPhys &ph,
+                                          const uint32_t *__restrict__ src,
+                                          uint32_t *__restrict__ dst, int xw, int y, int z) {
+  using P = Pair16<T2>;
+  constexpr int kW = kBlockNodes / 2;
+  float2 h[kQ];
+  const uint2 bb = pair_pull<T2>(g, src, xw, y, z, h);
+  const int self = (z * g.ny + y) * (g.pitch >> 1) + xw;
   collide_t<Ops2, FORCING>(h, ph);
   if ((bb.x | bb.y) & 1u) {
     if (bb.x & 1u)

@@ -54,3 +54,23 @@ def _compare(p, storage, tol, streaming):
     m = o != 0
     assert np.all(f[~m] == 0)
     assert np.max(np.abs(f[m] - o[m]) / np.abs(o[m])) < tol
+
+
+@pytest.mark.parametrize("nx,offset", [(32, 0), (32, 1), (33, 0), (33, 1)])
+def test_population_readout_alignment(nx, offset):
+    """Paired 8-byte stores only where the row length and the caller's memory
+    allow them: the same values wherever the caller wants them."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_0710_1272_gb300 as lb
+    p = dict(nx=nx, ny=5, nz=3, wall_x=16, pore_d=3, storage="f16", init_tg_amp=0.02)
+    sim = lb.Simulation(p)
+    sim.step(2)
+    n = 19 * nx * 5 * 3
+    buf = torch.full((n + 3,), 7.0, dtype=torch.float32, device="cuda")
+    lb.lbmd_read_populations(sim.ctx, buf[offset:].data_ptr(), 1)
+    torch.cuda.synchronize()
+    got = buf.cpu().numpy()
+    assert np.array_equal(got[offset:offset + n].reshape(19, 3, 5, nx), sim.populations())
+    assert np.all(got[:offset] == 7.0) and np.all(got[offset + n:] == 7.0)
