@@ -43,21 +43,27 @@ __device__ __forceinline__ F3 operator-(F3 a, F3 b) { return F3{a.x - b.x, a.y -
 __device__ __forceinline__ F3 operator*(float s, F3 a) { return F3{s * a.x, s * a.y, s * a.z}; }
 __device__ __forceinline__ float dot(F3 a, F3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
 
-// Threads of the MD block: one per bead in whole warps, at least three warps
-// (they share the evaluation of the force list), and one more warp for the
-// tridiagonal solves where the block's register class (512, 768 or 1024
-// threads: 128, 80 or 64 registers) has room for it; else warp 0 solves beside
-// its beads.
-__host__ __device__ inline int bead_threads(int N) { return max((N + 31) / 32 * 32, 96); }
+// Threads of the MD block: one per bead in whole warps; for chains of up to 224
+// beads warps that only evaluate the force list (two for up to 32 beads, else
+// eight), beside the bead warps' own work; and one more warp for the tridiagonal
+// solves where the block's register class (512, 768 or 1024 threads: 128, 80
+// or 64 registers) has room for it, else warp 0 solves beside its beads.
+__host__ __device__ inline int bead_threads(int N) { return (N + 31) / 32 * 32; }
 int md_threads(int N) {
-  const int t = bead_threads(N);
+  int t = bead_threads(N);
+  if (t <= 32)
+    t += 64;
+  else if (t <= 224)
+    t += 256;
   return t == 512 || t == 768 || t == LBMD_MAX_BEADS ? t : t + 32;
 }
 // The block of an ensemble's chains: sizes in steps of 64 threads up to 512,
 // then the register classes, so that few launches take chains of every length
-// (nine at most; warps without beads wait at the barriers).
+// (nine at most; the warps to spare evaluate the force list), and small, so that
+// several chains share an SM and leave registers to the stream-collide.
 int md_group_threads(int N) {
-  const int t = md_threads(N);
+  const int b = bead_threads(N) < 96 ? 96 : bead_threads(N);
+  const int t = b == 512 || b == 768 || b == LBMD_MAX_BEADS ? b : b + 32;
   return t <= 512 ? (t + 63) / 64 * 64 : t <= 768 ? 768 : LBMD_MAX_BEADS;
 }
 
@@ -354,66 +360,62 @@ __device__ __forceinline__ void block_sum(float (&v)[K], float *red) {
   for (int k = 0; k < K; ++k) v[k] = red[32 * K + k];
 }
 
-// Solid node test from the Sec. III geometry itself (the wall layers
-// wall_x .. wall_x + wall_t - 1 minus the d x d pore, and the rows y = 0 and
-// y = ny - 1 with y-walls): the rule the solid bitfield is built from, with
-// no memory read.  Coordinates inside the box.
-__device__ __forceinline__ bool wall_layer(const ChainArgs &a, int x) {
-  int dx = x - a.wall_x;
-  if (dx < 0) dx += a.geo.nx;
-  return a.has_wall && dx < a.wall_t;
-}
-__device__ __forceinline__ bool solid_geom(const ChainArgs &a, int x, int y, int z) {
-  if (a.y_walls && (y == 0 || y == a.geo.ny - 1)) return true;
-  if (!wall_layer(a, x)) return false;
-  return !(a.pore_d > 0 && y >= a.pore_y0 && y < a.pore_y0 + a.pore_d && z >= a.pore_z0 &&
-           z < a.pore_z0 + a.pore_d);
-}
-
 // Solid nodes around a bead within `radius` (node offsets n with
-// |n - s| < radius per axis).  For each solid node calls fn(node coordinate in
-// the chain's local frame).
+// |n - s| < radius per axis), from the Sec. III geometry itself (the wall layers
+// minus the pore, and the rows y = 0 and y = ny - 1 with y-walls): the rule the
+// solid bitfield is built from, with no memory read.  For each solid node calls
+// fn(node coordinate in the chain's local frame).
+//
+// Two things once made it 56-73 k, then 36 k cycles a list build (N = 20 to
+// 700), now 12 k.  Stepping through the x offsets had the lanes of a
+// warp reach the wall's layer at different steps, one scan of it behind the
+// other: without y-walls each layer is looked up.  And `a` may live in kernel
+// parameters read through a pointer here, again after every store of fn: all
+// that is needed of it is copied first.
 template <typename Fn>
 __device__ __forceinline__ void for_solid_nodes(const ChainArgs &a, float4 rh, float4 rl,
                                                 float radius, Fn fn) {
-  const LbGeom &g = a.geo;
-  if (!a.has_wall && !a.y_walls) return;
-  int c[3];
-  float sf[3];
-  cell_frac_hl(rh.x, rl.x, a.ox, g.nx, c[0], sf[0]);
-  const int lo0 = (int)ceilf(sf[0] - radius), hi0 = (int)floorf(sf[0] + radius);
+  const int nx = a.geo.nx, ny = a.geo.ny, nz = a.geo.nz, wall_x = a.wall_x, wall_t = a.wall_t;
+  const int py0 = a.pore_y0, pz0 = a.pore_z0, pd = a.pore_d, oy0 = a.oy, oz0 = a.oz;
+  const bool has_wall = a.has_wall, y_walls = a.y_walls;
+  if (!has_wall && !y_walls) return;
+  int cx0, cy0 = 0, cz0 = 0;
+  float sx, sy = 0.f, sz = 0.f;
+  cell_frac_hl(rh.x, rl.x, a.ox, nx, cx0, sx);
+  const int lo0 = (int)ceilf(sx - radius), hi0 = (int)floorf(sx + radius);
   const float fx = floorf(rh.x), fy = floorf(rh.y), fz = floorf(rh.z);
-  // Without y-walls only the wall layers hold solid nodes: each layer is met
-  // at one offset (the box is wider than the stencil), which is looked up.
-  // Stepping through the offsets instead had the lanes of a warp reach the
-  // layer at different steps, one scan of it behind the other (56-73 k cycles
-  // a list build, against 7 k).
-  const bool layers = !a.y_walls && g.nx > 2 * ((int)radius + 2) + a.wall_t;
-  const int steps = layers ? a.wall_t : hi0 - lo0 + 1;
+  // each layer is met at one offset where the box is wider than the stencil
+  const bool layers = !y_walls && nx > 2 * ((int)radius + 2) + wall_t;
+  const int steps = layers ? wall_t : hi0 - lo0 + 1;
   bool ready = false;
   int lo1 = 0, hi1 = 0, lo2 = 0, hi2 = 0;
   for (int k = 0; k < steps; ++k) {
     int ox = lo0 + k;
     if (layers) {
-      ox = a.wall_x + k - c[0];
-      if (ox < lo0) ox += g.nx;
-      if (ox > hi0) ox -= g.nx;
+      ox = wall_x + k - cx0;
+      if (ox < lo0) ox += nx;
+      if (ox > hi0) ox -= nx;
       if (ox < lo0 || ox > hi0) continue;
     }
-    const int x = wrap_near(c[0] + ox, g.nx);
-    if (!a.y_walls && !wall_layer(a, x)) continue;  // no solid node in this layer
+    int dx = wrap_near(cx0 + ox, nx) - wall_x;
+    if (dx < 0) dx += nx;
+    const bool layer = has_wall && dx < wall_t;
+    if (!y_walls && !layer) continue;  // no solid node in this layer
     if (!ready) {  // few beads get here
       ready = true;
-      cell_frac_hl(rh.y, rl.y, a.oy, g.ny, c[1], sf[1]);
-      cell_frac_hl(rh.z, rl.z, a.oz, g.nz, c[2], sf[2]);
-      lo1 = (int)ceilf(sf[1] - radius), hi1 = (int)floorf(sf[1] + radius);
-      lo2 = (int)ceilf(sf[2] - radius), hi2 = (int)floorf(sf[2] + radius);
+      cell_frac_hl(rh.y, rl.y, oy0, ny, cy0, sy);
+      cell_frac_hl(rh.z, rl.z, oz0, nz, cz0, sz);
+      lo1 = (int)ceilf(sy - radius), hi1 = (int)floorf(sy + radius);
+      lo2 = (int)ceilf(sz - radius), hi2 = (int)floorf(sz + radius);
     }
     for (int oy = lo1; oy <= hi1; ++oy) {
-      const int y = wrap_near(c[1] + oy, g.ny);
+      const int y = wrap_near(cy0 + oy, ny);
+      const bool row = y_walls && (y == 0 || y == ny - 1);
+      const bool open_y = pd > 0 && y >= py0 && y < py0 + pd;
+      if (!row && !layer) continue;
       for (int oz = lo2; oz <= hi2; ++oz) {
-        const int z = wrap_near(c[2] + oz, g.nz);
-        if (!solid_geom(a, x, y, z)) continue;
+        const int z = wrap_near(cz0 + oz, nz);
+        if (!row && open_y && z >= pz0 && z < pz0 + pd) continue;  // the pore
         fn(make_float4(fx + (float)ox, fy + (float)oy, fz + (float)oz, 0.f));
       }
     }
@@ -476,55 +478,50 @@ __device__ __forceinline__ bool fits_short(float4 n) {
 //
 // With a list per bead the chain waited for its fullest one (a bead in the
 // pore: ~25 entries at ~200-290 cycles each, 3.5-5 k cycles of every substep).
-// Spread over the block, two entries at a time.  The low parts of the positions
-// are read only near the cutoff: they change a separation by no more than 0.1
-// while the local coordinates stay below 1e6.
+// Spread over the block, two entries at a time and without a branch on the
+// cutoff, whose latencies would follow one another (400 beads: 2.7 k cycles with
+// the branch, 1.6 k without; 20 beads 1.3 and 0.8 k).
 __device__ __forceinline__ void eval_items(const ChainArgs &a, const uint2 *s_item, int n, int who,
                                            int of, const float4 *s_rh, const float4 *s_rl, float4 *s_f,
                                            unsigned *s_mask) {
   const float sig2 = a.sigma * a.sigma;
-  const float rc = kTwoSixth * a.sigma, rc2 = rc * rc, reach2 = (rc + 0.2f) * (rc + 0.2f);
+  const float rc = kTwoSixth * a.sigma, rc2 = rc * rc;
   const float eps24 = 24.0f * a.eps;
 #pragma unroll 1
   for (int q0 = who; q0 < n; q0 += 2 * of) {
     uint2 it[2];
-    float4 rh[2], oh[2];
+    float4 rh[2], rl[2], oh[2], ol[2];
     it[0] = s_item[q0];
     it[1] = s_item[min(q0 + of, n - 1)];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       const int i = it[k].x & (LBMD_MAX_BEADS - 1);
+      const int j = (it[k].x & kItemWall) ? i : (int)(it[k].y & (LBMD_MAX_BEADS - 1));
       rh[k] = s_rh[i];
-      oh[k] = s_rh[(it[k].x & kItemWall) ? i : (int)(it[k].y & (LBMD_MAX_BEADS - 1))];
+      rl[k] = s_rl[i];
+      oh[k] = s_rh[j];
+      ol[k] = s_rl[j];
     }
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       const int q = q0 + k * of;
-      const bool wall = (it[k].x & kItemWall) != 0;
-      const unsigned bit = (it[k].x >> 10) & 31u;
-      if (wall) {
-        oh[k].x = (float)((int)it[k].x >> 16);
-        oh[k].y = (float)(short)(it[k].y & 0xffffu);
-        oh[k].z = (float)((int)it[k].y >> 16);
-      }
-      F3 d{rh[k].x - oh[k].x, rh[k].y - oh[k].y, rh[k].z - oh[k].z};
+      const bool wall = (it[k].x & kItemWall) != 0, tail = (it[k].x >> 10 & 31u) == kItemTail;
       const bool image = !wall && (it[k].y & kItemImage) != 0;
-      if (q < n && (dot(d, d) < reach2 || image || bit == kItemTail)) {
-        const int i = it[k].x & (LBMD_MAX_BEADS - 1);
-        const float4 rl = s_rl[i];
-        float4 ol = s_rl[wall ? i : (int)(it[k].y & (LBMD_MAX_BEADS - 1))];
-        if (wall) ol = make_float4(0.f, 0.f, 0.f, 0.f);
-        d = diff_hl(rh[k], rl, oh[k], ol);
-        if (image) d = min_image(a.geo, d);
-        const float r2 = dot(d, d);
-        const bool in = r2 < rc2;
-        const float ir2 = rcp_newton(r2);
-        const float sr2 = sig2 * ir2;
-        const float sr6 = sr2 * sr2 * sr2;
-        const float f = eps24 * (2.0f * sr6 * sr6 - sr6) * ir2;
-        if (in || bit == kItemTail) s_f[q] = in ? f4(f * d) : make_float4(0.f, 0.f, 0.f, 0.f);
-        if (in && bit != kItemTail) atomicOr(&s_mask[i], 1u << bit);
+      if (wall) {
+        oh[k] = make_float4((float)((int)it[k].x >> 16), (float)(short)(it[k].y & 0xffffu),
+                            (float)((int)it[k].y >> 16), 0.f);
+        ol[k] = make_float4(0.f, 0.f, 0.f, 0.f);
       }
+      F3 d = diff_hl(rh[k], rl[k], oh[k], ol[k]);
+      if (image) d = min_image(a.geo, d);
+      const float r2 = dot(d, d);
+      const bool in = q < n && r2 < rc2;
+      const float ir2 = rcp_newton(r2);
+      const float sr2 = sig2 * ir2;
+      const float sr6 = sr2 * sr2 * sr2;
+      const float f = eps24 * (2.0f * sr6 * sr6 - sr6) * ir2;
+      if (in || (tail && q < n)) s_f[q] = in ? f4(f * d) : make_float4(0.f, 0.f, 0.f, 0.f);
+      if (in && !tail) atomicOr(&s_mask[it[k].x & (LBMD_MAX_BEADS - 1)], 1u << (it[k].x >> 10 & 31u));
     }
   }
 }
@@ -577,6 +574,8 @@ __device__ __noinline__ int build_lists(const ChainArgs &a, int i, bool bead, fl
   __syncthreads();
   short *G = a.nl_list + (size_t)i * kMaxPairs;
   float4 *W = a.wl_list + (size_t)i * kMaxWall;
+  uint2 *items = a.items;
+  const int reach = a.has_bonds ? 1 : 0;
   int np = 0, nw = 0;
   // a pair of the list moves by at most two half skins until the next
   // rebuild: within this box width it keeps the image it has now
@@ -603,7 +602,7 @@ __device__ __noinline__ int build_lists(const ChainArgs &a, int i, bool bead, fl
         if (dot(d, d) < rl2) mask |= 1u << jj;
       }
       // not the bead itself, nor its bonded neighbours
-      const int own = i - j0, reach = a.has_bonds ? 1 : 0;
+      const int own = i - j0;
       for (int k = own - reach; k <= own + reach; ++k)
         if (k >= 0 && k < 32) mask &= ~(1u << k);
       if (!bead) mask = 0u;
@@ -655,7 +654,7 @@ __device__ __noinline__ int build_lists(const ChainArgs &a, int i, bool bead, fl
     const auto tag = [&](int e) { return (unsigned)i | min((unsigned)e, kItemTail) << 10; };
     const auto put = [&](int e, uint2 it) {
       s_item[q + e] = it;
-      a.items[q + e] = it;
+      items[q + e] = it;
     };
     // read back what this thread has just written, in wide or several loads
     for (int k0 = 0; k0 < np; k0 += 8) {
@@ -792,10 +791,14 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
   const int N = a.N;
   const int i = threadIdx.x;  // bead of this thread
   const bool bead = i < N;
-  // the warp of the tridiagonal solves: the one after the beads', or the first
-  // of a block without a spare one
+  // the warp of the tridiagonal solves: the last one, or the first of a block
+  // without a spare one; the threads that evaluate the force list: those
+  // between the beads' and the solve's, where there are two warps of them and
+  // the chain is short, else all but the solve's
   const bool spare = (int)blockDim.x > bead_threads(N);
-  const bool solves = (i >> 5) == (spare ? bead_threads(N) >> 5 : 0);
+  const int workers = spare ? (int)blockDim.x - 32 : (int)blockDim.x;
+  const bool solves = (i >> 5) == (spare ? workers >> 5 : 0);
+  const int eval0 = N <= 224 && workers - bead_threads(N) >= 64 ? bead_threads(N) : 0;
   const int rows = 32 * solve_rows(N);
   float4 *s_row = smem4;         // rows of the tridiagonal system to solve
   float4 *s_full = s_row + rows; // halved rows: the whole system, two buffers
@@ -917,9 +920,8 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
   float4 xi = make_float4(0.f, 0.f, 0.f, 0.f);
   F3 Fp{0.f, 0.f, 0.f};
   auto prepare = [&](int k) {
-    if (lists && nl_ok == kNlFlat && (!spare || i < bead_threads(N)))
-      eval_items(a, s_item, n_items, i, spare ? bead_threads(N) : (int)blockDim.x, s_rh, s_rl, s_f,
-                 s_mask);
+    if (lists && nl_ok == kNlFlat && i >= eval0 && i < workers)
+      eval_items(a, s_item, n_items, i - eval0, workers - eval0, s_rh, s_rl, s_f, s_mask);
     if (!bead) return;
     xi = a.noise[(size_t)k * N + i];  // this thread wrote it
     F3 sb{0.f, 0.f, 0.f};
