@@ -134,20 +134,4 @@ __device__ __forceinline__ float uniform23(uint32_t x) {
   return (float)(x >> 9) * (1.0f / 8388608.0f) + (0.5f / 8388608.0f);
 }
 
-// Three standard normals for (bead, LB step, substep, stream): Box-Muller on
-// the four uniforms of one Philox block.
-__device__ __forceinline__ float3 gauss3(uint64_t seed, uint32_t bead, int64_t step,
-                                         uint32_t substep, uint32_t stream) {
-  U4 c{bead, (uint32_t)(uint64_t)step, (uint32_t)((uint64_t)step >> 32),
-       (substep & 0xFFu) | (stream << 8)};
-  U4 r = philox4x32_10(c, (uint32_t)seed, (uint32_t)(seed >> 32));
-  const float u1 = uniform23(r.x), u2 = uniform23(r.y);
-  const float u3 = uniform23(r.z), u4 = uniform23(r.w);
-  const float r1 = sqrtf(-2.0f * logf(u1)), r2 = sqrtf(-2.0f * logf(u3));
-  float s2, c2, s4, c4;
-  sincospif(2.0f * u2, &s2, &c2);
-  sincospif(2.0f * u4, &s4, &c4);
-  return make_float3(r1 * c2, r1 * s2, r2 * c4);
-}
-
 }  // namespace lbmd
