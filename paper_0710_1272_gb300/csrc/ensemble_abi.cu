@@ -29,10 +29,11 @@ constexpr int kEnsBlock = 16;   // steps per long graph
 const int kEnsGraphSteps[3] = {1, 2, kEnsBlock};
 
 struct EnsLayout {
-  size_t mem, lbd, tiles, n_tiles, beads, live, cap, chains, status, stage;
+  size_t mem, lbd, tiles, n_tiles, beads, live, cap, chains, status, rec, stage;
   size_t stage_floats;
   size_t max_tiles;  // tile capacity (rows = 4, every realisation)
   int nb;            // padded bead slots
+  bool lb_sets;      // the stream-collide sets the step (!spread_take_in_apply)
   std::vector<size_t> off;   // workspace offset of each realisation
   std::vector<Layout> L;
   size_t total;
@@ -83,11 +84,14 @@ EnsLayout make_ens_layout(const lbmd_params *m, int32_t count) {
   E.max_tiles = 0;
   E.nb = 0;
   E.stage_floats = 0;
+  long long nodes = 0;
   for (int k = 0; k < count; ++k) {
     E.max_tiles += tiles_of(m[k], 4);
     E.nb += (m[k].n_beads + 3) / 4 * 4;
     E.stage_floats = std::max(E.stage_floats, stage_floats_for(m[k]));
+    nodes += (long long)m[k].nx * m[k].ny * m[k].nz;
   }
+  E.lb_sets = !m[0].solvent_free && !spread_take_in_apply(m[0].storage, nodes);
   E.mem = take((size_t)count * sizeof(EnsMember));
   E.lbd = take((size_t)count * sizeof(EnsLb));
   E.tiles = take(std::max<size_t>(E.max_tiles, 1) * sizeof(EnsTile));
@@ -97,6 +101,7 @@ EnsLayout make_ens_layout(const lbmd_params *m, int32_t count) {
   E.cap = take(sizeof(long long));
   E.chains = take((size_t)count * sizeof(int));
   E.status = take((size_t)count * sizeof(DevStatus));
+  E.rec = E.lb_sets ? take(8 * (size_t)E.nb * sizeof(float4)) : 0;
   E.stage = take(E.stage_floats * sizeof(float));
   E.off.resize(count);
   E.L.resize(count);
@@ -129,6 +134,7 @@ struct lbmd_ensemble {
   int *d_n_tiles, *d_live, *d_chains;
   int2 *d_beads;
   long long *d_cap;
+  float4 *d_rec;        // [8 nb] apply records where the stream-collide sets the step, else null
   DevStatus *d_status;  // [count] the realisations' status words, gathered for a read-out
   float *stage;
   int rows, warps, claim, cpt, grid, sms;
@@ -286,12 +292,19 @@ cudaError_t enqueue_ens_step(lbmd_ensemble *e, int cur) {
   const int *live = e->d_live + cur * e->count;
   int *live_next = e->d_live + (cur ^ 1) * e->count;
   if (t[0] && (err = cudaEventRecord(t[0], e->own)) != cudaSuccess) return err;
+  // Where the stream-collide sets the step it starts at once, the gather beside
+  // it; where the MD groups do, the gather runs first.
+  const bool aside = e->E.lb_sets;
+  if (aside) {
+    if ((err = cudaEventRecord(e->ev_join[0], e->own)) != cudaSuccess) return err;
+    if ((err = cudaStreamWaitEvent(e->side[0], e->ev_join[0], 0)) != cudaSuccess) return err;
+  }
+  cudaStream_t first = aside ? e->side[0] : e->own;
   if (!e->solvent_free &&
-      (err = launch_ens_gather(e->storage, e->d_mem, e->d_beads, e->E.nb, live, cur,
-                               e->own)) != cudaSuccess)
+      (err = launch_ens_gather(e->storage, e->d_mem, e->d_beads, e->E.nb, live, cur, first)) != cudaSuccess)
     return err;
-  if ((err = cudaEventRecord(e->ev_fork, e->own)) != cudaSuccess) return err;
-  for (int s = 0; s < e->nside; ++s)
+  if ((err = cudaEventRecord(e->ev_fork, first)) != cudaSuccess) return err;
+  for (int s = aside ? 1 : 0; s < e->nside; ++s)
     if ((err = cudaStreamWaitEvent(e->side[s], e->ev_fork, 0)) != cudaSuccess) return err;
   for (size_t k = 0; k < e->groups.size(); ++k) {
     const Group &g = e->groups[k];
@@ -313,7 +326,7 @@ cudaError_t enqueue_ens_step(lbmd_ensemble *e, int cur) {
       if ((err = cudaEventRecord(e->ev_join[s], e->side[s])) != cudaSuccess) return err;
       if ((err = cudaStreamWaitEvent(e->side[0], e->ev_join[s], 0)) != cudaSuccess) return err;
     }
-    if ((err = launch_ens_spread_accum(e->d_mem, e->d_beads, e->E.nb, live, e->side[0])) !=
+    if ((err = launch_ens_spread_sum(e->d_mem, e->d_beads, e->E.nb, live, e->d_rec, e->side[0])) !=
         cudaSuccess)
       return err;
   }
@@ -322,7 +335,7 @@ cudaError_t enqueue_ens_step(lbmd_ensemble *e, int cur) {
     if ((err = cudaStreamWaitEvent(e->own, e->ev_join[s], 0)) != cudaSuccess) return err;
   }
   if ((err = launch_ens_spread(e->storage, e->d_mem, e->d_beads, e->E.nb, live, live_next, cur,
-                               e->d_cap, e->own)) != cudaSuccess)
+                               e->d_cap, e->d_rec, e->own)) != cudaSuccess)
     return err;
   if (t[3] && (err = cudaEventRecord(t[3], e->own)) != cudaSuccess) return err;
   return cudaSuccess;
@@ -461,6 +474,7 @@ int lbmd_ensemble_create(const lbmd_params *members, int32_t count, void *dev_wo
   e->d_beads = (int2 *)(e->ws + E.beads);
   e->d_live = (int *)(e->ws + E.live);
   e->d_cap = (long long *)(e->ws + E.cap);
+  e->d_rec = E.lb_sets ? (float4 *)(e->ws + E.rec) : nullptr;
   e->d_status = (DevStatus *)(e->ws + E.status);
   e->d_chains = (int *)(e->ws + E.chains);
   e->stage = (float *)(e->ws + E.stage);

@@ -244,17 +244,17 @@ cudaError_t launch_md_cycle(const ChainArgs &a, int priority, bool beside, cudaS
 // SMs (global atomics from one SM, in the MD block, were slow while the
 // stream-collide saturates HBM).  launch_spread_sum enqueues the sum as two
 // kernels, or only the first when the apply converts the sums itself
-// (records == false); an ensemble uses launch_ens_spread_accum and converts
-// in its apply.
+// (records == false); launch_ens_spread_sum does so for an ensemble.
 constexpr int kOwnerFree = 0x7f7f7f7f;
 cudaError_t launch_spread_sum(const ChainArgs &a, bool records, cudaStream_t s);
-// Single box: true when the apply should convert the sums itself (the MD
-// branch sets the step), false when the stream-collide sets it -- taken as a
-// stream-collide moving 240 MB or more per step (~40 us at the HBM rate, about
-// the MD branch of a 400-bead chain beside it).  The gather follows the same
-// rule (enqueue_step).  Step of a 400-bead chain, us, true against false:
-// 144x80x80 FP32 (140 MB) 47.7 / 54.5, FP16 44.2 / 47.1; 256x128x128 FP16
-// (318 MB) 73.3 / 69.1, FP32 (637 MB) 105.3 / 101.6.
+// True when the apply should convert the sums itself (the MD branch sets the
+// step), false when the stream-collide sets it -- taken as a stream-collide
+// moving 240 MB or more per step (~40 us at the HBM rate, about the MD branch of
+// a 400-bead chain beside it).  The gather follows the same rule (enqueue_step);
+// so does an ensemble, by the nodes of all its boxes.  Step of a 400-bead chain,
+// us, true against false: 144x80x80 FP32 (140 MB) 47.7 / 54.5, FP16 44.2 / 47.1;
+// 256x128x128 FP16 (318 MB) 73.3 / 69.1, FP32 (637 MB) 105.3 / 101.6; of an
+// ensemble of 32 chains of 120 - 400 beads, FP16 (764 MB): 194.6 / 191.0.
 inline bool spread_take_in_apply(int storage, long long nodes) {
   const long long bytes = 2LL * 19 * nodes * (storage == LBMD_STORE_F32 ? 4 : 2);
   return bytes < 240000000LL;
@@ -290,16 +290,17 @@ cudaError_t launch_ens_gather(int storage, const EnsMember *mem, const int2 *bea
 // threads each, with dynamic shared memory for `max_n` beads.
 cudaError_t launch_ens_md_cycle(const EnsMember *mem, const int *chains, int count, int threads,
                                 int max_n, const int *live, int priority, cudaStream_t s);
-// Sum part of the spread of every live realisation (after every MD group).
-cudaError_t launch_ens_spread_accum(const EnsMember *mem, const int2 *beads, int nb,
-                                    const int *live, cudaStream_t s);
-// Apply part of the spread (the owners convert their sums) into pop[1 - cur];
-// bumps each live realisation's step
+// Sum part of the spread of every live realisation (after every MD group); with
+// `rec` ([8 nb], or null) the owners' forces are converted to records there.
+cudaError_t launch_ens_spread_sum(const EnsMember *mem, const int2 *beads, int nb, const int *live,
+                                  float4 *rec, cudaStream_t s);
+// Apply part of the spread (from the records, or the owners convert their sums
+// if `rec` is null) into pop[1 - cur]; bumps each live realisation's step
 // count and writes its flag for the next step into `live_next` (still running
 // and step < *max_steps).
 cudaError_t launch_ens_spread(int storage, const EnsMember *mem, const int2 *beads, int nb,
                               const int *live, int *live_next, int cur,
-                              const long long *max_steps, cudaStream_t s);
+                              const long long *max_steps, const float4 *rec, cudaStream_t s);
 
 cudaError_t launch_read_beads(const float4 *pos, const float4 *pos_lo, const float4 *vel, int N,
                               int ox, int oy, int oz, double *dpos, double *dvel, cudaStream_t s);

@@ -762,14 +762,14 @@ __device__ __forceinline__ F3 spread_take(const ChainArgs &a, int node, int e) {
 
 // After every contribution is summed: entry e's record for the apply --
 // (F, node) if e owns its node, node = -1 otherwise.
-__device__ __forceinline__ void spread_finalize(const ChainArgs &a, int e) {
+__device__ __forceinline__ float4 spread_record(const ChainArgs &a, int e) {
   const int node = a.sp_node[e];
   float4 out = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
   if (node >= 0 && a.owner[node] == e) {
     const F3 F = spread_take(a, node, e);
     out = make_float4(F.x, F.y, F.z, __int_as_float(node));
   }
-  a.sp_src[e] = out;
+  return out;
 }
 
 // Three standard normals for (bead, LB step, substep): Box-Muller on the four
@@ -1359,7 +1359,7 @@ __global__ void __launch_bounds__(256) k_spread_finalize(ChainArgs a) {
   asm volatile("griddepcontrol.wait;" ::: "memory");  // every share
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= 8 * a.N) return;
-  spread_finalize(a, e);
+  a.sp_src[e] = spread_record(a, e);
 }
 
 // (3) extrapolation of the forces: node x_k receives -sum_i w_ik J_i as the
@@ -1372,7 +1372,7 @@ __global__ void __launch_bounds__(256) k_spread_finalize(ChainArgs a) {
 // the 18 words first and writes each rounded once.  The owner's force comes
 // from its record sp_src[e] (TAKE = false: converted by k_spread_finalize) or
 // straight from its fixed-point sum (TAKE = true: the conversion of
-// spread_finalize done here, one launch fewer after the MD cycle).
+// spread_record done here, one launch fewer after the MD cycle).
 template <int S, bool TAKE>
 __global__ void __launch_bounds__(256)
     k_spread_apply(LbGeom g, ChainArgs a, int nw, typename Store<S>::T *dst, int mode,
@@ -1475,27 +1475,34 @@ cudaError_t launch_spread_apply(int storage, const LbGeom &g, const ChainArgs &a
   return cudaGetLastError();
 }
 
-// Ensemble apply: same lane layout as k_ens_gather; each owner entry converts
-// its node's sum (k_ens_spread_accum) and adds the source as k_spread_apply
-// does.  The first lane of every realisation bumps its step count (if live)
-// and decides whether it takes part in the next step.
-template <int S>
+// Ensemble apply: same lane layout as k_ens_gather; each owner entry takes its
+// node's force -- from its record (TAKE = false: k_ens_spread_finalize) or its
+// sum (TAKE = true) -- and adds the source as k_spread_apply does.  The first
+// lane of every realisation bumps its step count (if live) and decides whether
+// it takes part in the next step.  Bound by the latency of dependent reads that
+// the stream-collide has driven out of L2: the records, in the entries' own
+// order, take the sum's three away.
+template <int S, bool TAKE>
 __global__ void __launch_bounds__(256)
     k_ens_spread(const EnsMember *__restrict__ mem, const int2 *__restrict__ beads, int nb,
                  const int *__restrict__ live, int *__restrict__ live_next, int cur,
-                 const long long *__restrict__ max_steps) {
+                 const long long *__restrict__ max_steps, const float4 *__restrict__ rec) {
   using St = Store<S>;
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   const int slot = e >> 3, k = e & 7;
   int2 mi = make_int2(-1, 0);
-  if (slot < nb) mi = beads[slot];
+  float4 r = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
+  if (slot < nb) {
+    mi = beads[slot];
+    if (!TAKE) r = rec[e];
+  }
   const bool valid = mi.x >= 0 && live[mi.x];
-  if (valid && mem[mi.x].a.owner) {
+  if (valid && (TAKE ? mem[mi.x].a.owner != nullptr : __float_as_int(r.w) >= 0)) {
     const ChainArgs &a = mem[mi.x].a;
     const int e2 = 8 * mi.y + k;
-    const int node = a.sp_node[e2];
-    if (node >= 0 && a.owner[node] == e2) {  // the owner converts its node's sum
-      const F3 F = spread_take(a, node, e2);
+    const int node = TAKE ? a.sp_node[e2] : __float_as_int(r.w);
+    if (!TAKE || (node >= 0 && a.owner[node] == e2)) {
+      const F3 F = TAKE ? spread_take(a, node, e2) : F3{r.x, r.y, r.z};
       const size_t st = pop_stride<S, size_t>((size_t)a.geo.Vp);
       typename St::T *dst = (typename St::T *)mem[mi.x].pop[cur ^ 1] +
                               pop_base<S, size_t>(pop_node<S, size_t>(a.geo, (size_t)node));
@@ -1560,7 +1567,8 @@ cudaError_t launch_ens_md_cycle(const EnsMember *mem, const int *chains, int cou
 
 // Ensemble sum part of the spread, after every MD group: one thread per
 // (realisation, bead, corner) entry as in k_ens_gather, adding the entry's
-// share to its owner's fixed-point sum (spread_add).
+// share to its owner's fixed-point sum (spread_add); k_ens_spread_finalize then
+// writes every entry's record (spread_record) to rec[entry].
 __global__ void __launch_bounds__(256)
     k_ens_spread_accum(const EnsMember *__restrict__ mem, const int2 *__restrict__ beads, int nb,
                        const int *__restrict__ live) {
@@ -1573,22 +1581,51 @@ __global__ void __launch_bounds__(256)
   if (a.owner == nullptr) return;  // no solvent: nothing to spread
   spread_add(a, 8 * mi.y + k, a.J[mi.y]);
 }
+__global__ void __launch_bounds__(256)
+    k_ens_spread_finalize(const EnsMember *__restrict__ mem, const int2 *__restrict__ beads, int nb,
+                          const int *__restrict__ live, float4 *__restrict__ rec) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // every share
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >> 3 >= nb) return;
+  const int2 mi = beads[e >> 3];
+  if (mi.x < 0 || !live[mi.x]) return;
+  rec[e] = spread_record(mem[mi.x].a, 8 * mi.y + (e & 7));
+}
 
-cudaError_t launch_ens_spread_accum(const EnsMember *mem, const int2 *beads, int nb,
-                                    const int *live, cudaStream_t s) {
+cudaError_t launch_ens_spread_sum(const EnsMember *mem, const int2 *beads, int nb, const int *live,
+                                  float4 *rec, cudaStream_t s) {
   if (nb <= 0) return cudaSuccess;
-  k_ens_spread_accum<<<(8 * nb + 255) / 256, 256, 0, s>>>(mem, beads, nb, live);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((8 * nb + 255) / 256);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_ens_spread_accum, mem, beads, nb, live);
+  if (e != cudaSuccess || !rec) return e;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_ens_spread_finalize, mem, beads, nb, live, rec);
+}
+
+template <int S>
+static void ens_spread_as(const EnsMember *mem, const int2 *beads, int nb, const int *live, int *live_next,
+                          int cur, const long long *max_steps, const float4 *rec, cudaStream_t s) {
+  const int blocks = nb > 0 ? (8 * nb + 255) / 256 : 1;
+  if (rec)
+    k_ens_spread<S, false><<<blocks, 256, 0, s>>>(mem, beads, nb, live, live_next, cur, max_steps, rec);
+  else
+    k_ens_spread<S, true><<<blocks, 256, 0, s>>>(mem, beads, nb, live, live_next, cur, max_steps, rec);
 }
 
 cudaError_t launch_ens_spread(int storage, const EnsMember *mem, const int2 *beads, int nb,
                               const int *live, int *live_next, int cur,
-                              const long long *max_steps, cudaStream_t s) {
-  const int blocks = nb > 0 ? (8 * nb + 255) / 256 : 1;
+                              const long long *max_steps, const float4 *rec, cudaStream_t s) {
   switch (storage) {
-    case LBMD_STORE_F32: k_ens_spread<LBMD_STORE_F32><<<blocks, 256, 0, s>>>(mem, beads, nb, live, live_next, cur, max_steps); break;
-    case LBMD_STORE_F16: k_ens_spread<LBMD_STORE_F16><<<blocks, 256, 0, s>>>(mem, beads, nb, live, live_next, cur, max_steps); break;
-    case LBMD_STORE_BF16: k_ens_spread<LBMD_STORE_BF16><<<blocks, 256, 0, s>>>(mem, beads, nb, live, live_next, cur, max_steps); break;
+    case LBMD_STORE_F32: ens_spread_as<LBMD_STORE_F32>(mem, beads, nb, live, live_next, cur, max_steps, rec, s); break;
+    case LBMD_STORE_F16: ens_spread_as<LBMD_STORE_F16>(mem, beads, nb, live, live_next, cur, max_steps, rec, s); break;
+    case LBMD_STORE_BF16: ens_spread_as<LBMD_STORE_BF16>(mem, beads, nb, live, live_next, cur, max_steps, rec, s); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
