@@ -787,7 +787,7 @@ __device__ __forceinline__ float4 gauss3(uint64_t seed, uint32_t bead, int64_t s
 
 // (2) the M MD substeps of one chain, one thread per bead, and (5) the
 // bookkeeping; `a` may live in parameter or shared memory.  BLOCK is the
-// register class (512 or 1024 threads).
+// register class (512, 768 or 1024 threads).
 //
 // One chain is one block, so a substep is a chain of dependent phases and its
 // bound is their latency.  The positions of a substep are final after SHAKE, so
