@@ -111,10 +111,10 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock, FLUCT ? 1 : (ODD ? 5 : 6))
 // node is not used.  Bound by instructions like the pull kernel, of which two
 // nodes need not many more than one.  us a step, one node per thread / even step
 // by pairs / both: 256x128x128 FP16 71.9 / - / 59.1, with a wall 76.7 / 71.9 /
-// 67.6, 256^3 280 / - / 227.  In the odd step a warp with a wall takes the halves'
+// 64.7, 192x96x96 with a wall 29.5 / 27.6 / 24.9, 256^3 280 / - / 227.  In the odd step a warp with a wall takes the halves'
 // way for most directions, so where one warp in two or three has one, or a box
 // is short of warps, the odd step stays with one node per thread: 160x96x96 with
-// a wall 24.6 / 24.2 / 26.3, 96x64x64 8.5 / 8.5 / 10.4, 48x96x96 without 10.8 /
+// a wall 24.6 / 24.2 / 24.8, 96x64x64 8.5 / 8.5 / 9.8, 48x96x96 without 10.8 /
 // 10.1 / 8.9, 64^3 5.8 / 5.5 / 5.3, 32^3 2.31 / 2.33 / 2.84.
 template <typename T2, int S, int FORCING, bool ODD>
 __device__ __forceinline__ void aa_pair(const LbGeom &g, const LbPhys &ph, typename Store<S>::T *buf,
@@ -152,16 +152,7 @@ __device__ __forceinline__ void aa_pair(const LbGeom &g, const LbPhys &ph, typen
       if (cx(p) == -1) w = __byte_perm(w0, words[word(row + xr) + opp(p) * kW], lone ? 0x5454 : 0x5432);
       h[p] = P::unpack(w);
     }
-    if (bb.x | bb.y)
-#pragma unroll
-      for (int p = 1; p < kQ; ++p) {
-        const bool ba = (bb.x >> p) & 1u, bbb = (bb.y >> p) & 1u;
-        if (ba || bbb) {
-          const float2 r = P::unpack(words[word(self) + p * kW]);
-          if (ba) h[p].x = r.x;
-          if (bbb) h[p].y = r.y;
-        }
-      }
+    if (bb.x | bb.y) pair_bounce<T2, true>(words + word(self), bb, h);
   }
   const bool skip_a = bb.x & 1u, skip_b = (bb.y & 1u) || lone;  // solid, or padding
   if (skip_a)
@@ -277,10 +268,10 @@ cudaError_t aa_launch_storage(int storage, const LbGeom &g, const LbPhys &ph, vo
   // 32-bit offsets when every population index fits
   const bool small = (long long)kQ * g.Vp < 0x7fffffffLL;
   // 16-bit storage: two nodes per thread, in the odd step only in boxes of 2^17 nodes or
-  // more without a wall across x or of 256 nodes or more in x (figures at aa_pair)
+  // more without a wall across x or of 192 nodes or more in x (figures at aa_pair)
   if constexpr (!FLUCT)
     if (small && g.pitch % 2 == 0 &&
-        (!odd || ((long long)g.nx * g.ny * g.nz >= 1 << 17 && (g.wall.wall_x < 0 || g.nx >= 256)))) {
+        (!odd || ((long long)g.nx * g.ny * g.nz >= 1 << 17 && (g.wall.wall_x < 0 || g.nx >= 192)))) {
       if (storage == LBMD_STORE_F16) return aa_launch_pair<__half2, LBMD_STORE_F16>(g, ph, buf, odd, bump, s);
       if (storage == LBMD_STORE_BF16)
         return aa_launch_pair<__nv_bfloat162, LBMD_STORE_BF16>(g, ph, buf, odd, bump, s);

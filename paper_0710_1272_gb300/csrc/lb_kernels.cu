@@ -79,8 +79,11 @@ static cudaError_t lb_launch(const LbGeom &g, const LbPhys &ph, const void *src,
                              DevStatus *bump, cudaStream_t s) {
   // 32-bit offsets when every population index fits
   const bool small = (long long)kQ * g.Vp < 0x7fffffffLL;
-  // 16-bit storage: two nodes per thread (rows of an even length, LbGeom::pitch)
-  if (small && g.pitch % 2 == 0) {
+  // 16-bit storage: two nodes per thread (rows of an even length, LbGeom::pitch),
+  // but not in boxes of up to 2^15 nodes, which are short of warps.  us a step,
+  // FP16, one node / two: 32^3 2.3 / 2.5, with a wall 2.7 / 3.0, 33x31x33 2.8 / 2.6
+  // (forced 3.3 / 2.9, with a wall 3.0 / 3.1), 48^3 3.6 / 3.1, 64^3 5.2 / 4.5.
+  if (small && g.pitch % 2 == 0 && (long long)g.nx * g.ny * g.nz > 1 << 15) {
     if (S == LBMD_STORE_F16) return lb_launch_pair<__half2>(g, ph, src, dst, bump, s);
     if (S == LBMD_STORE_BF16) return lb_launch_pair<__nv_bfloat162>(g, ph, src, dst, bump, s);
   }

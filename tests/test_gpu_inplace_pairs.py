@@ -1,6 +1,8 @@
-"""In-place streaming in 16-bit storage by pairs of nodes (boxes of 2^17 nodes or
-more): the same bits as pull streaming after every step, widths even and odd, walls
-at either half of a word, the box's edges and the pore included."""
+"""16-bit storage by pairs of nodes, in place and pull: the same bits after every step,
+widths even and odd, walls at either half of a word, the box's edges and the pore
+included.  Pull streaming takes pairs above 2^15 nodes, the in-place odd step from 2^17
+(with a wall across x from 192 nodes in x), so the boxes between hold pairs against
+single nodes."""
 import numpy as np
 import pytest
 
@@ -14,7 +16,12 @@ BOXES = [
     dict(nx=256, ny=23, nz=24, wall_x=127, pore_d=5),                     # wall in the second half
     dict(nx=257, ny=23, nz=24, wall_x=256, pore_d=3),                     # wall in a row's lone node
     dict(nx=257, ny=23, nz=24, wall_x=0, wall_thickness=3, pore_d=4, y_walls=1),
-    dict(nx=255, ny=23, nz=24, wall_x=100, pore_d=5),                     # odd step by single nodes
+    dict(nx=191, ny=31, nz=24, wall_x=100, pore_d=5),                     # odd step by single nodes
+    dict(nx=33, ny=32, nz=33, wall_x=16, pore_d=5),
+    dict(nx=35, ny=31, nz=31, wall_x=34, pore_d=3),
+    dict(nx=37, ny=30, nz=31, y_walls=1),
+    dict(nx=34, ny=32, nz=32, wall_x=33, wall_thickness=2, pore_d=4),
+    dict(nx=32, ny=32, nz=32, wall_x=15, pore_d=3),                       # 2^15: pull by single nodes
 ]
 
 
