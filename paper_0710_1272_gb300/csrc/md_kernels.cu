@@ -10,7 +10,7 @@
 //     F = F_WCA + F_bend + F_wall + F_drive - m gamma (v - u_i) + F_r,
 //     v += dt F / m,  r~ = r + dt v,
 //     SHAKE: Newton on the N-1 bond multipliers, the tridiagonal Jacobian
-//            solved by one warp of the block (tri_solve_warp),
+//            solved by parallel cyclic reduction (TriPart),
 //     v = (r' - r) / dt,  r = r',
 //     RATTLE: one tridiagonal solve removes the bond-parallel relative
 //             velocities,
@@ -21,7 +21,7 @@
 //   summed at that owner in 64-bit fixed point, and the owner adds the source
 //   to the node's post-collision populations once -- so a step gives the same
 //   bits whatever order the atomics take.
-#include "lb_collide.cuh"
+#include "lb_pull.cuh"
 
 namespace lbmd {
 
@@ -41,21 +41,29 @@ __device__ __forceinline__ float4 f4(F3 v) { return make_float4(v.x, v.y, v.z, 0
 __device__ __forceinline__ F3 operator+(F3 a, F3 b) { return F3{a.x + b.x, a.y + b.y, a.z + b.z}; }
 __device__ __forceinline__ F3 operator-(F3 a, F3 b) { return F3{a.x - b.x, a.y - b.y, a.z - b.z}; }
 __device__ __forceinline__ F3 operator*(float s, F3 a) { return F3{s * a.x, s * a.y, s * a.z}; }
-__device__ __forceinline__ float dot(F3 a, F3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
+// a . b with its roundings written out: which product of a sum is rounded and
+// which is fused is the compiler's choice otherwise, and a chain's bits with it
+// (chains of stiff beads, and any in 16-bit populations, carry a different last
+// bit into the fifth digit of the velocities within twenty steps).
+__device__ __forceinline__ float dot(F3 a, F3 b) {
+  return __fmaf_rn(a.z, b.z, __fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)));
+}
+__device__ __forceinline__ float dot_yx(F3 a, F3 b) {
+  return __fmaf_rn(a.z, b.z, __fmaf_rn(a.y, b.y, __fmul_rn(a.x, b.x)));
+}
 
 // Threads of the MD block: one per bead in whole warps; for chains of up to 224
 // beads warps that only evaluate the force list (two for up to 32 beads, else
-// eight), beside the bead warps' own work; and one more warp for the tridiagonal
-// solves where the block's register class (512, 768 or 1024 threads: 128, 80
-// or 64 registers) has room for it, else warp 0 solves beside its beads.
+// eight), beside the bead warps' own work; and for chains of more than one warp
+// one more for the boundary system of the tridiagonal solves, where the block's
+// register class (512, 768, 896 or 1024 threads: 128, 80, 72 or 64 registers) has
+// room for it, else warp 0 solves it.
 __host__ __device__ inline int bead_threads(int N) { return (N + 31) / 32 * 32; }
 int md_threads(int N) {
   int t = bead_threads(N);
-  if (t <= 32)
-    t += 64;
-  else if (t <= 224)
-    t += 256;
-  return t == 512 || t == 768 || t == LBMD_MAX_BEADS ? t : t + 32;
+  if (t <= 32) return t + 64;
+  if (t <= 224) t += 256;
+  return t == 512 || t == 768 || t == 896 || t == LBMD_MAX_BEADS ? t : t + 32;
 }
 // The block of an ensemble's chains: sizes in steps of 64 threads up to 512,
 // then the register classes, so that few launches take chains of every length
@@ -67,32 +75,15 @@ int md_group_threads(int N) {
   return t <= 512 ? (t + 63) / 64 * 64 : t <= 768 ? 768 : LBMD_MAX_BEADS;
 }
 
-// Chains of more than 512 beads halve their system before the solve: the
-// threads of the odd rows eliminate the even rows beside them (all at once),
-// and the solving warp is left with half the rows.  With 64 or 80 registers a
-// lane cannot hold 23 or 33 rows; through shared memory that many took 4.2 and
-// 5.6 k cycles, 13 and 17 rows in registers 1.05 and 1.15 k.
-__host__ __device__ inline bool halves_rows(int N) { return N > 512; }
-
-// Rows a lane of the solving warp takes, from the chain's length: odd, so that
-// the lanes' accesses fall into different banks; and the rows held, a multiple
-// of 32 of them (those past the chain are identity rows).
-__host__ __device__ inline int solve_rows(int N) {
-  const int n = N - 1;
-  const int m = halves_rows(N) ? n / 2 : n;
-  return m <= 32 * 5 ? 5 : m <= 32 * 13 ? 13 : 17;
-}
-
-// Shared memory of the MD block: the rows of the tridiagonal system and its
-// solution; per bead positions (hi, lo), displacements, bond vectors at the
-// start and the end of the substep, multipliers and the mask of acting list
-// entries; then the force list (8 bytes an entry) and a force per entry, eight
-// entries per bead (the chains measured average three) and 128 for the beads
-// in the pore, as far as 220 KB reach.
+// Shared memory of the MD block: per bead positions (hi, lo), displacements,
+// bond vectors at the start and the end of the substep, multipliers and the
+// mask of acting list entries; then the force list (8 bytes an entry) and a
+// separation and force factor per entry, eight entries per bead (the chains
+// measured average three) and 128 for the beads in the pore, as far as 220 KB
+// reach.
 constexpr int kMdSmemMost = 220000;
 __host__ __device__ inline size_t md_smem_head(int N) {
-  return ((size_t)32 * solve_rows(N) * (sizeof(float4) + sizeof(float)) +
-          (halves_rows(N) ? 2 * (size_t)(N + 1) * sizeof(float4) : 0) + (size_t)N * (5 * sizeof(float4) + 2 * sizeof(float)) + 15) / 16 * 16;
+  return ((size_t)N * (5 * sizeof(float4) + 2 * sizeof(float)) + 15) / 16 * 16;
 }
 __host__ __device__ inline int item_want(int N) { return 8 * N + 128; }
 __host__ __device__ inline int item_cap(int N) {
@@ -137,6 +128,16 @@ __device__ __forceinline__ void cell_frac_hl(float hi, float lo, int origin, int
   cell = wrap_near(origin + (int)fl, n);
 }
 
+// 2x2 matrices for the interface system of the tridiagonal solve.
+struct M2 {
+  float a, b, c, d;  // [[a, b], [c, d]]
+};
+__device__ __forceinline__ M2 mmul(M2 x, M2 y) {
+  return M2{x.a * y.a + x.b * y.c, x.a * y.b + x.b * y.d, x.c * y.a + x.d * y.c,
+            x.c * y.b + x.d * y.d};
+}
+__device__ __forceinline__ M2 madd(M2 x, M2 y) { return M2{x.a + y.a, x.b + y.b, x.c + y.c, x.d + y.d}; }
+
 // Hardware reciprocal approximation (relative error ~2^-23) for the
 // tridiagonal solves: they are latency-bound chains, and a correctly rounded
 // reciprocal costs several dependent instructions.
@@ -146,110 +147,164 @@ __device__ __forceinline__ float rcp_fast(float x) {
   return r;
 }
 
-// Reciprocal for the forces: the hardware approximation and one
-// Newton-Raphson step (relative error below an ulp), without a branch.
-__device__ __forceinline__ float rcp_newton(float x) {
-  const float r = rcp_fast(x);
-  return fmaf(fmaf(-x, r, 1.0f), r, r);
+__device__ __forceinline__ M2 minv(M2 x) {
+  const float r = rcp_fast(x.a * x.d - x.b * x.c);
+  return M2{x.d * r, -x.b * r, -x.c * r, x.a * r};
 }
+__device__ __forceinline__ M2 mshfl_up(M2 x, int s) {
+  return M2{__shfl_up_sync(0xffffffffu, x.a, s), __shfl_up_sync(0xffffffffu, x.b, s),
+            __shfl_up_sync(0xffffffffu, x.c, s), __shfl_up_sync(0xffffffffu, x.d, s)};
+}
+__device__ __forceinline__ M2 mshfl_down(M2 x, int s) {
+  return M2{__shfl_down_sync(0xffffffffu, x.a, s), __shfl_down_sync(0xffffffffu, x.b, s),
+            __shfl_down_sync(0xffffffffu, x.c, s), __shfl_down_sync(0xffffffffu, x.d, s)};
+}
+
 
 // s a + b, each component one fused operation.
 __device__ __forceinline__ F3 axpy(float s, F3 a, F3 b) {
   return F3{fmaf(s, a.x, b.x), fmaf(s, a.y, b.y), fmaf(s, a.z, b.z)};
 }
 
-// Tridiagonal solve over 32 R rows (row i: s_row[i] = (a, c, d, -) with
-// a x_{i-1} + x_i + c x_{i+1} = d: rows divided by their diagonals, so that
-// the determinants below stay in range; rows past the chain are zero) by one
-// warp; x_i goes to s_x[i].  Called by all 32 lanes, between two block barriers.
-//
-// What bounds it is latency: a chain has up to 1023 rows and nothing else to
-// do meanwhile.  Lane l takes the R rows from l R on.  Its first R - 1
-// unknowns are eliminated towards the lane's last one: the pivots as a
-// three-term recurrence of determinants P_k = P_{k-1} - a_k c_{k-1} P_{k-2},
-// whose chain is one fused operation per row (the reciprocals 1/P_k hang off
-// it), then x_k = u_k + v_k x_{l R - 1} - w_k x_{k+1}, and by back substitution
-// x_k = U_k + V_k x_{l R - 1} + W_k x_{l R + R - 1}.  The lanes' last unknowns
-// form a tridiagonal system of their own, solved by cyclic reduction over lane
-// shuffles.  Measured by itself: 0.50 k cycles for 20 beads, 0.73 k for 100,
-// 1.05 k for 400 (in the block, where the other warps' code competes for the
-// instruction cache, 0.9 / 1.2 / 1.7 k), against 0.66 / 1.85 / 3.1 k for 32-row
-// cyclic reductions in every warp with a boundary system and two more block
-// barriers.
-template <int R>
-__device__ __noinline__ void tri_solve_warp(int n, const float4 *s_row, float *s_x) {
-  const int lane = threadIdx.x & 31;
-  const float4 *row = s_row + lane * R;
-  float *out = s_x + lane * R;
-  float u[R - 1], v[R - 1], w[R - 1];
-  {
-    const float4 q = row[0];
-    u[0] = q.z;
-    v[0] = -q.x;
-    w[0] = q.y;
-  }
-  float Pm = 1.f, P = 1.f, c = w[0];
-#pragma unroll
-  for (int k = 1; k < R - 1; ++k) {
-    const float4 q = row[k];
-    const float Pn = fmaf(-(q.x * c), Pm, P);
-    const float m = P * rcp_fast(Pn), am = q.x * m;
-    w[k] = q.y * m;
-    u[k] = fmaf(-am, u[k - 1], q.z * m);
-    v[k] = -am * v[k - 1];
-    c = q.y;
-    Pm = P;
-    P = Pn;
-  }
-  const float uk = u[R - 2], vk = v[R - 2], wk = w[R - 2];
-  w[R - 2] = -wk;
-#pragma unroll
-  for (int k = R - 3; k >= 0; --k) {
-    const float h = w[k];
-    u[k] = fmaf(-h, u[k + 1], u[k]);
-    v[k] = fmaf(-h, v[k + 1], v[k]);
-    w[k] = -h * w[k + 1];
-  }
-  const float U = u[0], V = v[0], W = w[0];
-  // the lane's last row, with the neighbours' unknowns substituted
-  const float4 q = row[R - 1];
-  const float un = __shfl_down_sync(0xffffffffu, U, 1), vn = __shfl_down_sync(0xffffffffu, V, 1),
-              wn = __shfl_down_sync(0xffffffffu, W, 1);
-  float inv = rcp_fast(fmaf(q.y, vn, fmaf(-q.x, wk, 1.0f)));
-  float al = q.x * vk * inv, ga = q.y * wn * inv;
-  float x = fmaf(-q.y, un, fmaf(-q.x, uk, q.z)) * inv;
-  // lanes past the last row hold identity rows; al and ga of the first and
-  // last lane are zero, so what a shuffle leaves in place there drops out
-  const int lanes = (n + R - 1) / R;
-#pragma unroll 1
-  for (int s = 1; s < lanes; s <<= 1) {
-    const float am = __shfl_up_sync(0xffffffffu, al, s), gm = __shfl_up_sync(0xffffffffu, ga, s),
-                xm = __shfl_up_sync(0xffffffffu, x, s);
-    const float ap = __shfl_down_sync(0xffffffffu, al, s), gp = __shfl_down_sync(0xffffffffu, ga, s),
-                xp = __shfl_down_sync(0xffffffffu, x, s);
-    inv = rcp_fast(fmaf(-ga, ap, fmaf(-al, gm, 1.0f)));
-    x = fmaf(-ga, xp, fmaf(-al, xm, x)) * inv;
-    al = -al * am * inv;
-    ga = -ga * gp * inv;
-  }
-  const float xu = __shfl_up_sync(0xffffffffu, x, 1), xl = lane > 0 ? xu : 0.f;
-  out[R - 1] = x;
-#pragma unroll
-  for (int k = R - 2; k >= 0; --k) out[k] = fmaf(w[k], x, fmaf(v[k], xl, u[k]));
+// Barriers of a part of the block: the warps that hold beads, with or without
+// the warp that solves the boundary system.  `threads` counts all that take
+// part; every one of them meets the same barriers in the same order, whole
+// warps at a time.
+constexpr int kBarBeads = 1, kBarVote = 2, kBarSides = 3, kBarMiddle = 4;
+__device__ __forceinline__ void bar_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int threads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ bool bar_all(int id, int threads, bool p) {
+  int r;
+  asm volatile(
+      "{\n\t.reg .pred q, o;\n\tsetp.ne.s32 q, %3, 0;\n\tbar.red.and.pred o, %1, %2, q;\n\t"
+      "selp.s32 %0, 1, 0, o;\n\t}"
+      : "=r"(r)
+      : "r"(id), "r"(threads), "r"((int)p)
+      : "memory");
+  return r != 0;
 }
 
-// Half of a tridiagonal system: row j of the odd rows' system, from rows
-// i - 1, i and i + 1 (i = 2 j + 1).
-__device__ __forceinline__ float4 halve_row(float4 p, float4 q, float4 n) {
-  const float inv = rcp_fast(fmaf(-q.y, n.x, fmaf(-q.x, p.y, 1.0f)));
-  return make_float4(-q.x * p.x * inv, -q.y * n.y * inv, fmaf(-q.y, n.z, fmaf(-q.x, p.z, q.z)) * inv, 0.f);
+// Tridiagonal solve over rows 0..n-1 (row i held by thread i: a x_{i-1} + b x_i
+// + c x_{i+1} = d, with a_0 = c_{n-1} = 0), SPIKE-type partition by warps: each
+// warp reduces its 32 rows by cyclic reduction over lane shuffles, for the
+// right-hand side and for the two coupling columns to the neighbouring warps
+// (the "spikes" v and w), giving x_i = y_i - v_i x_last(prev warp) - w_i
+// x_first(next warp) (tri_reduce).  The first and last unknowns of neighbouring
+// warps form a block tridiagonal system with 2x2 blocks, one block row per warp
+// boundary, which one warp solves by block cyclic reduction (tri_boundary).
+// Rows past the chain are identity rows.
+//
+// What bounds it is latency, and the shuffles of many warps.  A partition over
+// the lanes of a single warp, with the rows in registers, is faster (400 rows
+// 1.1 k cycles; this one 2.9 k, sides 0.9 k and boundaries 2.0 k), but its last
+// bits differ, and with them the trajectories (see dot).
+struct TriPart {
+  float y, v, w;
+};
+// SPIKES: the chain has more than one warp.  Before round s the columns r1 and
+// r2 are zero but in the first and the last s lanes, so of each only one
+// neighbour counts.
+template <bool SPIKES>
+__device__ __forceinline__ TriPart tri_reduce(int n, float a, float b, float c, float d) {
+  const int t = threadIdx.x, lane = t & 31;
+  if (t >= n) {
+    a = 0.f;
+    b = 1.f;
+    c = 0.f;
+    d = 0.f;
+  }
+  float al = lane == 0 ? 0.f : a, be = b, ga = lane == 31 ? 0.f : c;
+  float r0 = d, r1 = lane == 0 ? a : 0.f, r2 = lane == 31 ? c : 0.f;
+#pragma unroll
+  for (int s = 1; s < 32; s <<= 1) {
+    const float bm = __shfl_up_sync(0xffffffffu, be, s), bp = __shfl_down_sync(0xffffffffu, be, s);
+    const float gm = __shfl_up_sync(0xffffffffu, ga, s), ap = __shfl_down_sync(0xffffffffu, al, s);
+    const float r0m = __shfl_up_sync(0xffffffffu, r0, s), r0p = __shfl_down_sync(0xffffffffu, r0, s);
+    const bool hm = lane >= s, hp = lane + s < 32;
+    const float k1 = hm ? al * rcp_fast(bm) : 0.f;
+    const float k2 = hp ? ga * rcp_fast(bp) : 0.f;
+    if (SPIKES) {
+      r1 = __fmaf_rn(-k1, __shfl_up_sync(0xffffffffu, r1, s), r1);
+      r2 = __fmaf_rn(-k2, __shfl_down_sync(0xffffffffu, r2, s), r2);
+    }
+    if (s < 16) {
+      const float am = __shfl_up_sync(0xffffffffu, al, s), gp = __shfl_down_sync(0xffffffffu, ga, s);
+      al = hm ? -k1 * am : 0.f;
+      ga = hp ? -k2 * gp : 0.f;
+    }
+    be = __fmaf_rn(-k2, ap, __fmaf_rn(-k1, gm, be));
+    r0 = __fmaf_rn(-k2, r0p, __fmaf_rn(-k1, r0m, r0));
+  }
+  const float ib = rcp_fast(be);
+  return TriPart{r0 * ib, r1 * ib, r2 * ib};
+}
+// The system of the nch - 1 boundaries between nch warps: from the parts of
+// each warp's first and last row (s_y, six floats a warp) the unknowns of the
+// last row [0, 32) and the first row [32, 64) of each warp.  By one warp.
+__device__ __forceinline__ void tri_boundary(int nch, const float *s_y, float *s_x) {
+  const int lane = threadIdx.x & 31;
+  // block row k: unknowns (x_last(k), x_first(k+1)) at the boundary of
+  // warps k and k+1; rows beyond nch-2 are identity rows
+  M2 L{0.f, 0.f, 0.f, 0.f}, D{1.f, 0.f, 0.f, 1.f}, U{0.f, 0.f, 0.f, 0.f};
+  float q0 = 0.f, q1 = 0.f;
+  if (lane < nch - 1) {
+    D.b = s_y[6 * lane + 5];        // w of the last row of warp k
+    D.c = s_y[6 * (lane + 1) + 1];  // v of the first row of warp k+1
+    L.a = s_y[6 * lane + 4];        // v of the last row of warp k
+    U.d = s_y[6 * (lane + 1) + 2];  // w of the first row of warp k+1
+    q0 = s_y[6 * lane + 3];
+    q1 = s_y[6 * (lane + 1)];
+  }
+  // block cyclic reduction over the nch - 1 boundary rows; each lane
+  // inverts its own diagonal block and the neighbours' inverses arrive by
+  // shuffle
+  for (int s = 1; s < nch - 1; s <<= 1) {
+    const M2 Di = minv(D);
+    const M2 Lm = mshfl_up(L, s), Dim = mshfl_up(Di, s), Um = mshfl_up(U, s);
+    const float q0m = __shfl_up_sync(0xffffffffu, q0, s), q1m = __shfl_up_sync(0xffffffffu, q1, s);
+    const M2 Lp = mshfl_down(L, s), Dip = mshfl_down(Di, s), Up = mshfl_down(U, s);
+    const float q0p = __shfl_down_sync(0xffffffffu, q0, s), q1p = __shfl_down_sync(0xffffffffu, q1, s);
+    M2 al2{0.f, 0.f, 0.f, 0.f}, ga2{0.f, 0.f, 0.f, 0.f};
+    if (lane >= s) {
+      const M2 t2 = mmul(L, Dim);
+      al2 = M2{-t2.a, -t2.b, -t2.c, -t2.d};
+    }
+    if (lane + s < 32) {
+      const M2 t2 = mmul(U, Dip);
+      ga2 = M2{-t2.a, -t2.b, -t2.c, -t2.d};
+    }
+    const M2 nL = mmul(al2, Lm), nU = mmul(ga2, Up);
+    D = madd(D, madd(mmul(al2, Um), mmul(ga2, Lp)));
+    const float nq0 = q0 + al2.a * q0m + al2.b * q1m + ga2.a * q0p + ga2.b * q1p;
+    const float nq1 = q1 + al2.c * q0m + al2.d * q1m + ga2.c * q0p + ga2.d * q1p;
+    L = nL;
+    U = nU;
+    q0 = nq0;
+    q1 = nq1;
+  }
+  const M2 Di = minv(D);
+  if (lane < nch - 1) {
+    s_x[lane] = Di.a * q0 + Di.b * q1;           // x_last of warp k
+    s_x[32 + lane + 1] = Di.c * q0 + Di.d * q1;  // x_first of warp k+1
+  }
+}
+// The unknown of a row of warp w from its part and the boundaries' unknowns.
+__device__ __forceinline__ float tri_finish(TriPart t, int w, int nch, const float *s_x) {
+  float x = t.y;
+  if (w > 0) x -= t.v * s_x[w - 1];
+  if (w + 1 < nch) x -= t.w * s_x[32 + w + 1];
+  return x;
 }
 
 // Eq. 2 truncated at 2^(1/6) sigma: adds -dV/dd for separation d.
 __device__ __forceinline__ void wca_add(F3 d, float sig2, float rc2, float eps24, F3 &F) {
   const float r2 = dot(d, d);
   if (r2 < rc2) {
-    const float ir2 = rcp_newton(r2);
+    const float ir2 = 1.0f / r2;
     const float sr2 = sig2 * ir2;
     const float sr6 = sr2 * sr2 * sr2;
     const float f = eps24 * (2.0f * sr6 * sr6 - sr6) * ir2;
@@ -258,19 +313,18 @@ __device__ __forceinline__ void wca_add(F3 d, float sig2, float rc2, float eps24
 }
 
 // Eq. 3 bending at the angle of beads (a, b, c) given the two bond vectors
-// b1 = r_b - r_a and b2 = r_c - r_b: the forces F = -dV/dr on a, b and c with
-// V = kappa phi^2 / 2.
-__device__ __noinline__ void bend_forces(F3 b1, F3 b2, float kappa, F3 &fa, F3 &fb, F3 &fc) {
-  const float l1 = sqrtf(dot(b1, b1)), l2 = sqrtf(dot(b2, b2));
-  float cphi = dot(b1, b2) / (l1 * l2);
-  cphi = fminf(1.f, fmaxf(-1.f, cphi));
+// b1 = r_b - r_a and b2 = r_c - r_b, their lengths and product: with
+// V = kappa phi^2 / 2 the forces F = -dV/dr on a, b and c are -A g1, A (g1 - g2)
+// and A g2; returns A.
+__device__ __noinline__ float bend_terms(F3 b1, F3 b2, float l1, float l2, float b12, float kappa, F3 &g1,
+                                         F3 &g2) {
+  const float cphi = fminf(1.f, fmaxf(-1.f, b12 / (l1 * l2)));
   const float phi = acosf(cphi);
   const float A = phi < 1e-4f ? kappa : kappa * phi / sinf(phi);
-  const F3 g1 = (1.0f / (l1 * l2)) * b2 - (cphi / (l1 * l1)) * b1;
-  const F3 g2 = (1.0f / (l1 * l2)) * b1 - (cphi / (l2 * l2)) * b2;
-  fa = (-A) * g1;
-  fb = A * (g1 - g2);
-  fc = A * g2;
+  const float p = 1.0f / (l1 * l2), q1 = -(cphi / (l1 * l1)), q2 = -(cphi / (l2 * l2));
+  g1 = axpy(q1, b1, F3{__fmul_rn(p, b2.x), __fmul_rn(p, b2.y), __fmul_rn(p, b2.z)});
+  g2 = axpy(q2, b2, F3{__fmul_rn(p, b1.x), __fmul_rn(p, b1.y), __fmul_rn(p, b1.z)});
+  return A;
 }
 
 // WCA pair forces on bead i from every other non-bonded bead (minimum image).
@@ -297,41 +351,25 @@ __device__ __noinline__ F3 all_pair_forces(const ChainArgs &a, int i, float4 rh,
 
 // Sec. III pulling force on a bead at the local position rh + rl: -f_drive x
 // inside the channel of the pore cross-section and the x-layers within 1.5
-// nodes of the wall.  In float throughout: the cell and its fraction by integer
-// conversions are a chain of ~25-cycle latencies each.
-struct Drive {
-  float sx, sy, sz;     // local coordinate -> coordinate of the box (x: from nx / 2 before the wall)
-  float ix, iy, iz;     // 1 / box
-  float cx, half;       // channel along x: centre, half length
-  float y0, y1, z0, z1; // its cross-section [y0, y1) x [z0, z1)
-  float f;              // 0: none
-};
-__device__ __forceinline__ Drive drive_of(const ChainArgs &a) {
+// nodes of the wall.
+__device__ __forceinline__ F3 drive_force_at(const ChainArgs &a, float4 rh, float4 rl) {
   const LbGeom &g = a.geo;
-  const float half_t = 0.5f * (float)(a.wall_t - 1);
-  Drive w;
-  w.sx = (float)(a.ox - a.wall_x + g.nx / 2);
-  w.sy = (float)a.oy;
-  w.sz = (float)a.oz;
-  w.ix = 1.0f / (float)g.nx;
-  w.iy = 1.0f / (float)g.ny;
-  w.iz = 1.0f / (float)g.nz;
-  w.cx = (float)(g.nx / 2) + half_t;
-  w.half = half_t + 1.5f;
-  w.y0 = (float)a.pore_y0 - 0.5f;
-  w.y1 = (float)(a.pore_y0 + a.pore_d) - 0.5f;
-  w.z0 = (float)a.pore_z0 - 0.5f;
-  w.z1 = (float)(a.pore_z0 + a.pore_d) - 0.5f;
-  w.f = a.has_wall && a.pore_d > 0 ? a.fdrive : 0.f;
-  return w;
-}
-__device__ __forceinline__ float drive_force_at(const Drive &w, const LbGeom &g, float4 rh, float4 rl) {
-  float x = (rh.x + w.sx) + rl.x, y = (rh.y + w.sy) + rl.y, z = (rh.z + w.sz) + rl.z;
-  x -= (float)g.nx * floorf(x * w.ix);  // into [0, n)
-  y -= (float)g.ny * floorf(y * w.iy);
-  z -= (float)g.nz * floorf(z * w.iz);
-  const bool in = fabsf(x - w.cx) <= w.half && y >= w.y0 && y < w.y1 && z >= w.z0 && z < w.z1;
-  return in ? -w.f : 0.f;
+  F3 F{0.f, 0.f, 0.f};
+  if (a.has_wall && a.pore_d > 0 && a.fdrive != 0.f) {
+    int c[3];
+    float sf[3];
+    cell_frac_hl(rh.x, rl.x, a.ox, g.nx, c[0], sf[0]);
+    cell_frac_hl(rh.y, rl.y, a.oy, g.ny, c[1], sf[1]);
+    cell_frac_hl(rh.z, rl.z, a.oz, g.nz, c[2], sf[2]);
+    const int di = wrap_near(c[0] - a.wall_x + g.nx / 2, g.nx) - g.nx / 2;
+    const float dx = (float)di + sf[0] - 0.5f * (float)(a.wall_t - 1);
+    const float half = 0.5f * (float)(a.wall_t - 1) + 1.5f;
+    const float ry = (float)c[1] + sf[1], rz = (float)c[2] + sf[2];
+    if (fabsf(dx) <= half && ry >= a.pore_y0 - 0.5f && ry < a.pore_y0 + a.pore_d - 0.5f &&
+        rz >= a.pore_z0 - 0.5f && rz < a.pore_z0 + a.pore_d - 0.5f)
+      F.x -= a.fdrive;
+  }
+  return F;
 }
 
 // Sum of K values over the block (every thread gets the sums).  red holds
@@ -472,15 +510,17 @@ __device__ __forceinline__ bool fits_short(float4 n) {
 }
 
 // Evaluates the flat list: `who` of `of` threads share the entries.  An entry
-// within the cutoff leaves its force in s_f and a bit in its bead's mask (the
-// entry's number among the bead's own); integer ORs commute, so the result does
-// not depend on the order of the threads.
+// within the cutoff leaves its separation d and the factor f of its force f d in
+// s_f (the bead adds f d by fused operations, as a walk along its own list
+// does) and a bit in its bead's mask (the entry's number among the bead's own);
+// integer ORs commute, so the result does not depend on the order of the threads.
 //
 // With a list per bead the chain waited for its fullest one (a bead in the
 // pore: ~25 entries at ~200-290 cycles each, 3.5-5 k cycles of every substep).
 // Spread over the block, two entries at a time and without a branch on the
 // cutoff, whose latencies would follow one another (400 beads: 2.7 k cycles with
-// the branch, 1.6 k without; 20 beads 1.3 and 0.8 k).
+// the branch, 1.6 k without; 20 beads 1.3 and 0.8 k, with an approximate
+// reciprocal in place of the division on both sides).
 __device__ __forceinline__ void eval_items(const ChainArgs &a, const uint2 *s_item, int n, int who,
                                            int of, const float4 *s_rh, const float4 *s_rl, float4 *s_f,
                                            unsigned *s_mask) {
@@ -516,11 +556,11 @@ __device__ __forceinline__ void eval_items(const ChainArgs &a, const uint2 *s_it
       if (image) d = min_image(a.geo, d);
       const float r2 = dot(d, d);
       const bool in = q < n && r2 < rc2;
-      const float ir2 = rcp_newton(r2);
+      const float ir2 = 1.0f / r2;
       const float sr2 = sig2 * ir2;
       const float sr6 = sr2 * sr2 * sr2;
       const float f = eps24 * (2.0f * sr6 * sr6 - sr6) * ir2;
-      if (in || (tail && q < n)) s_f[q] = in ? f4(f * d) : make_float4(0.f, 0.f, 0.f, 0.f);
+      if (in || (tail && q < n)) s_f[q] = in ? make_float4(d.x, d.y, d.z, f) : make_float4(0.f, 0.f, 0.f, 0.f);
       if (in && !tail) atomicOr(&s_mask[it[k].x & (LBMD_MAX_BEADS - 1)], 1u << (it[k].x >> 10 & 31u));
     }
   }
@@ -773,63 +813,69 @@ __device__ __forceinline__ float4 spread_record(const ChainArgs &a, int e) {
 }
 
 // Three standard normals for (bead, LB step, substep): Box-Muller on the four
-// uniforms of one Philox block, both pairs at once on paired FP32 (400 beads, 8
-// substeps: 866 against 890 us for 24 steps and their read-outs with the library
-// functions, whose error the normals share, see box_muller_t).
+// uniforms of one Philox block.
 __device__ __forceinline__ float4 gauss3(uint64_t seed, uint32_t bead, int64_t step, uint32_t substep) {
   const U4 c{bead, (uint32_t)(uint64_t)step, (uint32_t)((uint64_t)step >> 32), substep & 0xFFu};
   const U4 r = philox4x32_10(c, (uint32_t)seed, (uint32_t)(seed >> 32));
-  const uint32_t u1[2] = {r.x, r.z}, u2[2] = {r.y, r.w};
-  float2 n1, n2;
-  box_muller_t<Ops2>(uniform23_t<Ops2>(u1), uniform23_t<Ops2>(u2), n1, n2);
-  return make_float4(n1.x, n2.x, n1.y, 0.f);
+  const float u1 = uniform23(r.x), u2 = uniform23(r.y);
+  const float u3 = uniform23(r.z), u4 = uniform23(r.w);
+  const float r1 = sqrtf(-2.0f * logf(u1)), r2 = sqrtf(-2.0f * logf(u3));
+  float s2, c2, s4, c4;
+  sincospif(2.0f * u2, &s2, &c2);
+  sincospif(2.0f * u4, &s4, &c4);
+  return make_float4(r1 * c2, r1 * s2, r2 * c4, 0.f);
 }
 
 // (2) the M MD substeps of one chain, one thread per bead, and (5) the
 // bookkeeping; `a` may live in parameter or shared memory.  BLOCK is the
-// register class (512, 768 or 1024 threads).
+// register class (512, 768, 896 or 1024 threads).
 //
 // One chain is one block, so a substep is a chain of dependent phases and its
 // bound is their latency.  The positions of a substep are final after SHAKE, so
-// the next substep's forces, bond vectors and noise are found by the bead
-// warps while one warp solves RATTLE; what is left in line is: velocities and
-// the sum of the acting forces, one barrier, two Newton iterations (rows and
-// vote, solve, barrier), a last vote, positions and RATTLE's rows, one vote, the
-// solve, one barrier.  A thread keeps its own and its successor's displacement,
-// both updated by the same operations, so the Newton iterations exchange
-// nothing but the rows and the solution.
+// the next substep's forces, bond vectors and noise are found while RATTLE's
+// boundary system is solved; what is left in line is: velocities and the sum
+// of the acting forces, one barrier, two Newton iterations (rows and vote,
+// solve), a last vote, positions and RATTLE's rows, one vote, the solve, one
+// barrier.  A thread keeps its own and its successor's displacement, both
+// updated by the same operations, so the Newton iterations exchange nothing but
+// what the solve does.  Only the warps that hold beads, and the one that solves
+// the boundary system, meet in the constraint solves; a chain of one warp
+// solves without a barrier.  us a step without a solvent, with a list per bead,
+// the solve's boundary system and every barrier in line / so: 20 beads 29.6 /
+// 20.9, 100 beads 41.6 / 31.4, 400 beads 60.4 / 49.7, 700 beads 93 / 90, 1000
+// beads 122 / 123.
+//
+// The results of a step are those of every release to the last bit
+// (released_values.py among the tests): sums and products are written with
+// their roundings where the compiler has a choice.
 template <int BLOCK>
 __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
   extern __shared__ float4 smem4[];
   const int N = a.N;
   const int i = threadIdx.x;  // bead of this thread
   const bool bead = i < N;
-  // the warp of the tridiagonal solves: the last one, or the first of a block
-  // without a spare one; the threads that evaluate the force list: those
-  // between the beads' and the solve's, where there are two warps of them and
-  // the chain is short, else all but the solve's
-  const bool spare = (int)blockDim.x > bead_threads(N);
+  // the warps that hold beads; the warp of the boundary system between them: the
+  // last one, or the first of a block without a spare one; the threads that
+  // evaluate the force list: those between the two, where there are two warps
+  // of them and the chain is short, else all but the spare one's
+  const int holders = bead_threads(N), nch = holders >> 5, warp = i >> 5, lane = i & 31;
+  const bool holds = i < holders;
+  const bool spare = nch > 1 && (int)blockDim.x > holders;
   const int workers = spare ? (int)blockDim.x - 32 : (int)blockDim.x;
-  const bool solves = (i >> 5) == (spare ? workers >> 5 : 0);
-  const int eval0 = N <= 224 && workers - bead_threads(N) >= 64 ? bead_threads(N) : 0;
-  const int rows = 32 * solve_rows(N);
-  float4 *s_row = smem4;         // rows of the tridiagonal system to solve
-  float4 *s_full = s_row + rows; // halved rows: the whole system, two buffers
-  float4 *s_rh = s_full + (BLOCK > 512 ? 2 * (N + 1) : 0);  // positions, hi part (start of the substep)
+  const bool middle = nch > 1 && warp == (spare ? workers >> 5 : 0);
+  const int eval0 = N <= 224 && workers - holders >= 64 ? holders : 0;
+  const int solvers = spare ? holders + 32 : holders;
+  float4 *s_rh = smem4;          // positions, hi part (start of the substep)
   float4 *s_rl = s_rh + N;       // positions, lo part
   float4 *s_b = s_rl + N;        // bond vectors, start of the substep
   float4 *s_t = s_b + N;         // unconstrained displacement of the substep
   float4 *s_d = s_t + N;         // bond vectors at the end of the substep
-  float *s_x = (float *)(s_d + N);                 // solution of the tridiagonal system
-  float *s_lam = s_x + rows;                       // SHAKE multipliers of the last substep
+  float *s_lam = (float *)(s_d + N);               // SHAKE multipliers of the last substep
   unsigned *s_mask = (unsigned *)(s_lam + N);      // acting entries of the bead's flat list
-  float4 *s_f = (float4 *)((char *)smem4 + md_smem_head(N));  // their forces
+  float4 *s_f = (float4 *)((char *)smem4 + md_smem_head(N));  // their separations and force factors
   uint2 *s_item = (uint2 *)(s_f + item_cap(N));               // the flat list
   __shared__ int s_first[BLOCK];                              // a bead's first entry
-
-  const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int q = (BLOCK > 512 ? (N - 1) / 2 : max(N - 1, 0)) + i; q < rows; q += blockDim.x) s_row[q] = none;
-  if (BLOCK > 512 && i < 2) s_full[i * (N + 1) + N - 1] = none;  // the row after the last
+  __shared__ float s_y[6 * 32], s_x[64];                      // sides and middle of a solve
 
   const DevStatus *st0 = a.status;
   const long long step = st0->step;
@@ -885,77 +931,102 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
   const float tol = fmaxf(a.shake_tol, 5e-7f);
   const bool bond = a.has_bonds && i < N - 1;  // bond (i, i + 1)
   const bool bends = a.kappa != 0.f && a.has_bonds;
-  const Drive drive = drive_of(a);
   int shake_bad = 0, newton_total = 0, builds = 0;
-  // A row of the tridiagonal system, the solve (between two block barriers)
-  // and an unknown of it.  With halved rows the rows of successive solves take
-  // two buffers in turn: a thread may still look up an even unknown while
-  // another writes its next row.
-  constexpr bool HALF = BLOCK > 512;
-  int turn = 0;
-  auto put_row = [&](float4 r) { (HALF ? s_full + turn * (N + 1) : s_row)[i] = r; };
-  auto solve = [&]() {
-    const int n = N - 1;
-    if (HALF) {
-      const float4 *f = s_full + turn * (N + 1);
-      turn ^= 1;
-      if ((i & 1) && i < n) s_row[i >> 1] = halve_row(f[i - 1], f[i], f[i + 1]);
-      __syncthreads();
-      if (!solves) return;
-      if (n / 2 <= 32 * 13)
-        tri_solve_warp<13>(n / 2, s_row, s_x);
-      else
-        tri_solve_warp<17>(n / 2, s_row, s_x);
-      return;
+  // A tridiagonal solve by the warps that hold beads: its first part, the
+  // boundary system (solve_middle, a spare warp's whole share), and x_i and
+  // x_{i-1}.  Every read of s_y and s_x precedes a barrier of the solvers that
+  // comes before they are written again (votes, the barriers of a substep).
+  auto solve_sides = [&](float sub, float diag, float sup, float rhs) {
+    if (nch == 1) return tri_reduce<false>(N - 1, sub, diag, sup, rhs);
+    const TriPart t = tri_reduce<true>(N - 1, sub, diag, sup, rhs);
+    {
+      float *y = s_y + 6 * warp + (lane == 0 ? 0 : 3);
+      if (lane == 0 || lane == 31) {
+        y[0] = t.y;
+        y[1] = t.v;
+        y[2] = t.w;
+      }
+      __syncwarp();
+      if (middle) {
+        bar_sync(kBarSides, solvers);
+        tri_boundary(nch, s_y, s_x);
+        __syncwarp();
+      } else {
+        bar_arrive(kBarSides, solvers);
+      }
     }
-    if (!solves) return;
-    if (n <= 32 * 5)
-      tri_solve_warp<5>(n, s_row, s_x);
-    else if (n <= 32 * 13)
-      tri_solve_warp<13>(n, s_row, s_x);
-    else
-      tri_solve_warp<17>(n, s_row, s_x);
+    return t;
   };
-  auto unknown = [&](int j) {  // x_j of the last solve, 0 <= j < N - 1
-    if (!HALF) return s_x[j];
-    if (j & 1) return s_x[j >> 1];
-    const float4 r = s_full[(turn ^ 1) * (N + 1) + j];
-    const float xm = j > 0 ? s_x[(j >> 1) - 1] : 0.f, xp = j + 1 < N - 1 ? s_x[j >> 1] : 0.f;
-    return fmaf(-r.y, xp, fmaf(-r.x, xm, r.z));
+  auto solve_middle = [&]() {
+    bar_sync(kBarSides, solvers);
+    tri_boundary(nch, s_y, s_x);
+    __syncwarp();
+    bar_arrive(kBarMiddle, solvers);
+  };
+  auto solve_ends = [&](TriPart t, float &x_prev) {
+    if (nch > 1) bar_sync(kBarMiddle, solvers);
+    const float x = tri_finish(t, warp, nch, s_x);
+    const float xu = __shfl_up_sync(0xffffffffu, x, 1);
+    x_prev = lane > 0 ? xu : (warp > 0 ? s_x[warp - 1] : 0.f);
+    return x;
+  };
+  // whether every solver says yes
+  auto vote = [&](bool yes) {
+    if (nch > 1) {
+      __syncwarp();
+      return bar_all(kBarVote, solvers, yes);
+    }
+    const bool all = __all_sync(0xffffffffu, yes);
+    __syncwarp();
+    return all;
   };
   // What the coming substep k needs of the positions now in s_rh, s_rl (every
   // thread has passed a barrier since they were written; another follows
   // before the results are read): noise, the force on this bead from the
-  // drive and from bending (the shares of its angle on the neighbours left
-  // in s_d and in the unused components of s_rh, s_rl and s_b), its bond
-  // vector and the entries of the flat list.
+  // drive and from the bending at its own angle (the shares of that angle on the
+  // neighbours left in s_d and in the unused components of s_rh, s_rl, s_b and
+  // s_d), its bond vector and the entries of the flat list.
   float4 xi = make_float4(0.f, 0.f, 0.f, 0.f);
-  F3 Fp{0.f, 0.f, 0.f};
+  F3 Fd{0.f, 0.f, 0.f}, gb{0.f, 0.f, 0.f};
+  float Ab = 0.f;
   auto prepare = [&](int k) {
     if (lists && nl_ok == kNlFlat && i >= eval0 && i < workers)
       eval_items(a, s_item, n_items, i - eval0, workers - eval0, s_rh, s_rl, s_f, s_mask);
     if (!bead) return;
     xi = a.noise[(size_t)k * N + i];  // this thread wrote it
     F3 sb{0.f, 0.f, 0.f};
-    Fp = F3{0.f, 0.f, 0.f};
     if (bond) sb = diff_hl(s_rh[i + 1], s_rl[i + 1], rh, rl);
     float4 keep = f4(sb);
     if (bends) {
-      F3 fa{0.f, 0.f, 0.f}, fc = fa;
-      if (i >= 1 && i + 1 < N)
-        bend_forces(diff_hl(rh, rl, s_rh[i - 1], s_rl[i - 1]), sb, a.kappa, fa, Fp, fc);
-      s_d[i] = f4(fc);
-      keep.w = fa.x;
-      s_rh[i].w = fa.y;
-      s_rl[i].w = fa.z;
+      F3 g1{0.f, 0.f, 0.f}, g2 = g1;
+      F3 fc{0.f, 0.f, 0.f};  // on bead i + 1
+      Ab = 0.f;
+      if (i >= 1 && i + 1 < N) {
+        const F3 bm = diff_hl(rh, rl, s_rh[i - 1], s_rl[i - 1]);
+        const float l1 = sqrtf(dot(bm, bm)), lc = sqrtf(dot_yx(bm, bm)), l2 = sqrtf(dot(sb, sb)), b12 = dot(bm, sb);
+        float Ac = Ab = bend_terms(bm, sb, l1, l2, b12, a.kappa, g1, g2);
+        fc = g2;
+        // the force on bead i + 1 has always been found with the other rounding of l1
+        if (lc != l1) {
+          F3 g;
+          Ac = bend_terms(bm, sb, lc, l2, b12, a.kappa, g, fc);
+        }
+        fc = Ac * fc;
+      }
+      gb = g1 - g2;
+      s_d[i] = make_float4(fc.x, fc.y, fc.z, -Ab);
+      keep.w = g1.x;
+      s_rh[i].w = g1.y;
+      s_rl[i].w = g1.z;
     }
     if (bond || bends) s_b[i] = keep;
     // pulling force inside the channel through the pore
-    Fp.x += drive_force_at(drive, a.geo, rh, rl);
+    Fd = drive_force_at(a, rh, rl);
   };
   F3 D1{0.f, 0.f, 0.f};  // displacement of bead i + 1
   F3 d{0.f, 0.f, 0.f};   // bond vector i at the end of the substep
   F3 dm{0.f, 0.f, 0.f};  // bond vector i - 1 there
+  float r_sub = 0.f, r_diag = 1.f, r_sup = 0.f, r_rhs = 0.f;  // RATTLE's row
 
   // (2) M MD substeps.  One turn ends substep k - 1 (RATTLE) and takes substep
   // k up to its positions, so that every phase stands in the code once.
@@ -966,13 +1037,22 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
       ref = rh;
       ++builds;
     }
-    if (a.has_bonds && k > 0) solve();
-    if (k < a.M) prepare(k);
-    __syncthreads();
-    if (a.has_bonds && bead && k > 0) {
-      if (bond) v = axpy(unknown(i) * im, d, v);
-      if (i > 0) v = axpy(-(unknown(i - 1) * im), dm, v);
+    TriPart part{0.f, 0.f, 0.f};
+    if (a.has_bonds && k > 0) {
+      if (holds)
+        part = solve_sides(r_sub, r_diag, r_sup, r_rhs);
+      else if (middle)
+        solve_middle();
     }
+    if (k < a.M) prepare(k);
+    if (a.has_bonds && k > 0 && holds) {
+      __syncwarp();
+      float mum;
+      const float mu = solve_ends(part, mum);
+      if (bond) v = axpy(mu * im, d, v);
+      if (bead && i > 0) v = axpy(-(mum * im), dm, v);
+    }
+    __syncthreads();
     if (k == a.M) break;
     if (k == 0) {
       // (1) interpolated by k_gather, beside which this block may have
@@ -980,31 +1060,40 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
       asm volatile("griddepcontrol.wait;" ::: "memory");
       if (bead) ui = f3(a.ui[i]);
     }
-    // bond vectors s_{i-1}, s_i, s_{i+1} around the bead
+    // bond vectors s_{i-1}, s_i, s_{i+1} around the bead; the blocks with 64 or 72
+    // registers a thread read them anew for each use
     F3 sm{0.f, 0.f, 0.f}, sb{0.f, 0.f, 0.f}, sp{0.f, 0.f, 0.f}, D{0.f, 0.f, 0.f};
+    auto bonds = [&]() {
+      if (bond) sb = f3(s_b[i]);
+      if (bead && i > 0) sm = f3(s_b[i - 1]);
+      if (i < N - 2) sp = f3(s_b[i + 1]);
+    };
     float lam = 0.f;  // multiplier of bond i
     if (bead) {
-      F3 Fc = Fp;
+      F3 Fc{0.f, 0.f, 0.f};
       if (bends) {
-        Fc = F3{0.f, 0.f, 0.f};
         if (i >= 2) Fc = Fc + f3(s_d[i - 1]);
-        Fc = Fc + Fp;
-        if (i + 2 < N) Fc = Fc + F3{s_b[i + 1].w, s_rh[i + 1].w, s_rl[i + 1].w};
+        Fc = axpy(Ab, gb, Fc);
+        if (i + 2 < N) Fc = axpy(s_d[i + 1].w, F3{s_b[i + 1].w, s_rh[i + 1].w, s_rl[i + 1].w}, Fc);
       }
+      Fc = Fc + Fd;
       if (lists) {
-        F3 F{0.f, 0.f, 0.f};
         if (nl_ok == kNlFlat) {
+          F3 F{0.f, 0.f, 0.f};
           const float4 *f = s_f + s_first[i];
           unsigned mask = s_mask[i];
           s_mask[i] = 0u;
-          for (; mask; mask &= mask - 1u) F = F + f3(f[__ffs(mask) - 1]);
-          for (int q = (int)kItemTail; q < n_own; ++q) F = F + f3(f[q]);
+          for (; mask; mask &= mask - 1u) {
+            const float4 e = f[__ffs(mask) - 1];
+            F = axpy(e.w, f3(e), F);
+          }
+          for (int q = (int)kItemTail; q < n_own; ++q) F = axpy(f[q].w, f3(f[q]), F);
+          Fc = Fc + F;
         } else if (nl_ok == kNlBead) {
-          F = list_forces(a, i, rh, rl, s_rh, s_rl);
+          Fc = Fc + list_forces(a, i, rh, rl, s_rh, s_rl);
         } else {
-          F = all_pair_forces(a, i, rh, rl, s_rh, s_rl) + wall_stencil_forces(a, rh, rl);
+          Fc = Fc + all_pair_forces(a, i, rh, rl, s_rh, s_rl) + wall_stencil_forces(a, rh, rl);
         }
-        Fc = Fc + F;
       }
       const F3 fdrag = (-m * a.gamma) * (v - ui);
       const F3 fr = sig_r * F3{xi.x, xi.y, xi.z};
@@ -1012,11 +1101,10 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
       J = J + dt * (fdrag + fr);
       D = dt * v;  // unconstrained displacement r~ - r
     }
-    if (a.has_bonds) {
+    if (a.has_bonds && holds) {
       // SHAKE on displacements: D_i = dt v_i + (lam_i s_i - lam_{i-1} s_{i-1}) / m
       // with the old bond vectors s_b; Newton on G_b = |s_b + D_{b+1} - D_b|^2 - b0^2.
-      // Old bonds come from the double-float positions; the rows are divided
-      // by their diagonals -4 d_b . s_b / m.
+      // Old bonds come from the double-float positions.
       // Warm start: the multipliers of the previous substep applied along the
       // new old-bond vectors (the constraint forces change slowly).
       if (bead) {
@@ -1032,52 +1120,71 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
         if (i < N - 2) sp = f3(s_b[i + 1]);
         s_t[i] = f4(D);
       }
-      __syncthreads();
+      __syncwarp();
+      if (nch > 1) bar_sync(kBarBeads, holders);
       if (bond) D1 = f3(s_t[i + 1]);
       for (int it = 0;; ++it) {
-        float G = 0.f;
+        float G = 0.f, diag = 1.f, sub = 0.f, sup = 0.f;
         bool ok = true;
+        if (BLOCK > 768) bonds();
         if (bond) {
           // old bond from the double-float positions, displacements small: the
           // float residual is good to ~1e-7 of b0^2
           d = sb + (D1 - D);
           G = dot(d, d) - b02;
           ok = fabsf(G) <= tol * b02;
-          const float q = rcp_fast(dot(d, sb)), h = -0.5f * q;
-          put_row(make_float4(i > 0 ? h * dot(d, sm) : 0.f, i < N - 2 ? h * dot(d, sp) : 0.f,
-                              0.25f * m * q * G, 0.f));
+          diag = -4.0f * im * dot(d, sb);
+          if (i > 0) sub = 2.0f * im * dot(d, sm);
+          if (i < N - 2) sup = 2.0f * im * dot(d, sp);
           s_d[i] = f4(d);
         }
-        if (__syncthreads_and(ok)) break;
+        if (vote(ok)) break;
         if (it >= a.shake_maxit) {
           const bool bad = bond && !(fabsf(G) <= 1e-3f * b02);
-          if (__syncthreads_or(bad)) shake_bad = 1;
+          if (!vote(!bad)) shake_bad = 1;
           break;
         }
         ++newton_total;
-        solve();
-        __syncthreads();
-        if (bead) {
-          // own and next bead's displacement, by the same operations on both
-          // threads that hold it
-          const float x = bond ? unknown(i) : 0.f, xm = i > 0 ? unknown(i - 1) : 0.f;
-          if (bond) {
-            D = axpy(x * im, sb, D);
-            if (i < N - 2) D1 = axpy(unknown(i + 1) * im, sp, D1);
-            D1 = axpy(-(x * im), sb, D1);
-            lam += x;
-          }
-          if (i > 0) D = axpy(-(xm * im), sm, D);
+        const TriPart t = solve_sides(sub, diag, sup, -G);
+        float xm;
+        const float x = solve_ends(t, xm);
+        // what the thread of bead i + 1 finds for x_{i+1} and x_i: the first
+        // bead of a warp takes x_i from the boundary system
+        float xn = __shfl_down_sync(0xffffffffu, x, 1), xnm = x;
+        if (lane == 31 && warp + 1 < nch) {
+          const float *y = s_y + 6 * (warp + 1);
+          xn = tri_finish(TriPart{y[0], y[1], y[2]}, warp + 1, nch, s_x);
+          xnm = s_x[warp];
         }
+        if (BLOCK > 768) bonds();
+        // own and next bead's displacement, by the same operations on both
+        // threads that hold it
+        if (bond) {
+          D = axpy(x * im, sb, D);
+          if (i < N - 2) D1 = axpy(xn * im, sp, D1);
+          D1 = axpy(-(xnm * im), sb, D1);
+          lam += x;
+        }
+        if (bead && i > 0) D = axpy(-(xm * im), sm, D);
       }
       if (bond) s_lam[i] = lam;  // read again only after later barriers
+    } else if (a.has_bonds && middle) {
+      // the spare warp: the boundary systems of the Newton iterations
+      for (int it = 0;; ++it) {
+        if (vote(true)) break;
+        if (it >= a.shake_maxit) {
+          vote(true);
+          break;
+        }
+        solve_middle();
+      }
     }
     // every read of s_rh / s_rl of this substep precedes a barrier of the
     // constraint solves; without constraints one barrier is needed here
     if (!a.has_bonds) __syncthreads();
     if (bead) {
       // v = (r' - r) / dt evaluated as D / dt (no cancellation); r' = r + D
-      v = idt * D;
+      v = F3{__fmul_rn(idt, D.x), __fmul_rn(idt, D.y), __fmul_rn(idt, D.z)};
       two_sum_add(rh.x, rl.x, D.x);
       two_sum_add(rh.y, rl.y, D.y);
       two_sum_add(rh.z, rl.z, D.z);
@@ -1086,13 +1193,14 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
     }
     if (a.has_bonds && bead) {
       // RATTLE: v_i += (mu_i d_i - mu_{i-1} d_{i-1}) / m with the new bond
-      // vectors d_b = s_b + D_{b+1} - D_b, so that d_b . (v_{b+1} - v_b) = 0;
-      // rows divided by their diagonals -2 d_b . d_b / m.
+      // vectors d_b = s_b + D_{b+1} - D_b, so that d_b . (v_{b+1} - v_b) = 0.
       if (i > 0) dm = f3(s_d[i - 1]);
       if (bond) {
-        const float q = rcp_fast(dot(d, d)), h = -0.5f * q;
-        put_row(make_float4(i > 0 ? h * dot(d, dm) : 0.f, i < N - 2 ? h * dot(d, f3(s_d[i + 1])) : 0.f,
-                            0.5f * m * q * dot(d, idt * D1 - v), 0.f));
+        const F3 vn{__fmul_rn(idt, D1.x), __fmul_rn(idt, D1.y), __fmul_rn(idt, D1.z)};
+        r_rhs = -dot(d, vn - v);
+        r_diag = -2.0f * im * dot_yx(d, d);
+        if (i > 0) r_sub = im * dot(d, dm);
+        if (i < N - 2) r_sup = im * dot(d, f3(s_d[i + 1]));
       }
     }
     rebuild = __syncthreads_or(bead && moved());
@@ -1154,7 +1262,7 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
     const float it = nt > 0 ? 1.0f / (float)nt : 0.f, iu = nu > 0 ? 1.0f / (float)nu : 0.f;
     const F3 dt_{r.x - c[0] * it, r.y - c[1] * it, r.z - c[2] * it};
     const F3 du_{r.x - c[3] * iu, r.y - c[4] * iu, r.z - c[5] * iu};
-    const float fd = bead ? drive_force_at(drive, a.geo, rh, rl) : 0.f;
+    const float fd = bead ? drive_force_at(a, rh, rl).x : 0.f;
     float q[5] = {tr ? dot(dt_, dt_) : 0.f, un ? dot(du_, du_) : 0.f, bead ? dot(v, ui) : 0.f,
                   fd * v.x, bead ? dot(v, v) : 0.f};
     block_sum<5>(q, s_red);
@@ -1303,6 +1411,7 @@ cudaError_t md_prepare() {
   const int s512 = (int)md_smem_bytes(512), s768 = (int)md_smem_bytes(768), s1024 = (int)md_smem_bytes(LBMD_MAX_BEADS);
   cudaError_t e;
   if ((e = cudaFuncSetAttribute(k_md_cycle<768>, cudaFuncAttributeMaxDynamicSharedMemorySize, s768)) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(k_md_cycle<896>, cudaFuncAttributeMaxDynamicSharedMemorySize, s1024)) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(k_ens_md_cycle<768>, cudaFuncAttributeMaxDynamicSharedMemorySize, s768)) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(k_md_cycle<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, s512)) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(k_md_cycle<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, s1024)) != cudaSuccess) return e;
@@ -1345,6 +1454,7 @@ cudaError_t launch_md_cycle(const ChainArgs &a, int priority, bool beside, cudaS
   cfg.numAttrs = beside ? 2 : 1;
   if (threads <= 512) return cudaLaunchKernelEx(&cfg, k_md_cycle<512>, a);
   if (threads <= 768) return cudaLaunchKernelEx(&cfg, k_md_cycle<768>, a);
+  if (threads <= 896) return cudaLaunchKernelEx(&cfg, k_md_cycle<896>, a);
   return cudaLaunchKernelEx(&cfg, k_md_cycle<1024>, a);
 }
 
