@@ -6,7 +6,7 @@ namespace lbmd {
 
 cudaError_t launch_lb_aa(int storage, const LbGeom &g, const LbPhys &ph, void *buf, int odd,
                          DevStatus *bump, cudaStream_t s) {
-  return aa_launch_storage<false>(storage, g, ph, buf, odd, bump, s);
+  return aa_launch_storage<kNoNoise>(storage, g, ph, buf, odd, bump, s);
 }
 
 }  // namespace lbmd

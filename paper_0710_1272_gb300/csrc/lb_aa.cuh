@@ -26,7 +26,7 @@
 
 namespace lbmd {
 
-template <int S, int FORCING, typename I, bool ODD, bool FLUCT>
+template <int S, int FORCING, typename I, bool ODD, int NOISE>
 __device__ __forceinline__ void aa_node(const LbGeom &g, const LbPhys &ph,
                                         typename Store<S>::T *buf, int x, int y, int z,
                                         uint32_t bb) {
@@ -40,7 +40,7 @@ __device__ __forceinline__ void aa_node(const LbGeom &g, const LbPhys &ph,
   if (!ODD) {
 #pragma unroll
     for (int p = 0; p < kQ; ++p) h[p] = St::load_plain(buf + (I)p * st + pop_base<S, I>(self));
-    collide19<FORCING, FLUCT>(h, ph, (uint32_t)node);
+    collide19<FORCING, NOISE>(h, ph, (uint32_t)node);
     // The store addresses are the load addresses permuted; hiding the base
     // behind an empty asm makes the compiler recompute them after the
     // collision instead of keeping 19 of them live across it (which spills).
@@ -63,7 +63,7 @@ __device__ __forceinline__ void aa_node(const LbGeom &g, const LbPhys &ph,
     const I bidx = (I)p * st + pop_base<S, I>(self);
     h[p] = St::load_plain(buf + (((bb >> p) & 1u) ? bidx : sidx));
   }
-  collide19<FORCING, FLUCT>(h, ph, (uint32_t)node);
+  collide19<FORCING, NOISE>(h, ph, (uint32_t)node);
   // As in the even step: the store offsets equal the load offsets of the
   // opposite directions, so the coordinates are hidden behind an empty asm
   // and the offsets recomputed rather than kept live across the collision.
@@ -90,8 +90,8 @@ __device__ __forceinline__ void aa_node(const LbGeom &g, const LbPhys &ph,
 // kernel; without the thermal source six 256-thread blocks per SM for the
 // even step and five for the odd step (whose shifted stores need more
 // registers: at six it spills, and runs 1.7 % slower on a 256^3 solvent).
-template <int S, int FORCING, typename I, bool ODD, bool FLUCT>
-__global__ void __launch_bounds__(32 * kRowsPerBlock, FLUCT ? 1 : (ODD ? 5 : 6))
+template <int S, int FORCING, typename I, bool ODD, int NOISE>
+__global__ void __launch_bounds__(32 * kRowsPerBlock, NOISE ? 1 : (ODD ? 5 : 6))
     k_aa_stream_collide(LbGeom g, LbPhys ph, typename Store<S>::T *buf, DevStatus *bump) {
   const int x = blockIdx.x * 32 + threadIdx.x;
   const int y = blockIdx.y * kRowsPerBlock + threadIdx.y;
@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock, FLUCT ? 1 : (ODD ? 5 : 6))
   if (x >= g.nx || y >= g.ny) return;
   uint32_t bb = 0u;  // link mask; zero away from solid nodes
   if (beside_wall(g, x, y)) bb = __ldg(&g.lmask[((size_t)z * g.ny + y) * g.nx + x]);
-  aa_node<S, FORCING, I, ODD, FLUCT>(g, ph, buf, x, y, z, bb);
+  aa_node<S, FORCING, I, ODD, NOISE>(g, ph, buf, x, y, z, bb);
 }
 
 // 16-bit storage: the pair of x-adjacent nodes (2 xw, 2 xw + 1) whose deviations
@@ -236,7 +236,7 @@ cudaError_t aa_launch_pair(const LbGeom &g, const LbPhys &ph, void *buf, int odd
   return cudaGetLastError();
 }
 
-template <int S, typename I, bool FLUCT>
+template <int S, typename I, int NOISE>
 cudaError_t aa_launch(const LbGeom &g, const LbPhys &ph, void *buf, int odd, DevStatus *bump,
                       cudaStream_t s) {
   using T = typename Store<S>::T;
@@ -246,30 +246,37 @@ cudaError_t aa_launch(const LbGeom &g, const LbPhys &ph, void *buf, int odd, Dev
   const bool none = ph.g[0] == 0.f && ph.g[1] == 0.f && ph.g[2] == 0.f;
   if (odd) {
     if (none)
-      k_aa_stream_collide<S, kForcingNone, I, true, FLUCT><<<grid, block, 0, s>>>(g, ph, b, bump);
+      k_aa_stream_collide<S, kForcingNone, I, true, NOISE><<<grid, block, 0, s>>>(g, ph, b, bump);
     else if (ph.forcing == LBMD_FORCING_GUO)
-      k_aa_stream_collide<S, LBMD_FORCING_GUO, I, true, FLUCT><<<grid, block, 0, s>>>(g, ph, b, bump);
+      k_aa_stream_collide<S, LBMD_FORCING_GUO, I, true, NOISE><<<grid, block, 0, s>>>(g, ph, b, bump);
     else
-      k_aa_stream_collide<S, LBMD_FORCING_PAPER, I, true, FLUCT><<<grid, block, 0, s>>>(g, ph, b, bump);
+      k_aa_stream_collide<S, LBMD_FORCING_PAPER, I, true, NOISE><<<grid, block, 0, s>>>(g, ph, b, bump);
   } else {
     if (none)
-      k_aa_stream_collide<S, kForcingNone, I, false, FLUCT><<<grid, block, 0, s>>>(g, ph, b, bump);
+      k_aa_stream_collide<S, kForcingNone, I, false, NOISE><<<grid, block, 0, s>>>(g, ph, b, bump);
     else if (ph.forcing == LBMD_FORCING_GUO)
-      k_aa_stream_collide<S, LBMD_FORCING_GUO, I, false, FLUCT><<<grid, block, 0, s>>>(g, ph, b, bump);
+      k_aa_stream_collide<S, LBMD_FORCING_GUO, I, false, NOISE><<<grid, block, 0, s>>>(g, ph, b, bump);
     else
-      k_aa_stream_collide<S, LBMD_FORCING_PAPER, I, false, FLUCT><<<grid, block, 0, s>>>(g, ph, b, bump);
+      k_aa_stream_collide<S, LBMD_FORCING_PAPER, I, false, NOISE><<<grid, block, 0, s>>>(g, ph, b, bump);
   }
   return cudaGetLastError();
 }
 
-template <bool FLUCT>
+template <int NOISE>
+cudaError_t aa_launch_f32(const LbGeom &g, const LbPhys &ph, void *buf, int odd, DevStatus *bump,
+                          cudaStream_t s) {
+  if ((long long)kQ * g.Vp < 0x7fffffffLL) return aa_launch<LBMD_STORE_F32, int, NOISE>(g, ph, buf, odd, bump, s);
+  return aa_launch<LBMD_STORE_F32, size_t, NOISE>(g, ph, buf, odd, bump, s);
+}
+
+template <int NOISE>
 cudaError_t aa_launch_storage(int storage, const LbGeom &g, const LbPhys &ph, void *buf, int odd,
                               DevStatus *bump, cudaStream_t s) {
   // 32-bit offsets when every population index fits
   const bool small = (long long)kQ * g.Vp < 0x7fffffffLL;
   // 16-bit storage: two nodes per thread, in the odd step only in boxes of 2^17 nodes or
   // more without a wall across x or of 192 nodes or more in x (figures at aa_pair)
-  if constexpr (!FLUCT)
+  if constexpr (NOISE == kNoNoise)
     if (small && g.pitch % 2 == 0 &&
         (!odd || ((long long)g.nx * g.ny * g.nz >= 1 << 17 && (g.wall.wall_x < 0 || g.nx >= 192)))) {
       if (storage == LBMD_STORE_F16) return aa_launch_pair<__half2, LBMD_STORE_F16>(g, ph, buf, odd, bump, s);
@@ -278,14 +285,13 @@ cudaError_t aa_launch_storage(int storage, const LbGeom &g, const LbPhys &ph, vo
     }
   switch (storage) {
     case LBMD_STORE_F32:
-      return small ? aa_launch<LBMD_STORE_F32, int, FLUCT>(g, ph, buf, odd, bump, s)
-                   : aa_launch<LBMD_STORE_F32, size_t, FLUCT>(g, ph, buf, odd, bump, s);
+      return aa_launch_f32<NOISE>(g, ph, buf, odd, bump, s);
     case LBMD_STORE_F16:
-      return small ? aa_launch<LBMD_STORE_F16, int, FLUCT>(g, ph, buf, odd, bump, s)
-                   : aa_launch<LBMD_STORE_F16, size_t, FLUCT>(g, ph, buf, odd, bump, s);
+      return small ? aa_launch<LBMD_STORE_F16, int, NOISE>(g, ph, buf, odd, bump, s)
+                   : aa_launch<LBMD_STORE_F16, size_t, NOISE>(g, ph, buf, odd, bump, s);
     case LBMD_STORE_BF16:
-      return small ? aa_launch<LBMD_STORE_BF16, int, FLUCT>(g, ph, buf, odd, bump, s)
-                   : aa_launch<LBMD_STORE_BF16, size_t, FLUCT>(g, ph, buf, odd, bump, s);
+      return small ? aa_launch<LBMD_STORE_BF16, int, NOISE>(g, ph, buf, odd, bump, s)
+                   : aa_launch<LBMD_STORE_BF16, size_t, NOISE>(g, ph, buf, odd, bump, s);
   }
   return cudaErrorInvalidValue;
 }

@@ -151,8 +151,53 @@ __device__ __forceinline__ void box_muller_t(typename O::V u1, typename O::V u2,
 // with fifteen standard normals r_k from Box-Muller on four Philox blocks,
 // counter (node, step lo, step hi, block | 2 << 8), key (seed lo, seed hi).
 // The noise touches only non-conserved modes: mass and momentum are exact.
-// Returns v_p = xi_p / w_p.  The sum over modes (mode_row) is taken by the parity of the modes and of the
-// directions: 55 additions in place of 238 products.
+//
+// Two forms, equal up to the rounding of single precision (2e-8 of the
+// populations), of which launch_lb_*_fluct choose:
+//  kNoiseNode: the library's logarithm, sine and cosine and a sum over all
+//   modes, a node at a time;
+//  kNoisePair: box_muller_t and the modes by parity, one or two nodes.
+// What is rounded to 16 bits afterwards, or moves a chain, keeps kNoiseNode: a
+// last bit there turns a rounding of a stored population, and after 16 steps
+// the velocity field of a bfloat16 box is 1e-3 from that of the other form.
+enum Noise { kNoNoise = 0, kNoiseNode = 1, kNoisePair = 2 };
+
+__device__ __forceinline__ void thermal_source(const LbPhys &ph, uint32_t node, float rho,
+                                               float xi[kQ]) {
+  const long long step = *ph.step;
+  float r[16];
+#pragma unroll
+  for (uint32_t j = 0; j < 4; ++j) {
+    const U4 c{node, (uint32_t)(unsigned long long)step, (uint32_t)((unsigned long long)step >> 32),
+               j | (2u << 8)};
+    const U4 x = philox4x32_10(c, (uint32_t)ph.seed, (uint32_t)(ph.seed >> 32));
+    const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float rad = sqrtf(-2.0f * logf(uniform23(xs[2 * h])));
+      float sn, cs;
+      sincospif(2.0f * uniform23(xs[2 * h + 1]), &sn, &cs);
+      r[4 * j + 2 * h] = rad * cs;
+      r[4 * j + 2 * h + 1] = rad * sn;
+    }
+  }
+  const float sr = sqrtf(rho);
+  float t[15];
+#pragma unroll
+  for (int k = 0; k < 15; ++k) t[k] = ph.fl_amp[k] * sr * r[k];
+#pragma unroll
+  for (int p = 0; p < kQ; ++p) {
+    float acc = 0.f;
+#pragma unroll
+    for (int k = 4; k < kQ; ++k)
+      if (mode_row(k, p) != 0) acc = fmaf((float)mode_row(k, p), t[k - 4], acc);
+    xi[p] = wq(p) * acc;
+  }
+}
+
+// kNoisePair.  thermal_source_t returns v_p = xi_p / w_p.  The sum over modes
+// (mode_row) is taken by the parity of the modes and of the directions: 55
+// additions in place of 238 products.
 template <class O>
 __device__ __forceinline__ void thermal_normals_t(const LbPhys &ph, const uint32_t *node,
                                                   typename O::V r[16]) {
@@ -259,16 +304,17 @@ __device__ __forceinline__ typename O::V cdotu_t(int p, typename O::V ux, typena
 //   paper forcing: S_p = 3 w_p c_p . g;
 //   Guo forcing:   u = (j + g/2)/rho, S_p = (1 - omega/2) w_p [3 (c - u) + 9 (c.u) c] . g;
 //   kForcingNone (g = 0): u = j/rho, S_p = 0;
-//   FLUCT: plus the thermal source F_p of Eq. 5 (thermal_source_t) of the
-//   node's (nodes') fifteen normals.
+//   NOISE: plus the thermal source F_p of Eq. 5, of node `node` (kNoiseNode: Ops1
+//   only) or from the node's (nodes') fifteen normals (kNoisePair).
 // Opposite directions p, opp(p) = p + 1 (odd p) share c.u up to the sign, so
 // heq splits into the even part w_p [(rho - rho0) - 3/2 rho u.u + 9/2 rho (c.u)^2]
 // and the odd part +-3 w_p rho c.u, computed once per pair.  A node whose
 // density is not finite (a population is not) sets *ph.nonfinite.
-template <class O, int FORCING, bool FLUCT = false>
-__device__ __forceinline__ void collide_t(typename O::V h[kQ], const LbPhys &ph,
+template <class O, int FORCING, int NOISE = kNoNoise>
+__device__ __forceinline__ void collide_t(typename O::V h[kQ], const LbPhys &ph, uint32_t node = 0,
                                           const typename O::V *normals = nullptr) {
   using V = typename O::V;
+  static_assert(NOISE != kNoiseNode || O::N == 1, "one node per call");
   V drho, jx, jy, jz;
   moments_t<O>(h, drho, jx, jy, jz);
   const V rho = O::add(O::splat(ph.rho0), drho);
@@ -305,10 +351,15 @@ __device__ __forceinline__ void collide_t(typename O::V h[kQ], const LbPhys &ph,
     if (FORCING == LBMD_FORCING_PAPER) return O::add(v, O::splat(__fmul_rn(3.0f * wq(p), cg)));
     return v;
   };
-  V xi[kQ];  // F_p / w_p
-  if constexpr (FLUCT) thermal_source_t<O>(ph, normals, rho, xi);
+  V xi[kQ];  // F_p, or F_p / w_p
+  if constexpr (NOISE == kNoiseNode) thermal_source(ph, node, rho, xi);
+  if constexpr (NOISE == kNoisePair) thermal_source_t<O>(ph, normals, rho, xi);
+  const auto add_noise = [&](int p) {
+    if constexpr (NOISE == kNoiseNode) h[p] = O::add(h[p], xi[p]);
+    if constexpr (NOISE == kNoisePair) h[p] = O::fma(O::splat(wq(p)), xi[p], h[p]);
+  };
   h[0] = add_source(0, O::splat(0.f), O::fma(O::splat(__fmul_rn(om, wq(0))), A, O::mul(vom1, h[0])));
-  if constexpr (FLUCT) h[0] = O::fma(O::splat(wq(0)), xi[0], h[0]);
+  add_noise(0);
 #pragma unroll
   for (int p = 1; p < kQ; p += 2) {
     const V cu = cdotu_t<O>(p, ux, uy, uz);  // c_opp(p) . u = -cu
@@ -316,18 +367,16 @@ __device__ __forceinline__ void collide_t(typename O::V h[kQ], const LbPhys &ph,
     const V ow = O::splat(__fmul_rn(om, wq(p)));
     h[p] = add_source(p, cu, O::fma(ow, O::fma(r3, cu, even), O::mul(vom1, h[p])));
     h[p + 1] = add_source(p + 1, O::neg(cu), O::fma(ow, O::fma(O::neg(r3), cu, even), O::mul(vom1, h[p + 1])));
-    if constexpr (FLUCT) {
-      h[p] = O::fma(O::splat(wq(p)), xi[p], h[p]);
-      h[p + 1] = O::fma(O::splat(wq(p)), xi[p + 1], h[p + 1]);
-    }
+    add_noise(p);
+    add_noise(p + 1);
   }
 }
 
-template <int FORCING, bool FLUCT = false>
+template <int FORCING, int NOISE = kNoNoise>
 __device__ __forceinline__ void collide19(float h[kQ], const LbPhys &ph, uint32_t node = 0) {
   float r[16];
-  if constexpr (FLUCT) thermal_normals_t<Ops1>(ph, &node, r);
-  collide_t<Ops1, FORCING, FLUCT>(h, ph, r);
+  if constexpr (NOISE == kNoisePair) thermal_normals_t<Ops1>(ph, &node, r);
+  collide_t<Ops1, FORCING, NOISE>(h, ph, node, r);
 }
 
 __device__ __forceinline__ void zero19(float h[kQ]) {
@@ -345,7 +394,7 @@ __device__ __forceinline__ bool solid_is_left_out(const LbGeom &g, int y) {
 }
 
 // Stream and collide node (x, y, z) of one box: pull, Eq. 5 collision, store.
-template <int S, int FORCING, typename I>
+template <int S, int FORCING, typename I, int NOISE = kNoNoise>
 __device__ __forceinline__ void stream_collide_node(const LbGeom &g, const LbPhys &ph,
                                                     const typename Store<S>::T *__restrict__ src,
                                                     typename Store<S>::T *__restrict__ dst, int x,
@@ -364,7 +413,7 @@ __device__ __forceinline__ void stream_collide_node(const LbGeom &g, const LbPhy
   } else {
     pull19_mask<S, I>(g, src, x, y, z, 0u, h);  // constant mask: no selects
   }
-  collide19<FORCING>(h, ph);
+  collide19<FORCING, NOISE>(h, ph, (uint32_t)self);
   if (bb & 1u) zero19(h);
   const I st = pop_stride<S, I>((I)g.Vp);
   const I at = pop_base<S, I>(((I)z * g.ny + y) * row_pitch<S>(g) + x);

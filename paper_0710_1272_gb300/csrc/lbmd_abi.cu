@@ -152,8 +152,8 @@ cudaError_t enqueue_step(lbmd_ctx *c, int src) {
   if (c->phys.step) {
     // thermal source: the kernel reads the step count, so a box without
     // beads advances it in a separate launch afterwards
-    e = c->aa ? launch_lb_aa_fluct(c->p.storage, c->geo, c->phys, B, src, c->own)
-              : launch_lb_stream_collide_fluct(c->p.storage, c->geo, c->phys, A, B, c->own);
+    e = c->aa ? launch_lb_aa_fluct(c->p.storage, c->geo, c->phys, B, src, c->N > 0, c->own)
+              : launch_lb_stream_collide_fluct(c->p.storage, c->geo, c->phys, A, B, c->N > 0, c->own);
     if (e != cudaSuccess) return e;
     if (c->N == 0 && (e = launch_bump_step(c->status, c->own)) != cudaSuccess) return e;
   } else {

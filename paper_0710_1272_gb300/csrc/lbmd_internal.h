@@ -188,9 +188,10 @@ cudaError_t md_prepare();
 cudaError_t launch_lb_stream_collide(int storage, const LbGeom &g, const LbPhys &ph,
                                      const void *src, void *dst, DevStatus *bump,
                                      cudaStream_t s);
-// Stream-collide with the thermal source (ph.step != null); `bump` as above.
+// Stream-collide with the thermal source (ph.step != null).  `chain`: the box
+// holds beads, whose motion depends on the noise to the last bit.
 cudaError_t launch_lb_stream_collide_fluct(int storage, const LbGeom &g, const LbPhys &ph,
-                                           const void *src, void *dst, cudaStream_t s);
+                                           const void *src, void *dst, bool chain, cudaStream_t s);
 // Per-mode noise amplitudes a_k (k = 4..18) of the thermal source.
 void fluct_amplitudes(double kT, double tau, float amp[15]);
 // status->step += 1 (one thread): the step count of a box without beads when
@@ -214,7 +215,7 @@ cudaError_t launch_init_local(int storage, const LbGeom &g, float rho0, const fl
 cudaError_t launch_lb_aa(int storage, const LbGeom &g, const LbPhys &ph, void *buf, int odd,
                          DevStatus *bump, cudaStream_t s);
 cudaError_t launch_lb_aa_fluct(int storage, const LbGeom &g, const LbPhys &ph, void *buf,
-                               int odd, cudaStream_t s);
+                               int odd, bool chain, cudaStream_t s);
 // Read-outs of the pre-collision state of populations held in layout `mode`.
 cudaError_t launch_read_moments(int storage, const LbGeom &g, const LbPhys &ph,
                                 const void *src, int mode, long long z0, long long nzc,

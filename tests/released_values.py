@@ -1,6 +1,7 @@
 """Bead states and velocity fields of runs whose last bits matter: chains of stiff beads, and chains in
 16-bit populations, carry a different last bit of the MD cycle into the fifth digit of the velocities
-within twenty steps, so a change of its arithmetic shows here and nowhere else.  The values in
+within twenty steps, and thermal noise rounded to 16 bits does the same to the field, so a change of their
+arithmetic shows here and nowhere else.  The values in
 golden/*.npz were written by ``python tests/released_values.py KIND golden/KIND_values.npz`` with the
 release of commit 33770b1 (CUDA 13.0); the tests compare the present library with them."""
 import os
@@ -26,6 +27,19 @@ CASES = {
         "bf16_300": (dict(nx=128, ny=64, nz=64, wall_x=64, pore_d=5, n_beads=300, lj_eps=1.0, seed=8,
                           storage="bf16"), 12),
     },
+    "thermal": {
+        "bf16_pull": (dict(nx=26, ny=17, nz=12, kT_fluid=1e-4, tau=0.8, seed=3, storage="bf16"), 16),
+        "bf16_aa_guo": (dict(nx=24, ny=19, nz=14, kT_fluid=1e-4, tau=0.7, seed=4, storage="bf16", streaming="aa",
+                             forcing="guo", body_force=(1e-5, 0.0, 0.0)), 16),
+        "f16_walls": (dict(nx=27, ny=18, nz=15, wall_x=13, pore_d=3, kT_fluid=1e-4, seed=5, storage="f16",
+                           body_force=(1e-5, 0.0, 0.0)), 16),
+        "f16_above_2^15": (dict(nx=41, ny=33, nz=27, y_walls=1, kT_fluid=1e-4, tau=0.8, seed=6, storage="f16"), 9),
+        "f32": (dict(nx=25, ny=18, nz=13, kT_fluid=1e-4, tau=0.8, seed=7), 16),
+        "f32_chain": (dict(nx=84, ny=44, nz=58, wall_x=42, pore_d=5, n_beads=130, lj_eps=1.0, kT_fluid=1e-4,
+                           seed=29), 16),
+        "bf16_chain": (dict(nx=34, ny=16, nz=16, wall_x=17, pore_d=3, n_beads=24, lj_eps=1.0, kT_fluid=1e-4, seed=9,
+                            storage="bf16", streaming="aa"), 16),
+    },
 }
 
 
@@ -40,7 +54,7 @@ def run(kind, name):
     if p.get("n_beads", 0):
         pos, vel = sim.beads()
         out["pos"], out["vel"] = pos.astype(np.float32), vel.astype(np.float32)
-    if p["nx"] * p["ny"] * p["nz"] < 30000:
+    if p["nx"] * p["ny"] * p["nz"] < 40000:
         rho, u = sim.fields()
         out["rho"], out["u"] = rho.reshape(-1)[::7].copy(), u.reshape(3, -1)[:, ::7].copy()
     return out
