@@ -94,7 +94,7 @@ __device__ __forceinline__ bool tile_is_near(const LbGeom &g, int x, int y, int 
 // Pre-collision deviations h_p(x, t) of fluid node (x, y, z) for populations
 // held in layout `mode` (kPop*), taking the link mask only where a solid node
 // is within one node of the node's tile.  For read-outs and the bead gather,
-// which run while no kernel writes `src`.
+// which run while no kernel writes `src` (gather_goes_first).
 template <int S, typename I = size_t>
 __device__ __forceinline__ void fetch19(const LbGeom &g, const typename Store<S>::T *__restrict__ src,
                                         int x, int y, int z, int mode, float h[kQ]) {

@@ -124,7 +124,8 @@ cudaError_t enqueue_step(lbmd_ctx *c, int src) {
     // high-priority side stream while the stream-collide runs on the main
     // one.  Where the stream-collide sets the step, it starts at once; where
     // the MD branch sets it, the gather runs first, before the
-    // stream-collide takes the SMs (figures at spread_take_in_apply).
+    // stream-collide takes the SMs (figures at spread_take_in_apply); in place
+    // the stream-collide writes what the gather reads and always waits for it.
     ChainArgs a = c->chain;
     a.f = A;
     a.f_mode = pop_mode(c, src);
@@ -135,7 +136,7 @@ cudaError_t enqueue_step(lbmd_ctx *c, int src) {
     if ((e = cudaStreamWaitEvent(c->side, c->ev_fork, 0)) != cudaSuccess) return e;
     if (t[2] && (e = record_timing(t[2], c->side)) != cudaSuccess) return e;
     if ((e = launch_gather(c->p.storage, a, c->side)) != cudaSuccess) return e;
-    if (take) {
+    if (gather_goes_first(c->p.storage, c->geo.V, c->aa)) {
       if ((e = cudaEventRecord(c->ev_gather, c->side)) != cudaSuccess) return e;
       if ((e = cudaStreamWaitEvent(c->own, c->ev_gather, 0)) != cudaSuccess) return e;
     }

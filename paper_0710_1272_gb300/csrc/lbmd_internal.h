@@ -251,14 +251,21 @@ cudaError_t launch_spread_sum(const ChainArgs &a, bool records, cudaStream_t s);
 // True when the apply should convert the sums itself (the MD branch sets the
 // step), false when the stream-collide sets it -- taken as a stream-collide
 // moving 240 MB or more per step (~40 us at the HBM rate, about the MD branch of
-// a 400-bead chain beside it).  The gather follows the same rule (enqueue_step);
-// so does an ensemble, by the nodes of all its boxes.  Step of a 400-bead chain,
+// a 400-bead chain beside it).  The gather follows the same rule with two
+// population buffers (gather_goes_first); so does an ensemble, by the nodes of
+// all its boxes.  Step of a 400-bead chain,
 // us, true against false: 144x80x80 FP32 (140 MB) 47.7 / 54.5, FP16 44.2 / 47.1;
 // 256x128x128 FP16 (318 MB) 73.3 / 69.1, FP32 (637 MB) 105.3 / 101.6; of an
 // ensemble of 32 chains of 120 - 400 beads, FP16 (764 MB): 194.6 / 191.0.
 inline bool spread_take_in_apply(int storage, long long nodes) {
   const long long bytes = 2LL * 19 * nodes * (storage == LBMD_STORE_F32 ? 4 : 2);
   return bytes < 240000000LL;
+}
+// Whether the stream-collide of a single box waits for the step's gather: where
+// the MD branch sets the step, and always with in-place streaming, whose
+// stream-collide overwrites the populations that the gather reads.
+inline bool gather_goes_first(int storage, long long nodes, bool in_place) {
+  return in_place || spread_take_in_apply(storage, nodes);
 }
 // `take`: the owners' forces from their fixed-point sums (the sum ran with
 // records == false), else from the records.  `bump` (may be null):
