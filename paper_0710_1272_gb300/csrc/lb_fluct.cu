@@ -2,6 +2,7 @@
 // (fluctuating LB), in its own translation unit: the same node update as
 // k_stream_collide (pull) or k_aa_stream_collide (in place) plus fifteen
 // Philox normals per node.
+#include <algorithm>
 #include <cmath>
 
 #include "lb_aa.cuh"
@@ -54,9 +55,10 @@ __device__ __forceinline__ void bounce_six(const LbGeom &g, const float *__restr
 
 template <int FORCING, typename I, bool EARLY>
 __global__ void __launch_bounds__(32 * kFluctRows, EARLY ? 2 : 5)
-    k_stream_collide_fluct(LbGeom g, LbPhys ph, const float *__restrict__ src, float *__restrict__ dst) {
+    k_stream_collide_fluct(LbGeom g, LbPhys ph, int y0, const float *__restrict__ src,
+                           float *__restrict__ dst) {
   const int x = blockIdx.x * 32 + threadIdx.x;
-  const int y = blockIdx.y * kFluctRows + threadIdx.y;
+  const int y = y0 + blockIdx.y * kFluctRows + threadIdx.y;
   const int za = 2 * blockIdx.z, zb = min(za + 1, g.nz - 1);
   if (x >= g.nx || y >= g.ny) return;
   const I na = ((I)za * g.ny + y) * g.nx + x, nb = ((I)zb * g.ny + y) * g.nx + x;
@@ -96,16 +98,22 @@ template <typename I, bool EARLY>
 static cudaError_t fluct_launch_pair(const LbGeom &g, const LbPhys &ph, const void *src, void *dst,
                                      cudaStream_t s) {
   dim3 block(32, kFluctRows);
-  dim3 grid(g.ntx, (g.ny + kFluctRows - 1) / kFluctRows, (g.nz + 1) / 2);
   const float *a = (const float *)src;
   float *b = (float *)dst;
-  if (ph.g[0] == 0.f && ph.g[1] == 0.f && ph.g[2] == 0.f)
-    k_stream_collide_fluct<kForcingNone, I, EARLY><<<grid, block, 0, s>>>(g, ph, a, b);
-  else if (ph.forcing == LBMD_FORCING_GUO)
-    k_stream_collide_fluct<LBMD_FORCING_GUO, I, EARLY><<<grid, block, 0, s>>>(g, ph, a, b);
-  else
-    k_stream_collide_fluct<LBMD_FORCING_PAPER, I, EARLY><<<grid, block, 0, s>>>(g, ph, a, b);
-  return cudaGetLastError();
+  // the grid's 65535 rows of blocks are half as many nodes as the other
+  // kernels': boxes of ny > 262140 take two launches
+  for (int y0 = 0; y0 < g.ny; y0 += 65535 * kFluctRows) {
+    dim3 grid(g.ntx, std::min((g.ny - y0 + kFluctRows - 1) / kFluctRows, 65535), (g.nz + 1) / 2);
+    if (ph.g[0] == 0.f && ph.g[1] == 0.f && ph.g[2] == 0.f)
+      k_stream_collide_fluct<kForcingNone, I, EARLY><<<grid, block, 0, s>>>(g, ph, y0, a, b);
+    else if (ph.forcing == LBMD_FORCING_GUO)
+      k_stream_collide_fluct<LBMD_FORCING_GUO, I, EARLY><<<grid, block, 0, s>>>(g, ph, y0, a, b);
+    else
+      k_stream_collide_fluct<LBMD_FORCING_PAPER, I, EARLY><<<grid, block, 0, s>>>(g, ph, y0, a, b);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 template <int S, typename I>
