@@ -316,7 +316,7 @@ __device__ __forceinline__ void wca_add(F3 d, float sig2, float rc2, float eps24
 // b1 = r_b - r_a and b2 = r_c - r_b, their lengths and product: with
 // V = kappa phi^2 / 2 the forces F = -dV/dr on a, b and c are -A g1, A (g1 - g2)
 // and A g2; returns A.
-__device__ __noinline__ float bend_terms(F3 b1, F3 b2, float l1, float l2, float b12, float kappa, F3 &g1,
+__device__ __forceinline__ float bend_terms(F3 b1, F3 b2, float l1, float l2, float b12, float kappa, F3 &g1,
                                          F3 &g2) {
   const float cphi = fminf(1.f, fmaxf(-1.f, b12 / (l1 * l2)));
   const float phi = acosf(cphi);
