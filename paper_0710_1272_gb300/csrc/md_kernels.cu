@@ -53,17 +53,20 @@ __device__ __forceinline__ float dot_yx(F3 a, F3 b) {
 }
 
 // Threads of the MD block: one per bead in whole warps; for chains of up to 224
-// beads warps that only evaluate the force list (two for up to 32 beads, else
-// eight), beside the bead warps' own work; and for chains of more than one warp
-// one more for the boundary system of the tridiagonal solves, where the block's
-// register class (512, 768, 896 or 1024 threads: 128, 80, 72 or 64 registers) has
-// room for it, else warp 0 solves it.
+// beads warps that only evaluate the force list, beside the bead warps' own work
+// (two for up to 32 beads, four for up to 96, else eight: 40 beads 28.9 us a step
+// with four, 30.3 with eight; 100 beads 34.7 and 34.3; 128 beads 37.3 and 35.9);
+// and for chains of more than two warps one more for the boundary system of the
+// tridiagonal solves, where the block's register class (512, 768, 896 or 1024
+// threads: 128, 80, 72 or 64 registers) has room for it, else warp 0 solves it
+// (four chains of 40 beads 34.1 us a step, 34.8 with a warp of its own).
 __host__ __device__ inline int bead_threads(int N) { return (N + 31) / 32 * 32; }
 int md_threads(int N) {
   int t = bead_threads(N);
   if (t <= 32) return t + 64;
-  if (t <= 224) t += 256;
-  return t == 512 || t == 768 || t == 896 || t == LBMD_MAX_BEADS ? t : t + 32;
+  const bool two = t == 64;
+  if (t <= 224) t += t <= 96 ? 128 : 256;
+  return two || t == 512 || t == 768 || t == 896 || t == LBMD_MAX_BEADS ? t : t + 32;
 }
 // The block of an ensemble's chains: sizes in steps of 64 threads up to 512,
 // then the register classes, so that few launches take chains of every length
@@ -830,6 +833,9 @@ __device__ __forceinline__ float4 gauss3(uint64_t seed, uint32_t bead, int64_t s
 // bookkeeping; `a` may live in parameter or shared memory.  BLOCK is the
 // register class (512, 768, 896 or 1024 threads).
 //
+// `beside`: the block may have started beside the gather and waits for it before
+// it takes u_i; else u_i is there and read with the rest of the state.
+//
 // One chain is one block, so a substep is a chain of dependent phases and its
 // bound is their latency.  The positions of a substep are final after SHAKE, so
 // the next substep's forces, bond vectors and noise are found while RATTLE's
@@ -842,14 +848,15 @@ __device__ __forceinline__ float4 gauss3(uint64_t seed, uint32_t bead, int64_t s
 // the boundary system, meet in the constraint solves; a chain of one warp
 // solves without a barrier.  us a step without a solvent, with a list per bead,
 // the solve's boundary system and every barrier in line / so: 20 beads 29.6 /
-// 20.9, 100 beads 41.6 / 31.4, 400 beads 60.4 / 49.7, 700 beads 93 / 90, 1000
-// beads 122 / 123.
+// 19.4, 100 beads 41.6 / 29.9, 400 beads 60.4 / 49.5, 700 beads 93 / 90, 1000
+// beads 122 / 121; chains of 33 - 200 beads with no pair and no wall in reach,
+// whose lists cost nothing, are slower by it (40 beads 19.0 / 21.8).
 //
 // The results of a step are those of every release to the last bit
 // (released_values.py among the tests): sums and products are written with
 // their roundings where the compiler has a choice.
 template <int BLOCK>
-__device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
+__device__ __forceinline__ void md_cycle_body(const ChainArgs &a, bool beside) {
   extern __shared__ float4 smem4[];
   const int N = a.N;
   const int i = threadIdx.x;  // bead of this thread
@@ -860,7 +867,7 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
   // of them and the chain is short, else all but the spare one's
   const int holders = bead_threads(N), nch = holders >> 5, warp = i >> 5, lane = i & 31;
   const bool holds = i < holders;
-  const bool spare = nch > 1 && (int)blockDim.x > holders;
+  const bool spare = nch > 2 && (int)blockDim.x > holders;
   const int workers = spare ? (int)blockDim.x - 32 : (int)blockDim.x;
   const bool middle = nch > 1 && warp == (spare ? workers >> 5 : 0);
   const int eval0 = N <= 224 && workers - holders >= 64 ? holders : 0;
@@ -891,6 +898,7 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
     ref = a.nl_ref[i];
     v = f3(a.vel[i]);
     const float lam0 = a.lam[i];
+    if (!beside) ui = f3(a.ui[i]);
     const int own = a.it_first[i];
     if (i < N - 1 && a.has_bonds) b0 = a.b0[i];
     s_rh[i] = rh;
@@ -1054,7 +1062,7 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
     }
     __syncthreads();
     if (k == a.M) break;
-    if (k == 0) {
+    if (k == 0 && beside) {
       // (1) interpolated by k_gather, beside which this block may have
       // started; frozen for the M substeps
       asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1288,8 +1296,8 @@ __device__ __forceinline__ void md_cycle_body(const ChainArgs &a) {
 }
 
 template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK, 1) k_md_cycle(ChainArgs a) {
-  md_cycle_body<BLOCK>(a);
+__global__ void __launch_bounds__(BLOCK, 1) k_md_cycle(ChainArgs a, bool beside) {
+  md_cycle_body<BLOCK>(a, beside);
 }
 
 // Ensemble variant: block b runs chain chains[b] if its realisation is live.
@@ -1306,7 +1314,7 @@ __global__ void __launch_bounds__(BLOCK, 1)
   int *dst = reinterpret_cast<int *>(&s_a);
   for (int k = threadIdx.x; k < (int)(sizeof(ChainArgs) / sizeof(int)); k += blockDim.x) dst[k] = src[k];
   __syncthreads();
-  md_cycle_body<BLOCK>(s_a);
+  md_cycle_body<BLOCK>(s_a, false);
 }
 
 // Stage (1) for (bead, corner) pair e = 8 i + k handled by one thread; the
@@ -1452,10 +1460,10 @@ cudaError_t launch_md_cycle(const ChainArgs &a, int priority, bool beside, cudaS
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = beside ? 2 : 1;
-  if (threads <= 512) return cudaLaunchKernelEx(&cfg, k_md_cycle<512>, a);
-  if (threads <= 768) return cudaLaunchKernelEx(&cfg, k_md_cycle<768>, a);
-  if (threads <= 896) return cudaLaunchKernelEx(&cfg, k_md_cycle<896>, a);
-  return cudaLaunchKernelEx(&cfg, k_md_cycle<1024>, a);
+  if (threads <= 512) return cudaLaunchKernelEx(&cfg, k_md_cycle<512>, a, beside);
+  if (threads <= 768) return cudaLaunchKernelEx(&cfg, k_md_cycle<768>, a, beside);
+  if (threads <= 896) return cudaLaunchKernelEx(&cfg, k_md_cycle<896>, a, beside);
+  return cudaLaunchKernelEx(&cfg, k_md_cycle<1024>, a, beside);
 }
 
 // The sum of the spread as two kernels, one thread per (bead, corner) entry.
