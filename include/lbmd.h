@@ -439,7 +439,7 @@ int lbmd_ensemble_read_diagnostics(lbmd_ensemble *ens, int32_t member, lbmd_diag
 /*
  * Launch shape of the ensemble stream-collide: tile height rows (4, 8 or 16
  * rows of 32 consecutive nodes), register budget for warps resident warps per
- * SM (32: 64 registers, or 48: 40 registers), tiles per block `claim`
+ * SM (32: 64 registers, or 48: 40 registers, 48 in 16-bit storage), tiles per block `claim`
  * (1 .. 64; one block per claim tiles of the live realisations) and cells
  * per thread: 1; 2, the nodes at the same
  * (x, y) on two consecutive z-planes; or LBMD_ENS_XPAIR, two x-adjacent

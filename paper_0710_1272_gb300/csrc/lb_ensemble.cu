@@ -20,11 +20,17 @@ namespace lbmd {
 // not a multiple of 32).  With CPT = 3 (16-bit storage) a thread takes two
 // x-adjacent nodes instead, whose deviations share a 32-bit word (pair_node),
 // and a tile is 64 x ROWS consecutive nodes of one plane (every member's nx
-// is even, so a pair never straddles a row).  WARPS is the occupancy the register budget is sized for:
-// 48 warps per SM (40 registers, a little spilling) or 32 (64 registers,
-// none); population offsets are 32-bit.
+// is even, so a pair never straddles a row).  WARPS is the occupancy the register
+// budget is sized for: 48 warps per SM (40 registers, a little spilling) or 32
+// (64 registers, none); population offsets are 32-bit.  In 16-bit storage the
+// addresses in blocks of 64 nodes want more registers than 40, and 48 means 40
+// warps (48 registers): 300 boxes of 48x33x32, FP16, default shape 314 us a step
+// with 40 registers, 287 with 48 (302 with a stride of Vp and 40).
+constexpr int resident_warps(int storage, int warps) {
+  return storage != LBMD_STORE_F32 && warps == 48 ? 40 : warps;
+}
 template <int S, int FORCING, int ROWS, int WARPS, int CPT>
-__global__ void __launch_bounds__(32 * ROWS, WARPS / ROWS)
+__global__ void __launch_bounds__(32 * ROWS, resident_warps(S, WARPS) / ROWS)
     k_ens_stream_collide(const EnsLb *__restrict__ lbd, const EnsTile *__restrict__ tiles,
                          const int *__restrict__ n_tiles, const int *__restrict__ live, int cur,
                          int claim) {
