@@ -48,7 +48,8 @@ size_t stage_floats_for(const lbmd_params &p) {
 Layout make_layout(const lbmd_params &p, bool single_box) {
   Layout L{};
   const long long V = (long long)p.nx * p.ny * p.nz;
-  L.Vp = ((long long)pop_pitch(p) * p.ny * p.nz + 63) / 64 * 64;
+  L.pitch = pop_pitch(p, single_box);
+  L.Vp = ((long long)L.pitch * p.ny * p.nz + 63) / 64 * 64;
   L.ntx = (p.nx + 31) / 32;
   const size_t rows = (size_t)p.ny * p.nz;
   const size_t Np = (size_t)std::max(p.n_beads, 1);
@@ -377,7 +378,7 @@ cudaError_t init_instance(const lbmd_params &p, const Layout &L, char *ws, cudaS
   g.ntx = L.ntx;
   g.V = (long long)p.nx * p.ny * p.nz;
   g.Vp = L.Vp;
-  g.pitch = pop_pitch(p);
+  g.pitch = L.pitch;
   g.wall = WallGeom{p.wall_x, p.wall_thickness, p.wall_x >= 0 ? p.pore_d : 0, 0, 0, p.y_walls};
   if (p.wall_x >= 0) pore_origin(p, g.wall.pore_y0, g.wall.pore_z0);
   g.fill_solid = fill_solid(p, 2 * 19 * (size_t)L.Vp * store_bytes(p.storage));
