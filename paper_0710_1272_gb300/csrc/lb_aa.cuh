@@ -274,10 +274,11 @@ cudaError_t aa_launch_storage(int storage, const LbGeom &g, const LbPhys &ph, vo
                               DevStatus *bump, cudaStream_t s) {
   // 32-bit offsets when every population index fits
   const bool small = (long long)kQ * g.Vp < 0x7fffffffLL;
-  // 16-bit storage: two nodes per thread, in the odd step only in boxes of 2^17 nodes or
-  // more without a wall across x or of 192 nodes or more in x (figures at aa_pair)
+  // 16-bit storage: two nodes per thread except in narrow boxes (kNarrow), in the odd
+  // step only in boxes of 2^17 nodes or more without a wall across x or of 192 nodes
+  // or more in x (figures at aa_pair)
   if constexpr (NOISE == kNoNoise)
-    if (small && g.pitch % 2 == 0 &&
+    if (small && g.pitch % 2 == 0 && g.nx > kNarrow &&
         (!odd || ((long long)g.nx * g.ny * g.nz >= 1 << 17 && (g.wall.wall_x < 0 || g.nx >= 192)))) {
       if (storage == LBMD_STORE_F16) return aa_launch_pair<__half2, LBMD_STORE_F16>(g, ph, buf, odd, bump, s);
       if (storage == LBMD_STORE_BF16)

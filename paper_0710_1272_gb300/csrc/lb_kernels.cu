@@ -80,10 +80,11 @@ static cudaError_t lb_launch(const LbGeom &g, const LbPhys &ph, const void *src,
   // 32-bit offsets when every population index fits
   const bool small = (long long)kQ * g.Vp < 0x7fffffffLL;
   // 16-bit storage: two nodes per thread (rows of an even length, LbGeom::pitch),
-  // but not in boxes of up to 2^15 nodes, which are short of warps.  us a step,
+  // but not in narrow boxes (kNarrow) and in boxes of up to 2^15 nodes, which are
+  // short of warps.  us a step,
   // FP16, one node / two: 32^3 2.3 / 2.5, with a wall 2.7 / 3.0, 33x31x33 2.8 / 2.6
   // (forced 3.3 / 2.9, with a wall 3.0 / 3.1), 48^3 3.6 / 3.1, 64^3 5.2 / 4.5.
-  if (small && g.pitch % 2 == 0 && (long long)g.nx * g.ny * g.nz > 1 << 15) {
+  if (small && g.pitch % 2 == 0 && g.nx > kNarrow && (long long)g.nx * g.ny * g.nz > 1 << 15) {
     if (S == LBMD_STORE_F16) return lb_launch_pair<__half2>(g, ph, src, dst, bump, s);
     if (S == LBMD_STORE_BF16) return lb_launch_pair<__nv_bfloat162>(g, ph, src, dst, bump, s);
   }
@@ -406,7 +407,7 @@ cudaError_t launch_read_pulled(int storage, const LbGeom &g, float rho0, const v
   dim3 block(32, kRowsPerBlock);
   dim3 grid(g.ntx, (g.ny + kRowsPerBlock - 1) / kRowsPerBlock, (unsigned)nzc);
   const bool small = (long long)kQ * g.Vp < 0x7fffffffLL;  // 32-bit offsets
-  if (mode == kPopPull && small && g.pitch % 2 == 0) {
+  if (mode == kPopPull && small && g.pitch % 2 == 0 && g.nx > kNarrow) {
     if (storage == LBMD_STORE_F16)
       return read_pulled_pair<__half2>(g, rho0, src, src1, st, z0, nzc, f, fstride, s);
     if (storage == LBMD_STORE_BF16)

@@ -44,14 +44,14 @@ long long chunk_cells_for(const lbmd_params &p);
 // Row length of the populations: 16-bit ones of a single box start every row at a
 // word, so that two x-adjacent nodes share one whatever the box (not where the
 // padding would take the offsets beyond 32 bits).  Boxes that never take such
-// pairs (ensembles, which take them only where every
+// pairs (rows up to kNarrow nodes; ensembles, which take them only where every
 // width is even) have no padding: one node at a time it is never written, which
 // leaves a 32-byte sector of each row written in part, to be completed by a read
 // (300 boxes of 49x33x32, FP16: 403 us a step with it, 302 without).
 inline int pop_pitch(const lbmd_params &p, bool single_box) {
   const int even = p.nx + (p.nx & 1);
   const bool fits = 19LL * ((long long)even * p.ny * p.nz + 64) < 0x7fffffffLL;
-  return p.storage == LBMD_STORE_F32 || !single_box || !fits ? p.nx : even;
+  return p.storage == LBMD_STORE_F32 || !single_box || p.nx <= kNarrow || !fits ? p.nx : even;
 }
 // LbGeom::fill_solid of a box stepped with `traffic` bytes of populations per
 // step: beyond the 129 MB L2, and a wall of up to a sector's eight floats.

@@ -49,14 +49,21 @@ struct WallGeom {
   int wall_x, wall_t, pore_d, pore_y0, pore_z0, y_walls;
 };
 
+// Rows of up to this many nodes are taken one node per thread in 16-bit storage
+// too: by pairs half a warp and more would idle.  us a step, FP16, 2.8 M nodes,
+// one node / two: pull 24 wide 50.6 / 71.4, 32 wide 39.2 / 54.4, 33 wide 78.7 /
+// 54.3, 48 wide 50.5 / 38.8; with a wall 32 wide 49.0 / 70.4, 33 wide 84.0 / 69.8;
+// in place 32 wide 48.7 / 65.7, 33 wide 84.3 / 70.9.
+constexpr int kNarrow = 32;
+
 // Lattice geometry as the kernels see it.
 struct LbGeom {
   int nx, ny, nz;
   WallGeom wall;
   int fill_solid;               // stream-collides write zeros to solid nodes: a thin
                                 // wall in a box beyond the L2 cache
-  int pitch;                    // row length of the populations: nx, or nx + 1 if nx
-                                // is odd and they are held in 16 bits
+  int pitch;                    // row length of the populations: nx, or nx + 1 if nx is
+                                // odd and two nodes may share a word (pop_pitch)
   int ntx;                      // x-tiles of 32 nodes = words per bitfield row
   long long V;                  // nx * ny * nz
   long long Vp;                 // population stride (pitch * ny * nz rounded up to 64)
