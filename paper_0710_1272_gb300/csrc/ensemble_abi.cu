@@ -115,7 +115,23 @@ EnsLayout make_ens_layout(const lbmd_params *m, int32_t count) {
 
 struct Group {  // chains sharing one MD block size
   int threads, max_n, first, count;
+  bool alone;  // no other block on the SM of one of these
 };
+
+// The blocks of up to 128 threads leave an SM room for stream-collide blocks, which
+// take issue slots and the instruction cache from them: beside a stream-collide of
+// 128x33x32 boxes a cycle of 42 k cycles took 76 k.  Where the MD cycle and the
+// stream-collide take about as long, so that this sets the step, these blocks get
+// an SM to themselves; not where the stream-collide does little or takes much
+// longer, which then misses their SMs, nor with many chains.  us a step, shared /
+// alone, chains of 30 - 90 beads (MB: populations of a step): FP16, 16 chains 39 MB
+// 43.8 / 42.5, 119 MB 60.1 / 53.5, 358 MB 84.9 / 81.8, 1434 MB 243 / 250; 64 chains
+// 39 MB 55.9 / 54.9, 239 MB 84.5 / 74.3, 478 MB 111.6 / 114.6; 96 chains 358 MB 102.6 /
+// 105.0; FP32, 4 chains 19 MB 35.8 / 37.0, 32 chains 239 MB 81.7 / 72.0.  Chains of
+// 130 - 190 beads (256 threads) lose by it: 76.0 / 78.7.
+bool md_alone(int threads, int chains, size_t traffic) {
+  return threads <= 128 && chains <= 64 && traffic >= 60000000 && traffic <= 400000000;
+}
 
 }  // namespace
 
@@ -309,7 +325,7 @@ cudaError_t enqueue_ens_step(lbmd_ensemble *e, int cur) {
   for (size_t k = 0; k < e->groups.size(); ++k) {
     const Group &g = e->groups[k];
     if ((err = launch_ens_md_cycle(e->d_mem, e->d_chains + g.first, g.count, g.threads, g.max_n, live,
-                                   e->prio_high, e->side[k % e->nside])) != cudaSuccess)
+                                   g.alone, e->prio_high, e->side[k % e->nside])) != cudaSuccess)
       return err;
   }
   if (t[1] && (err = cudaEventRecord(t[1], e->own)) != cudaSuccess) return err;
@@ -558,7 +574,8 @@ int lbmd_ensemble_create(const lbmd_params *members, int32_t count, void *dev_wo
   for (int m = 0; m < count; ++m) by_threads[md_group_threads(members[m].n_beads)].push_back(m);
   std::vector<int> chains;
   for (auto &kv : by_threads) {
-    Group g{kv.first, 0, (int)chains.size(), (int)kv.second.size()};
+    Group g{kv.first, 0, (int)chains.size(), (int)kv.second.size(),
+            md_alone(kv.first, count, traffic)};
     for (int m : kv.second) {
       chains.push_back(m);
       g.max_n = std::max(g.max_n, members[m].n_beads);

@@ -302,9 +302,10 @@ int ens_lb_blocks_per_sm(int storage, int forcing, int rows, int warps, int cpt)
 cudaError_t launch_ens_gather(int storage, const EnsMember *mem, const int2 *beads, int nb,
                               const int *live, int cur, cudaStream_t s);
 // MD cycle of the `count` chains listed in `chains`, one block of `threads`
-// threads each, with dynamic shared memory for `max_n` beads.
+// threads each, with dynamic shared memory for `max_n` beads.  `alone` (up to 512
+// threads): with all there is, so that no other block shares an SM with one.
 cudaError_t launch_ens_md_cycle(const EnsMember *mem, const int *chains, int count, int threads,
-                                int max_n, const int *live, int priority, cudaStream_t s);
+                                int max_n, const int *live, bool alone, int priority, cudaStream_t s);
 // Sum part of the spread of every live realisation (after every MD group); with
 // `rec` ([8 nb], or null) the owners' forces are converted to records there.
 cudaError_t launch_ens_spread_sum(const EnsMember *mem, const int2 *beads, int nb, const int *live,

@@ -85,6 +85,7 @@ int md_group_threads(int N) {
 // measured average three) and 128 for the beads in the pore, as far as 220 KB
 // reach.
 constexpr int kMdSmemMost = 220000;
+constexpr size_t kSmemOfBlock = 227 * 1024;  // the most that one block may have
 __host__ __device__ inline size_t md_smem_head(int N) {
   return ((size_t)N * (5 * sizeof(float4) + 2 * sizeof(float)) + 15) / 16 * 16;
 }
@@ -1415,15 +1416,26 @@ __global__ void __launch_bounds__(256)
   if (valid && (e & 7) == 0) M.a.ui[mi.y] = f4(u);
 }
 
+// Dynamic shared memory with which a block of k_ens_md_cycle<512> leaves none on
+// its SM for another block.
+static cudaError_t md_alone_bytes(size_t *bytes) {
+  cudaFuncAttributes at;
+  const cudaError_t e = cudaFuncGetAttributes(&at, k_ens_md_cycle<512>);
+  if (e == cudaSuccess) *bytes = kSmemOfBlock - at.sharedSizeBytes;
+  return e;
+}
+
 cudaError_t md_prepare() {
-  const int s512 = (int)md_smem_bytes(512), s768 = (int)md_smem_bytes(768), s1024 = (int)md_smem_bytes(LBMD_MAX_BEADS);
+  size_t alone = 0;
   cudaError_t e;
+  if ((e = md_alone_bytes(&alone)) != cudaSuccess) return e;
+  const int s512 = (int)md_smem_bytes(512), s768 = (int)md_smem_bytes(768), s1024 = (int)md_smem_bytes(LBMD_MAX_BEADS);
   if ((e = cudaFuncSetAttribute(k_md_cycle<768>, cudaFuncAttributeMaxDynamicSharedMemorySize, s768)) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(k_md_cycle<896>, cudaFuncAttributeMaxDynamicSharedMemorySize, s1024)) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(k_ens_md_cycle<768>, cudaFuncAttributeMaxDynamicSharedMemorySize, s768)) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(k_md_cycle<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, s512)) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(k_md_cycle<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, s1024)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(k_ens_md_cycle<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, s512)) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(k_ens_md_cycle<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)alone)) != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_ens_md_cycle<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, s1024);
 }
 
@@ -1666,12 +1678,16 @@ cudaError_t launch_ens_gather(int storage, const EnsMember *mem, const int2 *bea
 }
 
 cudaError_t launch_ens_md_cycle(const EnsMember *mem, const int *chains, int count, int threads,
-                                int max_n, const int *live, int priority, cudaStream_t s) {
+                                int max_n, const int *live, bool alone, int priority, cudaStream_t s) {
   if (count <= 0) return cudaSuccess;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)count);
   cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = md_smem_bytes(max_n);
+  if (alone) {
+    const cudaError_t e = md_alone_bytes(&cfg.dynamicSmemBytes);
+    if (e != cudaSuccess) return e;
+  }
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributePriority;
