@@ -65,8 +65,8 @@ struct Ops2 {
   static __device__ __forceinline__ bool finite(V a) { return isfinite(a.x) && isfinite(a.y); }
 };
 
-// Uniforms in (0, 1) as uniform23 gives them: 1 + k 2^-23 by its bits, less
-// 1 - 2^-24, both exact.
+// Uniforms (k + 1/2) 2^-23 in (0, 1), as uniform23 gives them: 1 + k 2^-23 by its
+// bits, less 1 - 2^-24, both exact.
 template <class O>
 __device__ __forceinline__ typename O::V uniform23_t(const uint32_t *x) {
   float f[O::N];
@@ -79,12 +79,15 @@ __device__ __forceinline__ typename O::V uniform23_t(const uint32_t *x) {
 // cosine and sine of 2 pi u2, on operations that take one or two nodes at once
 // (the library functions take one, and were two fifths of the kernel).
 //   ln u = e ln 2 + ln(1 + f), 2^e (1 + f) = u, sqrt(1/2) <= 1 + f < sqrt(2):
-//     f - f^2/2 + f^3 Q(f), Q the minimax polynomial of degree 7 (6e-9);
+//     f - f^2/2 + f^3 Q(f), Q of degree 7 (6e-9);
 //   the angle is reduced to +-pi/4 exactly (2 u2 less a multiple of 1/2), sine
-//     and cosine there by minimax polynomials in r^2 (3e-9, 6e-11);
+//     and cosine there by polynomials in r^2 (3.1e-9, 6e-11);
 //   the root from the hardware's reciprocal root and one Newton step.
-// Against 64 bits over all 2^23 values of u1: rms 4.39e-8 relative for the normals,
-// largest error 1.7e-7 of the radius (library functions 4.38e-8, 1.7e-7).
+// The polynomials are weighted minimax ones by Lawson's iteration, fitted again
+// with their weights and errors by a test (test_noise_polynomials.py).  Against
+// 64 bits over all 2^23 values of u1 and of u2: rms 4.49e-8 relative for the
+// normals, largest error 1.78e-7 of the radius (library functions 4.60e-8,
+// 1.77e-7).
 template <class O>
 __device__ __forceinline__ void box_muller_t(typename O::V u1, typename O::V u2, typename O::V &n1,
                                              typename O::V &n2) {

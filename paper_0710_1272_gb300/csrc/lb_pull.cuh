@@ -6,16 +6,6 @@
 
 namespace lbmd {
 
-// Pre-collision deviations h_p(x, t+1) of node (x, y, z) from the
-// post-collision buffer `src` (Eq. 5 free streaming, pull form):
-//   h_p(x) = h*_p(x - c_p)      if x - c_p is fluid,
-//   h_p(x) = h*_opp(p)(x)       otherwise (the population that left x towards
-//                               the solid node comes back reversed),
-// where bit p of `bb` says whether x - c_p is solid (the node's link mask; 0
-// for a node known to be far from any solid node).  h*_q(y) sits at [q][y]
-// (SWAP = false, kPopPull) or at [opp(q)][y] (SWAP = true, kPopAASwap).  I is
-// the index type of the population offsets: int when 19 Vp < 2^31 (cheaper
-// address arithmetic), size_t otherwise.
 // Row length of the populations of storage S (pad: see LbGeom::pitch).
 template <int S>
 __device__ __forceinline__ int row_pitch(const LbGeom &g) {
@@ -28,6 +18,16 @@ __device__ __forceinline__ I pop_node(const LbGeom &g, I node) {
   return node + (I)((unsigned)node / (unsigned)g.nx);  // one padding element per row
 }
 
+// Pre-collision deviations h_p(x, t+1) of node (x, y, z) from the
+// post-collision buffer `src` (Eq. 5 free streaming, pull form):
+//   h_p(x) = h*_p(x - c_p)      if x - c_p is fluid,
+//   h_p(x) = h*_opp(p)(x)       otherwise (the population that left x towards
+//                               the solid node comes back reversed),
+// where bit p of `bb` says whether x - c_p is solid (the node's link mask; 0
+// for a node known to be far from any solid node).  h*_q(y) sits at [q][y]
+// (SWAP = false, kPopPull) or at [opp(q)][y] (SWAP = true, kPopAASwap).  I is
+// the index type of the population offsets: int when 19 Vp < 2^31 (cheaper
+// address arithmetic), size_t otherwise.
 template <int S, typename I = size_t, bool SWAP = false>
 __device__ __forceinline__ void pull19_mask(const LbGeom &g,
                                             const typename Store<S>::T *__restrict__ src, int x,
