@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock, 6)
 }
 
 // 16-bit storage: one thread per pair of x-adjacent nodes (pair_node).  A
-// warp covers 64 nodes of one row, i.e. two 32-node tiles.  Register budget:
+// warp covers 64 nodes of one row.  Register budget:
 // 64 (four blocks per SM) for the benchmark's zero-force collision, 80 (three)
 // for the forced variants, which would spill at 64.
 template <typename T2, int FORCING>
@@ -179,7 +179,6 @@ __global__ void k_init(LbGeom g, float rho0, const float *rho, const float *u, f
   const int y = blockIdx.y * kRowsPerBlock + threadIdx.y;
   const int z = blockIdx.z;
   if (x >= g.nx || y >= g.ny) return;
-  const size_t self = ((size_t)z * g.ny + y) * g.nx + x;
   const size_t st = pop_stride<S, size_t>((size_t)g.Vp);
   const size_t at = pop_base<S, size_t>(((size_t)z * g.ny + y) * row_pitch<S>(g) + x);
   if (solid_at(g.solid, g.ntx, g.ny, x, y, z)) {
@@ -238,7 +237,6 @@ __global__ void k_init_local(LbGeom g, float rho0, const float *rho, const float
   const int y = blockIdx.y * kRowsPerBlock + threadIdx.y;
   const int z = z0 + blockIdx.z;
   if (x >= g.nx || y >= g.ny) return;
-  const size_t self = ((size_t)z * g.ny + y) * g.nx + x;
   const size_t st = pop_stride<S, size_t>((size_t)g.Vp);
   const size_t at = pop_base<S, size_t>(((size_t)z * g.ny + y) * row_pitch<S>(g) + x);
   float r = rho0, ux = 0.f, uy = 0.f, uz = 0.f;
@@ -406,7 +404,11 @@ cudaError_t launch_read_pulled(int storage, const LbGeom &g, float rho0, const v
                                long long nzc, float *f, long long fstride, cudaStream_t s) {
   dim3 block(32, kRowsPerBlock);
   dim3 grid(g.ntx, (g.ny + kRowsPerBlock - 1) / kRowsPerBlock, (unsigned)nzc);
-  const bool small = (long long)kQ * g.Vp < 0x7fffffffLL;  // 32-bit offsets
+  // 32-bit offsets; not for a plain copy to rows of odd width, whose 19 stores then
+  // run further apart than memory likes (255x131x127 in place, even step: FP32
+  // 118.2 us by 64-bit offsets, 123.0 by 32-bit ones, FP16 106.3 and 113.6; 256 wide
+  // 101.5 and 97.5, 86.3 and 82.6)
+  const bool small = (long long)kQ * g.Vp < 0x7fffffffLL && !(mode == kPopAALocal && g.nx % 2);
   if (mode == kPopPull && small && g.pitch % 2 == 0 && g.nx > kNarrow) {
     if (storage == LBMD_STORE_F16)
       return read_pulled_pair<__half2>(g, rho0, src, src1, st, z0, nzc, f, fstride, s);

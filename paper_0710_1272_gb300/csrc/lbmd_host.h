@@ -54,7 +54,10 @@ inline int pop_pitch(const lbmd_params &p, bool single_box) {
   return p.storage == LBMD_STORE_F32 || !single_box || p.nx <= kNarrow || !fits ? p.nx : even;
 }
 // LbGeom::fill_solid of a box stepped with `traffic` bytes of populations per
-// step: beyond the 129 MB L2, and a wall of up to a sector's eight floats.
+// step: beyond the 129 MB L2, and a wall of up to a sector's eight floats.  FP32,
+// 256x128x128, us a step, left out / filled: one layer 100.3 / 95.1, two to six
+// 100.3 - 107.2 / 95.2, eight 107.2 / 95.1, eight that begin with a sector 93.9 /
+// 95.2; 141x160x160, one to eight layers 121 - 124 / 107.
 inline int fill_solid(const lbmd_params &p, size_t traffic) {
   return p.wall_x >= 0 && p.wall_thickness <= 8 && traffic > (size_t)129 << 20;
 }
