@@ -91,7 +91,7 @@ EnsLayout make_ens_layout(const lbmd_params *m, int32_t count) {
     E.stage_floats = std::max(E.stage_floats, stage_floats_for(m[k]));
     nodes += (long long)m[k].nx * m[k].ny * m[k].nz;
   }
-  E.lb_sets = !m[0].solvent_free && !spread_take_in_apply(m[0].storage, nodes);
+  E.lb_sets = !m[0].solvent_free && !spread_take_in_apply(m[0].storage, nodes, true);
   E.mem = take((size_t)count * sizeof(EnsMember));
   E.lbd = take((size_t)count * sizeof(EnsLb));
   E.tiles = take(std::max<size_t>(E.max_tiles, 1) * sizeof(EnsTile));

@@ -118,7 +118,7 @@ cudaError_t enqueue_step(lbmd_ctx *c, int src) {
   // Where the owners' sums are converted: when the MD branch sets the step,
   // in the apply (one launch fewer on that branch); when the stream-collide
   // sets it, beside it in k_spread_finalize, keeping the apply after it short.
-  const bool take = spread_take_in_apply(c->p.storage, c->geo.V);
+  const bool take = spread_take_in_apply(c->p.storage, c->geo.V, false);
   if (c->N > 0) {
     // (1) gather from the pre-step populations, and the MD cycle on the
     // high-priority side stream while the stream-collide runs on the main
@@ -250,7 +250,7 @@ cudaError_t capture_read(lbmd_ctx *c, int start) {
 // The chain's buffers (positions through the status word: ~1 MB for 400
 // beads) as an L2-persisting window of the side stream, whose kernels (the MD
 // cycle, the spread sums) run beside the stream-collide: its 637 MB per step
-// would otherwise evict them from the 126 MB L2 between steps.  Raises the
+// would otherwise evict them from the 129 MB L2 between steps.  Raises the
 // context's persisting-L2 limit to the window if it is lower.  Best effort:
 // a device without persisting L2 keeps the default policy.  FP16 coupled step
 // 85.4 -> 83.8 us on the 256x128x128, N = 400 box.

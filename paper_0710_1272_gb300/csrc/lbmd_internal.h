@@ -257,22 +257,24 @@ constexpr int kOwnerFree = 0x7f7f7f7f;
 cudaError_t launch_spread_sum(const ChainArgs &a, bool records, cudaStream_t s);
 // True when the apply should convert the sums itself (the MD branch sets the
 // step), false when the stream-collide sets it -- taken as a stream-collide
-// moving 240 MB or more per step (~40 us at the HBM rate, about the MD branch of
-// a 400-bead chain beside it).  The gather follows the same rule with two
-// population buffers (gather_goes_first); so does an ensemble, by the nodes of
-// all its boxes.  Step of a 400-bead chain,
-// us, true against false: 144x80x80 FP32 (140 MB) 47.7 / 54.5, FP16 44.2 / 47.1;
-// 256x128x128 FP16 (318 MB) 73.3 / 69.1, FP32 (637 MB) 105.3 / 101.6; of an
-// ensemble of 32 chains of 120 - 400 beads, FP16 (764 MB): 194.6 / 191.0.
-inline bool spread_take_in_apply(int storage, long long nodes) {
+// moving 280 MB or more per step (~45 us at the HBM rate, about the MD branch of
+// a 400-bead chain beside it), in an ensemble 600 MB by the nodes of all its boxes
+// (its MD blocks share the SMs with it).  The gather follows the same rule with two
+// population buffers (gather_goes_first).  Step of a 400-bead chain, us, true
+// against false: 144x80x80 FP32 (140 MB) 57.9 / 63.0, FP16 55.8 / 59.8; 192x112x112
+// FP16 (183 MB) 59.5 / 64.8; 176x96x96 FP32 (247 MB) 60.0 / 65.2; 256x128x128 FP16
+// (319 MB) 70.6 / 66.9, FP32 (638 MB) 105.9 / 102.0.  Ensembles of 24 chains of
+// 130 - 190 beads, FP16 (291 MB) 107.1 / 112.2, FP32 (582 MB) 139 / 144.6; of 32
+// chains of 120 - 400 beads, FP16 (772 MB) 183.5 / 179.1, FP32 269 / 260.
+inline bool spread_take_in_apply(int storage, long long nodes, bool ensemble) {
   const long long bytes = 2LL * 19 * nodes * (storage == LBMD_STORE_F32 ? 4 : 2);
-  return bytes < 240000000LL;
+  return bytes < (ensemble ? 600000000LL : 280000000LL);
 }
 // Whether the stream-collide of a single box waits for the step's gather: where
 // the MD branch sets the step, and always with in-place streaming, whose
 // stream-collide overwrites the populations that the gather reads.
 inline bool gather_goes_first(int storage, long long nodes, bool in_place) {
-  return in_place || spread_take_in_apply(storage, nodes);
+  return in_place || spread_take_in_apply(storage, nodes, false);
 }
 // `take`: the owners' forces from their fixed-point sums (the sum ran with
 // records == false), else from the records.  `bump` (may be null):

@@ -33,3 +33,20 @@ def test_short_chains_alone_equal_single_boxes(storage, shape):
         for x, y in zip(ens.beads(k), one.beads()):
             np.testing.assert_array_equal(x, y)
         np.testing.assert_array_equal(ens.populations(k), one.populations())
+
+
+# 594 and 627 MB: the gather beside the stream-collide and the forces through records from 600 MB on
+@pytest.mark.parametrize("storage,shape", [("f32", (96, 102, 133)), ("f32", (96, 102, 141)), ("f16", (161, 128, 134))])
+def test_large_ensembles_equal_single_boxes(storage, shape):
+    nx, ny, nz = shape
+    members = [dict(nx=nx, ny=ny, nz=nz, n_beads=n, lj_sigma=1.0, lj_eps=2e-3, seed=n, storage=storage) for n in (5, 40, 75)]
+    starts = [_line(m["n_beads"], ny, nz) for m in members]
+    ens = lb.Ensemble(members, starts)
+    ens.step(18)
+    steps = ens.results()["steps"]
+    for k, (m, start) in enumerate(zip(members, starts)):
+        one = lb.Simulation(m, init_pos=start)
+        one.step(int(steps[k]))
+        for x, y in zip(ens.beads(k), one.beads()):
+            np.testing.assert_array_equal(x, y)
+        np.testing.assert_array_equal(ens.populations(k), one.populations())

@@ -19,8 +19,8 @@ def _chain(n, nx, ny, nz):
 
 
 @pytest.mark.parametrize("storage,shape", [
-    ("f32", (128, 112, 109)), ("f32", (128, 112, 112)), ("f16", (160, 144, 135)), ("f16", (160, 144, 138)),
-    ("f16", (161, 144, 137)), ("bf16", (160, 144, 138))])
+    ("f32", (128, 112, 109)), ("f32", (128, 112, 112)), ("f32", (128, 112, 128)), ("f32", (128, 112, 129)),
+    ("f16", (160, 144, 135)), ("f16", (160, 144, 160)), ("f16", (161, 144, 159)), ("bf16", (160, 144, 160))])
 def test_in_place_equals_pull_with_a_chain(storage, shape):
     nx, ny, nz = shape
     n = 100

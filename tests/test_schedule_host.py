@@ -33,7 +33,7 @@ def test_gather_precedes_an_in_place_stream_collide(tmp_path):
                                                               text=True).stdout.splitlines()]
     assert rows and all(in_place == 1 for _, _, in_place, _ in rows)
     for storage, nodes, _, two in rows:
-        assert two == (2 * 19 * nodes * (4 if storage == 0 else 2) < 240_000_000)
+        assert two == (2 * 19 * nodes * (4 if storage == 0 else 2) < 280_000_000)
 
 
 def test_the_step_asks_for_that_order():
