@@ -853,7 +853,7 @@ __device__ __forceinline__ float4 gauss3(uint64_t seed, uint32_t bead, int64_t s
 // beads 122 / 121; chains of 33 - 200 beads with no pair and no wall in reach,
 // whose lists cost nothing, are slower by it (40 beads 19.0 / 21.8).
 //
-// The results of a step are those of every release to the last bit
+// The results of a step are those of earlier releases to the last bit
 // (released_values.py among the tests): sums and products are written with
 // their roundings where the compiler has a choice.
 template <int BLOCK>
